@@ -101,8 +101,10 @@ typedef struct {
     int64_t sum_face_rank;          /* ACA ranks of the far faces, summed */
     int64_t stored_complex;         /* complex numbers stored (faces + fibres) */
     int64_t dense_complex;          /* rows * cols * unique frequencies */
-    int64_t entries_regular;        /* regular entries evaluated */
-    int64_t entries_tube;           /* fibre (all-frequency) entries evaluated */
+    int64_t entries_regular;        /* regular entries evaluated (near and far; a near block of the
+                                       mixed form evaluates the frequencies it selects) */
+    int64_t entries_tube;           /* fibre (all-frequency) entries evaluated (far blocks, and near
+                                       blocks of the mixed form) */
     int64_t pairs_singular;         /* touching pairs integrated (per frequency) */
     double ms_plan, ms_singular, ms_near, ms_far, ms_total;
     int64_t pool_growths;           /* face pool grown during compression: far blocks redone
@@ -138,9 +140,10 @@ int tdbem_ctx_sync(tdbem_ctx_t ctx);
  * or polls >= 2^31. */
 int tdbem_ctx_set_wait_limit(tdbem_ctx_t ctx, int64_t polls);
 /* Size in bytes of the buffer in which tdbem_compress forms and compresses
- * the near-field tensor, batch by batch of near blocks (default 16 GiB; a
- * block larger than the buffer forms a batch of its own).  TDBEM_ERR_ARG if
- * bytes <= 0. */
+ * the near-field tensor of the FP64 form, batch by batch of near blocks
+ * (default 16 GiB; a block larger than the buffer forms a batch of its own;
+ * the mixed form evaluates its near entries on demand and has no buffer).
+ * TDBEM_ERR_ARG if bytes <= 0. */
 int tdbem_ctx_set_near_batch(tdbem_ctx_t ctx, int64_t bytes);
 /* Scale (> 0, default 1) of the far-field part of the first face-pool size
  * of tdbem_compress (estimated from the far blocks' sizes or the predicted
@@ -228,12 +231,13 @@ int tdbem_entries(tdbem_mesh_t mesh, const tdbem_op *op, tdbem_freqs_t f, const 
 /* The same entries through one of the kernels that tdbem_compress runs, so
  * that each can be checked on its own against an independent evaluation:
  *   path = TDBEM_PATH_GENERIC: tdbem_entries itself;
- *   path = TDBEM_PATH_NEAR: the near-field phases of the compression on the
+ *   path = TDBEM_PATH_NEAR: the near-field entries of the compression on the
  *     single block rows x cols: the touching-pair table of the mesh
- *     (Sauter-Schwab, Sec. 3), then the dense near-field tensor kernel
- *     (regular pairs by the 7-point rule with the point geometry shared
- *     across frequencies, touching pairs read from the table); at most 256
- *     frequencies and 2^31 - 1 entries per frequency;
+ *     (Sauter-Schwab, Sec. 3), then the dense near-field tensor (regular
+ *     pairs by the 7-point rule with the point geometry shared across
+ *     frequencies, touching pairs read from the table; the mixed form's
+ *     compression runs the same sums one entry and frequency at a time); at
+ *     most 256 frequencies and 2^31 - 1 entries per frequency;
  *   path = TDBEM_PATH_FIBRE: the far-field engine's entry evaluation (the
  *     8-lane point-pair groups with which Algorithm 1's fibres and frequency
  *     tubes are formed in tdbem_compress), which applies the regular 7 x 7
@@ -302,11 +306,10 @@ int tdbem_tensor_destroy(tdbem_tensor_t t);
  *     (64/128/256 threads, 2..16 CTAs per SM);
  *   - mixed form only: frequencies per pass of the touching-pair table
  *     (register tiles of 4/8/16 frequencies for the single layer and its adjoint, 2/4/8
- *     for the double layer) and of the near-field tensor kernel (8/4/16),
- *     each timed on its own phase.
+ *     for the double layer), timed on its own phase.
  * chosen (nullable, host int32 [4]) receives {far threads per CTA, far CTAs
  * per SM, touching-pair frequencies per pass, near-field frequencies per
- * pass} (0 for the two mixed-form choices of an FP64 form).  Defaults without
+ * pass of TDBEM_PATH_NEAR (not tuned)} (0 for the two of an FP64 form).  Defaults without
  * tuning: {128, 4 (FP64) / 5 (mixed), 36 or 12, 8}. */
 int tdbem_autotune(tdbem_ctx_t ctx, tdbem_mesh_t mesh, const tdbem_op *op, tdbem_freqs_t f, tdbem_tree_t tree,
                    const tdbem_aca_cfg *cfg, int32_t *chosen);

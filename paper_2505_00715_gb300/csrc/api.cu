@@ -159,6 +159,38 @@ int prepare_sing(tdbem_ctx *ctx, const tdbem_mesh *m, int op, int ng, std::vecto
     return TDBEM_OK;
 }
 
+// Separated frequency sums of one operator and frequency list: the split into
+// separated and direct frequencies, the coefficient tables (near field,
+// touching pairs) and the reference quadrature points of the touching-pair
+// classes, formed on the context's stream in one device buffer (owned).
+// sigma: host s / c of the nf frequencies, sig: the same on the device.
+int prepare_sep(tdbem_ctx *ctx, const tdbem_mesh *m, int op, int prec, int ng, const double *gx, const double *gw,
+                const double *sigma, const double *sig, int nf, std::vector<void *> &owned, SepSet &near,
+                SepSet &sing, double **rule) {
+    std::vector<int> ka, kb;
+    // 1e-6 relative slack: the distances are formed in the working precision
+    const double slack = 1.0 + 1e-6;
+    td_sep_split(op, prec, sigma, nf, slack * (m->rad_tri + (op == TDBEM_DLP ? m->rad_vert : m->rad_tri)), false, ka, near);
+    td_sep_split(op, prec, sigma, nf, slack * m->edge_max, true, kb, sing);
+    ka.insert(ka.end(), kb.begin(), kb.end());
+    auto al = [](size_t x) { return (x + 255) & ~(size_t)255; };
+    const size_t o1 = al(sizeof(int) * 4 * nf), o2 = o1 + al(td_sep_coef_bytes(op, near, false));
+    const size_t o3 = o2 + al(td_sep_coef_bytes(op, sing, true)), o4 = o3 + sizeof(double) * td_ss_rule_size(ng);
+    char *buf = nullptr;
+    int rc;
+    if ((rc = dalloc(ctx, &buf, o4, &owned)) || (rc = upload(ctx, (int *)buf, ka.data(), ka.size()))) return rc;
+    near.klist = (const int *)buf;
+    sing.klist = near.klist + nf;
+    near.pk = (int *)buf + 2 * nf;
+    near.coef = (c64 *)(buf + o1);
+    sing.coef = (c64 *)(buf + o2);
+    *rule = (double *)(buf + o3);
+    if (td_launch_sep_coef(ctx->stream, op, sig, near, false) || td_launch_sep_coef(ctx->stream, op, sig, sing, true) ||
+        td_launch_ss_rule(ctx->stream, ng, gx, gw, *rule))
+        return td_fail(ctx, TDBEM_ERR_CUDA, "separated-sum tables failed: %s", cudaGetErrorString(cudaGetLastError()));
+    return TDBEM_OK;
+}
+
 }  // namespace
 
 // ============================================================================
@@ -291,6 +323,9 @@ extern "C" int tdbem_mesh_create(tdbem_ctx_t ctx, const double *verts, int64_t n
         const double v[3] = {c[0] - a[0], c[1] - a[1], c[2] - a[2]};
         const double n[3] = {u[1] * v[2] - u[2] * v[1], u[2] * v[0] - u[0] * v[2], u[0] * v[1] - u[1] * v[0]};
         const double len = std::sqrt(n[0] * n[0] + n[1] * n[1] + n[2] * n[2]);
+        const double w[3] = {v[0] - u[0], v[1] - u[1], v[2] - u[2]};
+        for (const double *d : {u, v, w})
+            m->edge_max = std::max(m->edge_max, std::sqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]));
         if (!(len > 0.0)) {
             delete m;
             return td_fail(ctx, TDBEM_ERR_ARG, "degenerate triangle %lld", (long long)e);
@@ -304,20 +339,32 @@ extern "C" int tdbem_mesh_create(tdbem_ctx_t ctx, const double *verts, int64_t n
     td_rule7(bary, w7);
     std::vector<double> q(3 * 7 * nt), qw(7 * nt);
     std::vector<float> qh(3 * 7 * nt), ql(3 * 7 * nt), qw32(7 * nt), n32(3 * nt);
+    double rad2_tri = 0.0, rad2_vert = 0.0;
     for (int64_t e = 0; e < nt; ++e)
         for (int p = 0; p < 7; ++p) {
+            double r2[4] = {0.0, 0.0, 0.0, 0.0};  // squared distances from the centroid and the vertices
             for (int c = 0; c < 3; ++c) {
-                double x = 0.0;
+                double x = 0.0, g = 0.0;
                 for (int k = 0; k < 3; ++k) x += bary[p][k] * verts[3 * tris[3 * e + k] + c];
+                for (int k = 0; k < 3; ++k) {
+                    const double v = verts[3 * tris[3 * e + k] + c];
+                    r2[1 + k] += (x - v) * (x - v);
+                    g += v / 3.0;
+                }
+                r2[0] += (x - g) * (x - g);
                 const int64_t o = ((int64_t)c * 7 + p) * nt + e;
                 q[o] = x;
                 qh[o] = (float)x;
                 ql[o] = (float)(x - (double)qh[o]);
             }
+            rad2_tri = std::max(rad2_tri, r2[0]);
+            rad2_vert = std::max(rad2_vert, std::max(r2[1], std::max(r2[2], r2[3])));
             qw[p * nt + e] = w7[p] * m->area[e];
             qw32[p * nt + e] = (float)qw[p * nt + e];
         }
     for (int64_t k = 0; k < 3 * nt; ++k) n32[k] = (float)nrm[k];
+    m->rad_tri = std::sqrt(rad2_tri);
+    m->rad_vert = std::sqrt(rad2_vert);
     // 16-byte packs: (hi xyz, weight) and (lo xyz, 0) per point, (normal, 0) per triangle
     std::vector<float> qp(8 * 7 * (size_t)nt), nrm4(4 * (size_t)nt, 0.f);
     for (int64_t e = 0; e < nt; ++e) {
@@ -734,14 +781,24 @@ extern "C" int tdbem_entries_path(tdbem_mesh_t mesh, const tdbem_op *op, tdbem_f
         c64 *table;
         int32_t *blk;
         int64_t *pre;
-        if ((rc = dalloc(ctx, &table, (size_t)std::max(np, 1) * nf * 3, &g.p)) || (rc = dalloc(ctx, &blk, 8, &g.p)) ||
+        const int nv = op->op == TDBEM_DLP ? 3 : 1;
+        SepSet snear, ssing;
+        double *rule;
+        if ((rc = prepare_sep(ctx, mesh, op->op, op->prec, op->ng, gx, gw, hs.data(), sig, (int)nf, g.p, snear, ssing,
+                              &rule)))
+            return rc;
+        if ((rc = dalloc(ctx, &table, (size_t)std::max(np, 1) * nf * nv, &g.p)) || (rc = dalloc(ctx, &blk, 8, &g.p)) ||
             (rc = dalloc(ctx, &pre, 2, &g.p)))
             return rc;
         const int32_t hb[8] = {0, (int32_t)nr, 0, (int32_t)nc, 0, 0, 0, 0};  // block, then near_ids = {0}
         const int64_t hp[2] = {0, 0};                                        // eprefix, noff
         if ((rc = upload(ctx, blk, hb, 8)) || (rc = upload(ctx, pre, hp, 2))) return rc;
         MeshDev md = td_mesh_dev(mesh, op->ng, gx, gw, tp_slot);
-        lrc = td_launch_sing_table(ctx->stream, md, op->op, op->prec, pti, ptj, np, sig, (int)nf, table, ctx->num_sms);
+        lrc = td_launch_sing_sep(ctx->stream, md, op->op, pti, ptj, np, rule, ssing, (int)nf, table,
+                                 ctx->num_sms);
+        if (!lrc)
+            lrc = td_launch_sing_table(ctx->stream, md, op->op, op->prec, pti, ptj, np, rule, sig, (int)nf,
+                                       ssing.klist + ssing.nsep, ssing.ndir, table, ctx->num_sms);
         NearArgs na{};
         na.nf = (int)nf;
         na.sig = sig;
@@ -754,7 +811,10 @@ extern "C" int tdbem_entries_path(tdbem_mesh_t mesh, const tdbem_op *op, tdbem_f
         na.perm_c = cols;
         na.nentries = nr * nc;
         na.near = out;
-        if (!lrc) lrc = td_launch_near_entries(ctx->stream, md, op->op, op->prec, na, table, ctx->num_sms);
+        if (!lrc) lrc = td_launch_near_sep(ctx->stream, md, op->op, na, snear, table, ctx->num_sms);
+        if (!lrc)
+            lrc = td_launch_near_entries(ctx->stream, md, op->op, op->prec, na, snear.klist + snear.nsep, snear.ndir,
+                                         table, ctx->num_sms);
     }
     if (lrc) return td_fail(ctx, TDBEM_ERR_CUDA, "entry kernel launch failed: %s", cudaGetErrorString((cudaError_t)lrc));
     TD_CUDA(ctx, cudaStreamSynchronize(ctx->stream));  // transient buffers are freed on return
@@ -857,15 +917,16 @@ extern "C" int tdbem_compress(tdbem_ctx_t ctx, tdbem_mesh_t mesh, const tdbem_op
             max_near_rows = std::max(max_near_rows, nI);
         }
     }
-    // The near tensor [Nu][nI][nJ] per near block is formed and compressed in
-    // batches of consecutive near blocks of at most ctx->near_batch_bytes (one
-    // batch when it fits); every batch reuses one buffer.  eprefix / noff
-    // become offsets within the batch.
+    // FP64 form: the near tensor [Nu][nI][nJ] per near block is formed and
+    // compressed in batches of consecutive near blocks of at most
+    // ctx->near_batch_bytes (one batch when it fits); every batch reuses one
+    // buffer.  eprefix / noff become offsets within the batch.  The mixed form
+    // evaluates its near entries on demand: one batch, no buffer.
     std::vector<int> nbatch(1, 0);
     std::vector<int64_t> batch_nent;
     int64_t max_batch_tens = 1;
     {
-        const int64_t budget = std::max<int64_t>(1, ctx->near_batch_bytes / (int64_t)es);
+        const int64_t budget = pf ? INT64_MAX : std::max<int64_t>(1, ctx->near_batch_bytes / (int64_t)es);
         const int nn = (int)near_ids.size();
         int64_t acc = 0;
         for (int q = 0; q < nn; ++q) {
@@ -952,6 +1013,8 @@ extern "C" int tdbem_compress(tdbem_ctx_t ctx, tdbem_mesh_t mesh, const tdbem_op
         hs[2 * u] = f->s[2 * f->uidx[u]] / op->c;
         hs[2 * u + 1] = f->s[2 * f->uidx[u] + 1] / op->c;
     }
+    SepSet snear, ssing;
+    double *rule;
     c64 *table;
     char *nearbuf, *scr_near, *scr_far;
     int32_t *dnear_ids, *dfar_ids, *flags, *redo_a, *redo_b;
@@ -977,7 +1040,9 @@ extern "C" int tdbem_compress(tdbem_ctx_t ctx, tdbem_mesh_t mesh, const tdbem_op
     }
     const int64_t sper_far = (int64_t)kcap * (maxI + maxJ) + dense_cap + std::min<int64_t>(dense_cap, td_far_cd_max());
     if ((rc = dalloc(ctx, &sig, 2 * Nu, &g.p)) || (rc = upload(ctx, sig, hs.data(), hs.size())) ||
-        (rc = dalloc(ctx, &table, (size_t)npairs * Nu * 3, &g.p)) || (rc = dalloc(ctx, &nearbuf, es * max_batch_tens, &g.p)) ||
+        (rc = prepare_sep(ctx, mesh, op->op, op->prec, op->ng, gx, gw, hs.data(), sig, Nu, g.p, snear, ssing, &rule)) ||
+        (rc = dalloc(ctx, &table, (size_t)npairs * Nu * (op->op == TDBEM_DLP ? 3 : 1), &g.p)) ||
+        (rc = dalloc(ctx, &nearbuf, pf ? 0 : es * max_batch_tens, &g.p)) ||
         (rc = dalloc(ctx, &scr_near, es * maxIJ * nctas_near, &g.p)) ||
         (rc = dalloc(ctx, &scr_far, es * sper_far * nctas_far, &g.p)) ||
         (rc = dalloc(ctx, &dnear_ids, near_ids.size(), &g.p)) || (rc = dalloc(ctx, &dfar_ids, far_ids.size(), &g.p)) ||
@@ -1003,6 +1068,8 @@ extern "C" int tdbem_compress(tdbem_ctx_t ctx, tdbem_mesh_t mesh, const tdbem_op
     na.perm_c = T->dperm_c;
     na.nentries = nent;
     na.near = nearbuf;
+    na.table = table;
+    na.evals = evals;
     AcaParams ap{cfg->eps, cfg->eps_aca, kcap};
     FarArgs fa{};
     fa.nfar = (int)far_ids.size();
@@ -1089,12 +1156,13 @@ extern "C" int tdbem_compress(tdbem_ctx_t ctx, tdbem_mesh_t mesh, const tdbem_op
                 cudaMemsetAsync(counter, 0, sizeof(unsigned int) * 4, ls);
                 cudaMemsetAsync(redo_count, 0, sizeof(unsigned int) * 4, ls);
                 cudaMemsetAsync(T->drank, 0, sizeof(int32_t) * nb, ls);
-                lrc |= td_launch_sing_table(ls, md, op->op, op->prec, pti, ptj, npairs, sig, Nu, table, ctx->num_sms,
-                                            ctx->sing_var);
-                nlaunch += npairs > 0;
+                lrc |= td_launch_sing_sep(ls, md, op->op, pti, ptj, npairs, rule, ssing, Nu, table, ctx->num_sms);
+                lrc |= td_launch_sing_table(ls, md, op->op, op->prec, pti, ptj, npairs, rule, sig, Nu,
+                                            ssing.klist + ssing.nsep, ssing.ndir, table, ctx->num_sms, ctx->sing_var);
+                nlaunch += npairs > 0 ? (ssing.nsep > 0) + (ssing.ndir > 0) : 0;
             } else if (ph == 1 || ph == 2) {
-                // one batch: entries (phase 1) and 3D-ACA (phase 2); several: both per
-                // batch in phase 1
+                // one batch: entries (phase 1, FP64 form) and 3D-ACA (phase 2); several:
+                // both per batch in phase 1
                 const int nbt = (int)batch_nent.size();
                 for (int bt = 0; bt < nbt; ++bt) {
                     NearArgs nab = na;
@@ -1105,13 +1173,14 @@ extern "C" int tdbem_compress(tdbem_ctx_t ctx, tdbem_mesh_t mesh, const tdbem_op
                     nab.noff = dnoff + q0;
                     nab.nentries = batch_nent[bt];
                     const int nct = std::min(nctas_near, nab.nnear);
-                    if (ph == 1) {
-                        lrc |= td_launch_near_entries(ls, md, op->op, op->prec, nab, table, ctx->num_sms,
-                                                      ctx->near_var);
-                        nlaunch += nab.nentries > 0;
+                    if (ph == 1 && !pf) {
+                        lrc |= td_launch_near_sep(ls, md, op->op, nab, snear, table, ctx->num_sms);
+                        lrc |= td_launch_near_entries(ls, md, op->op, op->prec, nab, snear.klist + snear.nsep,
+                                                      snear.ndir, table, ctx->num_sms, ctx->near_var);
+                        nlaunch += nab.nentries > 0 ? (snear.nsep > 0) + (snear.ndir > 0) : 0;
                     }
                     if ((ph == 2 && nbt == 1) || (ph == 1 && nbt > 1)) {
-                        lrc |= td_launch_near_aca(ls, op->prec, nab, o, ap, scr_near, maxIJ, nct);
+                        lrc |= td_launch_near_aca(ls, md, op->op, op->prec, nab, o, ap, scr_near, maxIJ, nct);
                         nlaunch += nab.nnear > 0;
                     }
                 }
@@ -1279,7 +1348,7 @@ extern "C" int tdbem_compress(tdbem_ctx_t ctx, tdbem_mesh_t mesh, const tdbem_op
         }
     }
     st.dense_complex = T->nrows * T->ncols * (int64_t)Nu;
-    st.entries_regular = nent * Nu + hev[0];
+    st.entries_regular = (pf ? 0 : nent * Nu) + hev[0];
     st.entries_tube = hev[1];
     st.aca_tests = hev[2];
     st.pairs_singular = (int64_t)npairs * Nu;
@@ -1733,38 +1802,31 @@ extern "C" int tdbem_autotune(tdbem_ctx_t ctx, tdbem_mesh_t mesh, const tdbem_op
     }
     ctx->far_nt[pf] = bnt;
     ctx->far_cps[pf] = bcps;
-    // 2. mixed form: frequencies per pass of the touching-pair table and of the
-    // near-field tensor kernel (register tiles of FC frequencies), each phase
-    // timed on its own from the same compressions
-    int bsing = ctx->sing_var, bnear = ctx->near_var;
+    // 2. mixed form: frequencies per pass of the touching-pair table (register tiles
+    // of FC frequencies), timed on its own phase
+    int bsing = ctx->sing_var;
     if (pf) {
-        double ts = 1e300, tn = 1e300;
+        double ts = 1e300;
         for (int v = 0; v < 3; ++v) {
-            ctx->sing_var = ctx->near_var = v;
+            ctx->sing_var = v;
             tdbem_stats st{};
             const int rc = run(st);
             if (rc) {
                 ctx->sing_var = bsing;
-                ctx->near_var = bnear;
                 return rc;
             }
             if (st.ms_singular < ts) {
                 ts = st.ms_singular;
                 bsing = v;
             }
-            if (st.ms_near < tn) {
-                tn = st.ms_near;
-                bnear = v;
-            }
         }
         ctx->sing_var = bsing;
-        ctx->near_var = bnear;
     }
     if (chosen) {
         chosen[0] = bnt;
         chosen[1] = bcps;
         chosen[2] = pf ? td_sing_fc(op->op, bsing) : 0;
-        chosen[3] = pf ? td_near_fc(bnear) : 0;
+        chosen[3] = pf ? td_near_fc(ctx->near_var) : 0;
     }
     return TDBEM_OK;
 }

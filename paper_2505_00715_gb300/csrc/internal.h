@@ -54,6 +54,9 @@ struct tdbem_mesh {
     std::vector<double> verts;
     std::vector<int32_t> tris;
     std::vector<double> area;
+    // longest edge; largest distance of a rule point from its triangle's centroid
+    // and from one of its vertices (distance intervals of the separated sums)
+    double edge_max = 0.0, rad_tri = 0.0, rad_vert = 0.0;
     // vertex -> triangle incidence (P1 supports)
     std::vector<int32_t> v2t_ptr, v2t;
     std::vector<int8_t> v2t_loc;
@@ -149,6 +152,11 @@ int td_noalloc_setup(int device);
 
 // api.cu: radius factor of the gCQ contour for nsteps steps of method rk
 double td_gcq_radius(int rk, int nsteps);
+
+// k_sep.cu: separated and direct frequencies of the host list sigma = s / c
+// (interleaved, nf values) for distance half interval D; fills s.nsep, ndir, P, D
+struct SepSet;
+void td_sep_split(int op, int prec, const double *sigma, int nf, double D, bool touching, std::vector<int> &klist, SepSet &s);
 
 // planner.cpp
 void td_plan_tree(const tdbem_mesh *m, int basis, int leaf, HostTree &t);

@@ -8,8 +8,8 @@
 //   stop when ||H_l||_F ||f_l|| <= eps ||C^(l)||_F  (the last term is dropped),
 //   ||C^(l)||_F^2 = sum_{d,d'} <H_d, H_d'> <f_d, f_d'>   (eq. norm, FP64),
 //   k_{l+1} = argmax |f_l[k]| over frequencies not selected yet.
-// Near-field blocks (k_near_aca): dense faces from the precomputed near tensor,
-// one CTA per block.  Far-field blocks (k_far_aca): every residual face is
+// Near-field blocks (k_near_aca): dense faces, from the precomputed near tensor
+// (FP64 form) or evaluated on demand (mixed form), one CTA per block.  Far-field blocks (k_far_aca): every residual face is
 // compressed by ACA with partial pivoting (row fibre at i*, column fibre at
 // j*, FP64 norm recursion of the matrix analogue of eq. norm) from entries
 // evaluated on the fly; the face is rebuilt to find the pivot and discarded
@@ -21,7 +21,7 @@
 
 #include "internal.h"
 #include "kernels.h"
-#include "pair.cuh"
+#include "near.cuh"
 
 namespace {
 
@@ -87,8 +87,16 @@ TD_D cx<T> lowrank_at(const cx<T> *U, int64_t su, const cx<T> *V, int64_t sv, in
 // ============================================================================
 // Near field
 // ============================================================================
-template <class T>
-__global__ void __launch_bounds__(128) k_near_aca(NearArgs a, TensorOut o, AcaParams p,
+// FP64 form (OP = -1): the entries of every frequency come from the near tensor.
+// Mixed form: Algorithm 1 reads one face per selected frequency and one tube per
+// term, so the entries are evaluated as they are asked for, with the sums of the
+// near tensor's kernel (same values).  A face entry costs about 1.7 x an entry of
+// the near tensor (its geometry is not shared between frequencies), but on the 30k
+// housing a block asks for 8 of 128 frequencies: near field 229 -> 29 ms, and no
+// near tensor of 28 GB; on the 5120-triangle sphere (12 of 33) 5.5 -> 3.6 ms.
+// Bound: FP32 issue (40 instructions per point pair).
+template <class T, int OP>
+__global__ void __launch_bounds__(128) k_near_aca(MeshDev m, NearArgs a, TensorOut o, AcaParams p,
                                                   cx<T> *scratch, int64_t sper) {
     using AM = typename AmOf<T>::type;
     __shared__ cx<T> s_fl[kMaxNu];
@@ -106,12 +114,21 @@ __global__ void __launch_bounds__(128) k_near_aca(NearArgs a, TensorOut o, AcaPa
     cx<T> *H = scratch + (int64_t)blockIdx.x * sper;
     cx<T> *fib = (cx<T> *)o.fib;
     cx<T> *pool = (cx<T> *)o.face;
+    long long ev_face = 0, ev_tube = 0;  // entries evaluated on demand
     for (int nb = blockIdx.x; nb < a.nnear; nb += gridDim.x) {
         const int b = a.near_ids[nb];
         const int *bl = a.blocks + 5 * b;
         const int nI = bl[1] - bl[0], nJ = bl[3] - bl[2];
         const int64_t nIJ = (int64_t)nI * nJ;
-        const cx<T> *N = (const cx<T> *)a.near + a.noff[nb];
+        const cx<T> *N = OP < 0 ? (const cx<T> *)a.near + a.noff[nb] : nullptr;
+        const int *rows = a.perm_r + bl[0], *cols = a.perm_c + bl[2];
+        // entry (i, j) of the block at frequency kk
+        auto entry = [&](int i, int j, int e, int kk) -> cx<T> {
+            if constexpr (OP >= 0)
+                return near_entry<OP>(m, rows[i], cols[j], (float)a.sig[2 * kk], (float)a.sig[2 * kk + 1], a.table, Nu, kk);
+            else
+                return N[kk * nIJ + e];
+        };
         const int64_t tb = (int64_t)b * Nu;
         for (int kk = tid; kk < Nu; kk += blockDim.x) s_sel[kk] = 0;
         if (tid == 0) s_normC2 = 0.0;
@@ -125,22 +142,25 @@ __global__ void __launch_bounds__(128) k_near_aca(NearArgs a, TensorOut o, AcaPa
             }
             __syncthreads();
             for (int64_t e = tid; e < nIJ; e += blockDim.x) {
-                cx<T> h = apply_coef(N[k * nIJ + e], s_fk, s_base, l, (int)e);
+                const int i = (int)e / nJ;
+                cx<T> h = apply_coef(entry(i, (int)e - i * nJ, (int)e, k), s_fk, s_base, l, (int)e);
                 H[e] = h;
                 const auto key = pivot_key(h);
                 if (am_better(key, (int)e, am.v, am.i)) am = {key, (int)e};
             }
+            ev_face += nIJ;
             am = block_argmax(am, red);
             if (!(am.v > 0)) {
                 r = l;
                 break;
             }
             const int ep = am.i;
+            ev_tube += Nu;
             const cx<T> piv = H[ep];
             for (int d = tid; d < l; d += blockDim.x) s_hd[d] = pool[o.foff[tb + d] + ep];
             __syncthreads();
             for (int kk = tid; kk < Nu; kk += blockDim.x) {
-                cx<T> v = N[kk * nIJ + ep];
+                cx<T> v = entry(ep / nJ, ep % nJ, ep, kk);
                 for (int d = 0; d < l; ++d) cfms(v, s_hd[d], fib[(tb + d) * Nu + kk]);
                 s_fl[kk] = cdiv(v, piv);
             }
@@ -218,6 +238,10 @@ __global__ void __launch_bounds__(128) k_near_aca(NearArgs a, TensorOut o, AcaPa
         if (r < 0) r = l;
         if (tid == 0) o.rank[b] = r;
         __syncthreads();
+    }
+    if (OP >= 0 && tid == 0 && a.evals) {
+        atomicAdd((unsigned long long *)&a.evals[0], (unsigned long long)ev_face);
+        atomicAdd((unsigned long long *)&a.evals[1], (unsigned long long)ev_tube);
     }
 }
 
@@ -1397,13 +1421,13 @@ int td_launch_fibre_entries(cudaStream_t st, const MeshDev &m, int op, int prec,
     return (int)cudaGetLastError();
 }
 
-int td_launch_near_aca(cudaStream_t st, int prec, const NearArgs &a, const TensorOut &o,
+int td_launch_near_aca(cudaStream_t st, const MeshDev &m, int op, int prec, const NearArgs &a, const TensorOut &o,
                        const AcaParams &p, void *scratch, int64_t sper, int nctas) {
     if (a.nnear == 0) return 0;
-    if (prec == TDBEM_FP64)
-        k_near_aca<double><<<nctas, 128, 0, st>>>(a, o, p, (c64 *)scratch, sper);
-    else
-        k_near_aca<float><<<nctas, 128, 0, st>>>(a, o, p, (c32 *)scratch, sper);
+    if (prec == TDBEM_FP64) k_near_aca<double, -1><<<nctas, 128, 0, st>>>(m, a, o, p, (c64 *)scratch, sper);
+    else if (op == TD_SLP) k_near_aca<float, TD_SLP><<<nctas, 128, 0, st>>>(m, a, o, p, (c32 *)scratch, sper);
+    else if (op == TD_DLP) k_near_aca<float, TD_DLP><<<nctas, 128, 0, st>>>(m, a, o, p, (c32 *)scratch, sper);
+    else k_near_aca<float, TD_ADLP><<<nctas, 128, 0, st>>>(m, a, o, p, (c32 *)scratch, sper);
     return (int)cudaGetLastError();
 }
 

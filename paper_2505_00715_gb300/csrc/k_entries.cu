@@ -1,15 +1,17 @@
 // Entry kernels (Sec. 3; the ENTRY function of Algorithm 1):
 //   k_entries_generic : arbitrary rows x cols x frequencies (C-ABI tdbem_entries)
 //   (operators: single layer, double layer, adjoint double layer K')
-//   k_sing_table      : touching pairs (Sauter-Schwab, FP64) at all unique
+//   k_sing_table      : touching pairs (Sauter-Schwab, FP64) at a list of
 //                       frequencies, one warp per pair
-//   k_near_entries    : every entry of every near-field block at all unique
+//   k_near_entries    : every entry of a list of near-field blocks at a list of
 //                       frequencies; regular pairs in the block precision with
 //                       the quadrature geometry shared across frequencies,
 //                       touching pairs read from the table.
+// In the compression the FP64 form takes most frequencies by the separated sums
+// of k_sep.cu, and the mixed form forms its near entries on demand (k_near_aca).
 #include "internal.h"
 #include "kernels.h"
-#include "pair.cuh"
+#include "near.cuh"
 
 namespace {
 
@@ -69,10 +71,13 @@ __global__ void k_entries_generic(MeshDev m, const double *sig, int nq, const in
 }
 
 // ---- touching-pair table ----------------------------------------------------
-// table layout: [slot][nf][3] complex128 (SLP uses component 0), 1/(4 pi) applied.
+// table layout: [slot][nf][1 or 3 (P1 columns)] complex128, 1/(4 pi) applied.
+// Both forms run the nd frequencies of klist, those that the separated sums
+// (k_sep.cu) leave: |sigma| times the longest edge beyond their terms.
 template <int OP, int FC>
 __global__ void k_sing_table(MeshDev m, const int *pti, const int *ptj, int npairs,
-                             const double *sig, int nf, c64 *table) {
+                             const double *sig, int nf, const int *klist, int nd, c64 *table) {
+    constexpr int NV = TD_P1_TRIAL(OP) ? 3 : 1;
     const int lane = threadIdx.x & 31;
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int nwarps = (gridDim.x * blockDim.x) >> 5;
@@ -87,7 +92,7 @@ __global__ void k_sing_table(MeshDev m, const int *pti, const int *ptj, int npai
         classify_pair(m, ti, tj, G);
         const int nq = ss_npoints(G.cls, m.ng);
         const bool zero = (OP != TD_SLP && G.cls == 3) || G.cls == 0;
-        for (int f0 = 0; f0 < nf; f0 += FC) {
+        for (int f0 = 0; f0 < nd; f0 += FC) {
             c64 acc[FC][3];
 #pragma unroll
             for (int j = 0; j < FC; ++j)
@@ -106,8 +111,9 @@ __global__ void k_sing_table(MeshDev m, const int *pti, const int *ptj, int npai
                     (void)pre;
 #pragma unroll
                     for (int j = 0; j < FC; ++j) {
-                        if (f0 + j < nf) {
-                            double sr = sig[2 * (f0 + j)], si = sig[2 * (f0 + j) + 1];
+                        if (f0 + j < nd) {
+                            const int kf = klist[f0 + j];
+                            double sr = sig[2 * kf], si = sig[2 * kf + 1];
                             c64 e = expm_sr(sr, si, r);
                             if (OP == TD_SLP) {
                                 acc[j][0].x += base * e.x;
@@ -137,11 +143,10 @@ __global__ void k_sing_table(MeshDev m, const int *pti, const int *ptj, int npai
 #pragma unroll
                 for (int k = 0; k < 3; ++k)
                     outv[k] = {warp_sum(acc[j][k].x) * inv4pi, warp_sum(acc[j][k].y) * inv4pi};
-                if (lane == 0 && f0 + j < nf) {
-                    c64 *o = table + ((int64_t)p * nf + f0 + j) * 3;
+                if (lane == 0 && f0 + j < nd) {
+                    c64 *o = table + ((int64_t)p * nf + klist[f0 + j]) * NV;
                     if (!TD_P1_TRIAL(OP)) {
                         o[0] = zero ? c64{0.0, 0.0} : outv[0];
-                        o[1] = o[2] = {0.0, 0.0};
                     } else {
                         // parametrisation order -> mesh-local trial vertex
                         c64 z = {0.0, 0.0};
@@ -162,18 +167,22 @@ __global__ void k_sing_table(MeshDev m, const int *pti, const int *ptj, int npai
 // are FP32.  The points of a pair are taken in chunks of 32 P (P per lane,
 // held in registers): the FP64 point geometry of a chunk is formed once and
 // reused by every frequency, FC frequencies per pass; each pass's lane sums
-// are reduced over the warp and added to the pair's table rows.
+// are reduced over the warp and added to the pair's table rows.  The reference
+// points come from an array formed once per call (k_ss_rule): a point then takes
+// 18 FP64 operations instead of about 100 (30k housing: 65 -> 43 ms; bound by FP32
+// issue, 24 instructions per point and frequency, and by the FP64 pipe).
 template <int OP, int FC>
-__global__ void k_sing_table_mixed(MeshDev m, const int *pti, const int *ptj, int npairs, const double *sig,
-                                   int nf, c64 *table) {
+__global__ void k_sing_table_mixed(MeshDev m, const int *pti, const int *ptj, int npairs, const double *rule,
+                                   const double *sig, int nf, const int *klist, int nd, c64 *table) {
     const int lane = threadIdx.x & 31;
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int nwarps = (gridDim.x * blockDim.x) >> 5;
     constexpr int NV = TD_P1_TRIAL(OP) ? 3 : 1;
     constexpr int P = TD_P1_TRIAL(OP) ? 8 : 16;  // points per lane and chunk
-    // s / c of every frequency in shared memory (nf <= 256, checked by the caller)
+    // s / c of every frequency in shared memory (nd <= nf <= 256, checked by the caller)
     __shared__ float2 s_sig[256];
-    for (int k = threadIdx.x; k < nf; k += blockDim.x) s_sig[k] = make_float2((float)sig[2 * k], (float)sig[2 * k + 1]);
+    for (int k = threadIdx.x; k < nd; k += blockDim.x)
+        s_sig[k] = make_float2((float)sig[2 * klist[k]], (float)sig[2 * klist[k] + 1]);
     __syncthreads();
     const double inv4pi = 1.0 / TD_FOUR_PI;
     for (int p = warp; p < npairs; p += nwarps) {
@@ -187,10 +196,13 @@ __global__ void k_sing_table_mixed(MeshDev m, const int *pti, const int *ptj, in
         classify_pair(m, ti, tj, G);
         const int nq = ss_npoints(G.cls, m.ng);
         const bool zero = (OP != TD_SLP && G.cls == 3) || G.cls == 0;
-        c64 *o = table + (int64_t)p * nf * 3;
-        for (int e = lane; e < nf * 3; e += 32) o[e] = c64{0.0, 0.0};
+        c64 *o = table + (int64_t)p * nf * NV;
+        for (int e = lane; e < nd * NV; e += 32) o[(int64_t)klist[e / NV] * NV + e % NV] = c64{0.0, 0.0};
         __syncwarp();
         if (zero) continue;
+        SsEdges E;
+        ss_edges(G, E);
+        const double *rl = rule + ss_rule_off(G.cls, m.ng);
         for (int q0 = 0; q0 < nq; q0 += 32 * P) {
             // the transformed point and the difference x - y in FP64 (no
             // cancellation near the singularity); |d|^2 is exact to FP64
@@ -205,17 +217,20 @@ __global__ void k_sing_table_mixed(MeshDev m, const int *pti, const int *ptj, in
 #pragma unroll
                 for (int k = 0; k < NV; ++k) lf[i][k] = 0.0f;
                 if (q < nq) {
-                    double d[3], w, lam[3];
-                    ss_point(G, q, m.ng, m.gx, m.gw, d, w, lam);
+                    double a[4], d[3];
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) a[e] = __ldg(rl + (int64_t)e * nq + q);
+                    const double w = __ldg(rl + (int64_t)4 * nq + q) * G.g;
+                    ss_diff(G.cls, a, E, d);
                     const float r2 = (float)(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
                     const float rinv = rsqrtf(r2);
                     rf[i] = r2 * rinv;
                     bf[i] = OP == TD_SLP ? (float)w * rinv : (float)w * (float)ss_dn<OP>(G, d) * rinv * rinv * rinv;
 #pragma unroll
-                    for (int k = 0; k < NV; ++k) lf[i][k] = TD_P1_TRIAL(OP) ? (float)lam[k] : 1.0f;
+                    for (int k = 0; k < NV; ++k) lf[i][k] = TD_P1_TRIAL(OP) ? (float)__ldg(rl + (int64_t)(5 + k) * nq + q) : 1.0f;
                 }
             }
-            for (int f0 = 0; f0 < nf; f0 += FC) {
+            for (int f0 = 0; f0 < nd; f0 += FC) {
                 c32 acc[FC][NV];
 #pragma unroll
                 for (int j = 0; j < FC; ++j)
@@ -225,7 +240,7 @@ __global__ void k_sing_table_mixed(MeshDev m, const int *pti, const int *ptj, in
                 for (int i = 0; i < P; ++i) {
 #pragma unroll
                     for (int j = 0; j < FC; ++j) {
-                        const float2 sgj = s_sig[min(f0 + j, nf - 1)];
+                        const float2 sgj = s_sig[min(f0 + j, nd - 1)];
                         const c32 e = expm_sr(sgj.x, sgj.y, rf[i]);
                         c32 v;
                         if (OP == TD_SLP) {
@@ -247,8 +262,8 @@ __global__ void k_sing_table_mixed(MeshDev m, const int *pti, const int *ptj, in
 #pragma unroll
                     for (int k = 0; k < NV; ++k) {
                         const float sx = warp_sum(acc[j][k].x), sy = warp_sum(acc[j][k].y);
-                        if (lane == 0 && f0 + j < nf) {
-                            c64 &t = o[(int64_t)(f0 + j) * 3 + (TD_P1_TRIAL(OP) ? G.loc[k] : 0)];
+                        if (lane == 0 && f0 + j < nd) {
+                            c64 &t = o[(int64_t)klist[f0 + j] * NV + (TD_P1_TRIAL(OP) ? G.loc[k] : 0)];
                             t.x += (double)sx * inv4pi;
                             t.y += (double)sy * inv4pi;
                         }
@@ -260,56 +275,7 @@ __global__ void k_sing_table_mixed(MeshDev m, const int *pti, const int *ptj, in
 }
 
 // ---- near-field dense entries -------------------------------------------------
-// Regular pair at FC frequencies with the geometry computed once per point
-// pair (test triangle in registers, trial points streamed from the tables).
-template <int OP, int FC>
-TD_D void pair_multi(const TestF &X, const MeshDev &m, int tj, const float *sg, int nfc, c32 *acc, int loc) {
-    // signed kernel normal: -n_y (DLP) or +n_x (ADLP), multiplied by d = y - x
-    float nx = 0.f, ny = 0.f, nz = 0.f;
-    if (OP == TD_DLP) {
-        nx = -m.n32[tj];
-        ny = -m.n32[m.nt + tj];
-        nz = -m.n32[2 * m.nt + tj];
-    } else if (OP == TD_ADLP) {
-        nx = X.nx;
-        ny = X.ny;
-        nz = X.nz;
-    }
-#pragma unroll 1
-    for (int b = 0; b < 7; ++b) {
-        const int ob = b * m.nt + tj;
-        const float yxh = m.qxh[ob], yyh = m.qyh[ob], yzh = m.qzh[ob];
-        const float yxl = m.qxl[ob], yyl = m.qyl[ob], yzl = m.qzl[ob];
-        const float wyb = m.qw32[ob] * (OP == TD_DLP ? bary7f(b, loc) : 1.0f);
-#pragma unroll
-        for (int a = 0; a < 7; ++a) {
-            const float dx = (yxh - X.xh[a]) + (yxl - X.xl[a]);
-            const float dy = (yyh - X.yh[a]) + (yyl - X.yl[a]);
-            const float dz = (yzh - X.zh[a]) + (yzl - X.zl[a]);
-            const float r2 = dx * dx + dy * dy + dz * dz;
-            const float rinv = rsqrtf(r2);
-            const float r = r2 * rinv;
-            float w = X.w[a] * wyb * rinv;
-            if (OP != TD_SLP) w *= (dx * nx + dy * ny + dz * nz) * rinv * rinv;
-#pragma unroll
-            for (int j = 0; j < FC; ++j) {
-                if (j < nfc) {
-                    const float sr = sg[2 * j], si = sg[2 * j + 1];
-                    const c32 e = expm_sr(sr, si, r);
-                    if (OP == TD_SLP) {
-                        acc[j].x = fmaf(w, e.x, acc[j].x);
-                        acc[j].y = fmaf(w, e.y, acc[j].y);
-                    } else {
-                        const float pr = fmaf(sr, r, 1.0f), pi = si * r;
-                        acc[j].x = fmaf(w, pr * e.x - pi * e.y, acc[j].x);
-                        acc[j].y = fmaf(w, pr * e.y + pi * e.x, acc[j].y);
-                    }
-                }
-            }
-        }
-    }
-}
-
+// FP64 version of pair_multi (near.cuh).
 template <int OP, int FC>
 TD_D void pair_multi(const TestD &X, const MeshDev &m, int tj, const double *sg, int nfc, c64 *acc, int loc) {
     double nx = 0.0, ny = 0.0, nz = 0.0;  // signed kernel normal, as in the FP32 version
@@ -353,13 +319,14 @@ TD_D void pair_multi(const TestD &X, const MeshDev &m, int tj, const double *sg,
 }
 
 // near[noff[b] + (k * nI + i) * nJ + j] for every near block b (list nb_idx),
-// all nf unique frequencies.  Entry e of the flattened list belongs to the
+// the nd frequencies of klist (those that the separated sums of k_sep.cu leave).  Entry e of the flattened list belongs to the
 // near block found by binary search in the prefix `eprefix` (entries per block).
 template <class T, int OP, int FC>
-__global__ void __launch_bounds__(128) k_near_entries(MeshDev m, NearArgs a, const c64 *table) {
+__global__ void __launch_bounds__(128) k_near_entries(MeshDev m, NearArgs a, const int *klist, int nd, const c64 *table) {
+    constexpr int NV = TD_P1_TRIAL(OP) ? 3 : 1;
     __shared__ T sg[2 * 256];
     const int nf = a.nf;  // <= 256 (checked by the caller)
-    for (int i = threadIdx.x; i < 2 * nf; i += blockDim.x) sg[i] = (T)a.sig[i];
+    for (int i = threadIdx.x; i < 2 * nd; i += blockDim.x) sg[i] = (T)a.sig[2 * klist[i >> 1] + (i & 1)];
     __syncthreads();
     for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < a.nentries;
          t += (int64_t)gridDim.x * blockDim.x) {
@@ -380,8 +347,8 @@ __global__ void __launch_bounds__(128) k_near_entries(MeshDev m, NearArgs a, con
         typename Reg<T>::Test X;
         load_test(m, row, X);
         const int nsup = TD_P1_TRIAL(OP) ? m.v2t_ptr[col + 1] - m.v2t_ptr[col] : 1;
-        for (int f0 = 0; f0 < nf; f0 += FC) {
-            const int nfc = min(FC, nf - f0);
+        for (int f0 = 0; f0 < nd; f0 += FC) {
+            const int nfc = min(FC, nd - f0);
             cx<T> acc[FC];
 #pragma unroll
             for (int jj = 0; jj < FC; ++jj) acc[jj] = {0, 0};
@@ -402,7 +369,7 @@ __global__ void __launch_bounds__(128) k_near_entries(MeshDev m, NearArgs a, con
                 if (slot >= 0) {
 #pragma unroll
                     for (int jj = 0; jj < FC; ++jj)
-                        if (jj < nfc) sing[jj] = sing[jj] + table[((int64_t)slot * nf + f0 + jj) * 3 + l];
+                        if (jj < nfc) sing[jj] = sing[jj] + table[((int64_t)slot * nf + klist[f0 + jj]) * NV + l];
                 } else {
                     pair_multi<OP, FC>(X, m, e, sg + 2 * f0, nfc, acc, l);
                 }
@@ -411,7 +378,7 @@ __global__ void __launch_bounds__(128) k_near_entries(MeshDev m, NearArgs a, con
 #pragma unroll
             for (int jj = 0; jj < FC; ++jj)
                 if (jj < nfc)
-                    dst[(int64_t)(f0 + jj) * fstride] =
+                    dst[klist[f0 + jj] * fstride] =
                         cx<T>{(T)(acc[jj].x * inv4pi + (T)sing[jj].x), (T)(acc[jj].y * inv4pi + (T)sing[jj].y)};
         }
     }
@@ -455,58 +422,59 @@ int td_sing_fc(int op, int variant) { return op == TD_DLP ? kSingFcDlp[variant %
 int td_near_fc(int variant) { return kNearFc[variant % 3]; }
 
 int td_launch_sing_table(cudaStream_t st, const MeshDev &m, int op, int prec, const int *pti, const int *ptj,
-                         int npairs, const double *sig, int nf, c64 *table, int num_sms, int variant) {
-    if (npairs == 0) return 0;
+                         int npairs, const double *rule, const double *sig, int nf, const int *klist, int nd,
+                         c64 *table, int num_sms, int variant) {
+    if (npairs == 0 || nd == 0) return 0;
     if (nf > 256) return (int)cudaErrorInvalidValue;  // the frequencies are staged in shared memory
     int grid = std::min((npairs + 3) / 4, num_sms * 8);
     if (prec == TDBEM_MIXED) {
         const int v = variant % 3;
         if (op == TD_SLP) {
-            if (v == 1) k_sing_table_mixed<TD_SLP, 8><<<grid, 128, 0, st>>>(m, pti, ptj, npairs, sig, nf, table);
-            else if (v == 2) k_sing_table_mixed<TD_SLP, 16><<<grid, 128, 0, st>>>(m, pti, ptj, npairs, sig, nf, table);
-            else k_sing_table_mixed<TD_SLP, 4><<<grid, 128, 0, st>>>(m, pti, ptj, npairs, sig, nf, table);
+            if (v == 1) k_sing_table_mixed<TD_SLP, 8><<<grid, 128, 0, st>>>(m, pti, ptj, npairs, rule, sig, nf, klist, nd, table);
+            else if (v == 2) k_sing_table_mixed<TD_SLP, 16><<<grid, 128, 0, st>>>(m, pti, ptj, npairs, rule, sig, nf, klist, nd, table);
+            else k_sing_table_mixed<TD_SLP, 4><<<grid, 128, 0, st>>>(m, pti, ptj, npairs, rule, sig, nf, klist, nd, table);
         } else if (op == TD_DLP) {
-            if (v == 1) k_sing_table_mixed<TD_DLP, 4><<<grid, 128, 0, st>>>(m, pti, ptj, npairs, sig, nf, table);
-            else if (v == 2) k_sing_table_mixed<TD_DLP, 8><<<grid, 128, 0, st>>>(m, pti, ptj, npairs, sig, nf, table);
-            else k_sing_table_mixed<TD_DLP, 2><<<grid, 128, 0, st>>>(m, pti, ptj, npairs, sig, nf, table);
+            if (v == 1) k_sing_table_mixed<TD_DLP, 4><<<grid, 128, 0, st>>>(m, pti, ptj, npairs, rule, sig, nf, klist, nd, table);
+            else if (v == 2) k_sing_table_mixed<TD_DLP, 8><<<grid, 128, 0, st>>>(m, pti, ptj, npairs, rule, sig, nf, klist, nd, table);
+            else k_sing_table_mixed<TD_DLP, 2><<<grid, 128, 0, st>>>(m, pti, ptj, npairs, rule, sig, nf, klist, nd, table);
         } else {
-            if (v == 1) k_sing_table_mixed<TD_ADLP, 8><<<grid, 128, 0, st>>>(m, pti, ptj, npairs, sig, nf, table);
-            else if (v == 2) k_sing_table_mixed<TD_ADLP, 16><<<grid, 128, 0, st>>>(m, pti, ptj, npairs, sig, nf, table);
-            else k_sing_table_mixed<TD_ADLP, 4><<<grid, 128, 0, st>>>(m, pti, ptj, npairs, sig, nf, table);
+            if (v == 1) k_sing_table_mixed<TD_ADLP, 8><<<grid, 128, 0, st>>>(m, pti, ptj, npairs, rule, sig, nf, klist, nd, table);
+            else if (v == 2) k_sing_table_mixed<TD_ADLP, 16><<<grid, 128, 0, st>>>(m, pti, ptj, npairs, rule, sig, nf, klist, nd, table);
+            else k_sing_table_mixed<TD_ADLP, 4><<<grid, 128, 0, st>>>(m, pti, ptj, npairs, rule, sig, nf, klist, nd, table);
         }
         return (int)cudaGetLastError();
     }
     if (op == TD_SLP)
-        k_sing_table<TD_SLP, 8><<<grid, 128, 0, st>>>(m, pti, ptj, npairs, sig, nf, table);
+        k_sing_table<TD_SLP, 8><<<grid, 128, 0, st>>>(m, pti, ptj, npairs, sig, nf, klist, nd, table);
     else if (op == TD_DLP)
-        k_sing_table<TD_DLP, 4><<<grid, 128, 0, st>>>(m, pti, ptj, npairs, sig, nf, table);
+        k_sing_table<TD_DLP, 4><<<grid, 128, 0, st>>>(m, pti, ptj, npairs, sig, nf, klist, nd, table);
     else
-        k_sing_table<TD_ADLP, 4><<<grid, 128, 0, st>>>(m, pti, ptj, npairs, sig, nf, table);
+        k_sing_table<TD_ADLP, 4><<<grid, 128, 0, st>>>(m, pti, ptj, npairs, sig, nf, klist, nd, table);
     return (int)cudaGetLastError();
 }
 
-int td_launch_near_entries(cudaStream_t st, const MeshDev &m, int op, int prec, const NearArgs &a,
-                           const c64 *table, int num_sms, int variant) {
-    if (a.nentries == 0) return 0;
+int td_launch_near_entries(cudaStream_t st, const MeshDev &m, int op, int prec, const NearArgs &a, const int *klist,
+                           int nd, const c64 *table, int num_sms, int variant) {
+    if (a.nentries == 0 || nd == 0) return 0;
     int grid = (int)std::min<int64_t>((a.nentries + 127) / 128, (int64_t)num_sms * 16);
     if (prec == TDBEM_FP64) {
-        if (op == TD_SLP) k_near_entries<double, TD_SLP, 4><<<grid, 128, 0, st>>>(m, a, table);
-        else if (op == TD_DLP) k_near_entries<double, TD_DLP, 4><<<grid, 128, 0, st>>>(m, a, table);
-        else k_near_entries<double, TD_ADLP, 4><<<grid, 128, 0, st>>>(m, a, table);
+        if (op == TD_SLP) k_near_entries<double, TD_SLP, 4><<<grid, 128, 0, st>>>(m, a, klist, nd, table);
+        else if (op == TD_DLP) k_near_entries<double, TD_DLP, 4><<<grid, 128, 0, st>>>(m, a, klist, nd, table);
+        else k_near_entries<double, TD_ADLP, 4><<<grid, 128, 0, st>>>(m, a, klist, nd, table);
     } else {
         const int v = variant % 3;
         if (op == TD_SLP) {
-            if (v == 1) k_near_entries<float, TD_SLP, 4><<<grid, 128, 0, st>>>(m, a, table);
-            else if (v == 2) k_near_entries<float, TD_SLP, 16><<<grid, 128, 0, st>>>(m, a, table);
-            else k_near_entries<float, TD_SLP, 8><<<grid, 128, 0, st>>>(m, a, table);
+            if (v == 1) k_near_entries<float, TD_SLP, 4><<<grid, 128, 0, st>>>(m, a, klist, nd, table);
+            else if (v == 2) k_near_entries<float, TD_SLP, 16><<<grid, 128, 0, st>>>(m, a, klist, nd, table);
+            else k_near_entries<float, TD_SLP, 8><<<grid, 128, 0, st>>>(m, a, klist, nd, table);
         } else if (op == TD_DLP) {
-            if (v == 1) k_near_entries<float, TD_DLP, 4><<<grid, 128, 0, st>>>(m, a, table);
-            else if (v == 2) k_near_entries<float, TD_DLP, 16><<<grid, 128, 0, st>>>(m, a, table);
-            else k_near_entries<float, TD_DLP, 8><<<grid, 128, 0, st>>>(m, a, table);
+            if (v == 1) k_near_entries<float, TD_DLP, 4><<<grid, 128, 0, st>>>(m, a, klist, nd, table);
+            else if (v == 2) k_near_entries<float, TD_DLP, 16><<<grid, 128, 0, st>>>(m, a, klist, nd, table);
+            else k_near_entries<float, TD_DLP, 8><<<grid, 128, 0, st>>>(m, a, klist, nd, table);
         } else {
-            if (v == 1) k_near_entries<float, TD_ADLP, 4><<<grid, 128, 0, st>>>(m, a, table);
-            else if (v == 2) k_near_entries<float, TD_ADLP, 16><<<grid, 128, 0, st>>>(m, a, table);
-            else k_near_entries<float, TD_ADLP, 8><<<grid, 128, 0, st>>>(m, a, table);
+            if (v == 1) k_near_entries<float, TD_ADLP, 4><<<grid, 128, 0, st>>>(m, a, klist, nd, table);
+            else if (v == 2) k_near_entries<float, TD_ADLP, 16><<<grid, 128, 0, st>>>(m, a, klist, nd, table);
+            else k_near_entries<float, TD_ADLP, 8><<<grid, 128, 0, st>>>(m, a, klist, nd, table);
         }
     }
     return (int)cudaGetLastError();

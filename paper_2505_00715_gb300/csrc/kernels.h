@@ -17,7 +17,9 @@ struct NearArgs {
     const int *blocks;       // [nb][5]
     const int *perm_r, *perm_c;
     int64_t nentries;
-    void *near;
+    void *near;              // near tensor (FP64 form)
+    const c64 *table;        // touching-pair table (mixed form: entries on demand)
+    int64_t *evals;          // [2] regular, tube entries evaluated on demand
 };
 
 // Output arrays of the compressed tensor (fixed slots per block and term).
@@ -70,13 +72,39 @@ int td_launch_entries(cudaStream_t st, const MeshDev &m, int op, int prec, const
                       int64_t nf, void *out);
 // variant: tuning choice of the mixed form's frequencies per pass (0 = default;
 // td_sing_fc / td_near_fc give the values)
+// Both run the nd frequencies klist[0..nd) of the nf of the call; the table
+// holds one value per pair and frequency (three for P1 columns).
 int td_launch_sing_table(cudaStream_t st, const MeshDev &m, int op, int prec, const int *pti, const int *ptj,
-                         int npairs, const double *sig, int nf, c64 *table, int num_sms, int variant = 0);
-int td_launch_near_entries(cudaStream_t st, const MeshDev &m, int op, int prec, const NearArgs &a,
-                           const c64 *table, int num_sms, int variant = 0);
+                         int npairs, const double *rule, const double *sig, int nf, const int *klist, int nd,
+                         c64 *table, int num_sms, int variant = 0);
+int td_launch_near_entries(cudaStream_t st, const MeshDev &m, int op, int prec, const NearArgs &a, const int *klist,
+                           int nd, const c64 *table, int num_sms, int variant = 0);
 int td_sing_fc(int op, int variant);
 int td_near_fc(int variant);
-int td_launch_near_aca(cudaStream_t st, int prec, const NearArgs &a, const TensorOut &o,
+
+// ---- separated frequency sums of the FP64 form (k_sep.cu) ----
+// Frequencies of one call split into those evaluated by separated sums over
+// Chebyshev moments and those evaluated directly (|sigma| D beyond the longest
+// variant, or too few to pay for the moments).
+struct SepSet {
+    int nsep, ndir, P;   // P: terms of the kernel variant
+    int P1;              // terms of the inner of two intervals, before the P of the outer one (0: one)
+    const int *klist;    // device [nsep + ndir]: separated frequencies, then direct ones
+    int *pk;             // device [nsep][2]: terms of each interval a regular frequency keeps
+                         // (touching pairs: all)
+    c64 *coef;           // device: regular pairs [nsep][1 or 2 sets][P1 + P], touching pairs [P1 + P][nsep]
+    double D;            // half length of the distance interval (touching pairs: [0, 2D])
+};
+size_t td_sep_coef_bytes(int op, const SepSet &s, bool touching);
+int td_launch_sep_coef(cudaStream_t st, int op, const double *sig, const SepSet &s, bool touching);
+// reference quadrature points of the touching-pair classes (doubles)
+int64_t td_ss_rule_size(int ng);
+int td_launch_ss_rule(cudaStream_t st, int ng, const double *gx, const double *gw, double *rule);
+int td_launch_near_sep(cudaStream_t st, const MeshDev &m, int op, const NearArgs &a, const SepSet &s, const c64 *table,
+                       int num_sms);
+int td_launch_sing_sep(cudaStream_t st, const MeshDev &m, int op, const int *pti, const int *ptj, int npairs,
+                       const double *rule, const SepSet &s, int nf, c64 *table, int num_sms);
+int td_launch_near_aca(cudaStream_t st, const MeshDev &m, int op, int prec, const NearArgs &a, const TensorOut &o,
                        const AcaParams &p, void *scratch, int64_t scratch_per_cta, int nctas);
 // Dense faces a far-field CTA keeps per block at most, and the largest block
 // that forms C(k) once per term (the scratch of a CTA holds dense_cap entries

@@ -355,42 +355,38 @@ TD_HD int ss_npoints(int cls, int ng) {
     return cls == 3 ? 6 * n2 : cls == 2 ? 6 * n2 * ng : cls == 1 ? 2 * n2 * n2 : 0;
 }
 
-// Quadrature point q of the transformed integral: difference vector d = y - x,
-// weight (including the Jacobian factor g) and trial barycentric weights lam
+// Reference point q of a class's transformed integral: up to four coordinates
+// a (identical: z1, z2, xi; edge: u, p, q; vertex: x1, x2, y1, y2), the weight
+// without the Jacobian factor g, and the trial barycentric weights lam
 // (parametrisation order; use G.loc to map to mesh-local vertices).
-TD_D void ss_point(const SingGeom &G, int q, int ng, const double *gx, const double *gw,
-                   double d[3], double &wgt, double lam[3]) {
-    if (G.cls == 3) {
+TD_D void ss_ref(int cls, int q, int ng, const double *gx, const double *gw, double a[4], double &wgt, double lam[3]) {
+    a[3] = 0.0;
+    if (cls == 3) {
         // six sectors of the z-plane, rays e_a, e_b with |det| = 1
         const double SA[6][2] = {{1, 0}, {1, 1}, {0, 1}, {-1, 0}, {-1, -1}, {0, -1}};
         const double SB[6][2] = {{1, 1}, {0, 1}, {-1, 0}, {-1, -1}, {0, -1}, {1, 0}};
-        int sct = q / (ng * ng), a = (q / ng) % ng, b = q % ng;
-        double xi = gx[a], eta = gx[b];
-        double z1 = SA[sct][0] + eta * (SB[sct][0] - SA[sct][0]);
-        double z2 = SA[sct][1] + eta * (SB[sct][1] - SA[sct][1]);
-        for (int k = 0; k < 3; ++k)
-            d[k] = xi * (z1 * (G.P[1][k] - G.P[0][k]) + z2 * (G.P[2][k] - G.P[1][k]));
-        wgt = gw[a] * gw[b] * xi * (1.0 - xi) * (1.0 - xi) * 0.5 * G.g;
+        int sct = q / (ng * ng), i = (q / ng) % ng, b = q % ng;
+        double xi = gx[i], eta = gx[b];
+        a[0] = SA[sct][0] + eta * (SB[sct][0] - SA[sct][0]);
+        a[1] = SA[sct][1] + eta * (SB[sct][1] - SA[sct][1]);
+        a[2] = xi;
+        wgt = gw[i] * gw[b] * xi * (1.0 - xi) * (1.0 - xi) * 0.5;
         lam[0] = lam[1] = lam[2] = 0.0;  // identical pairs only occur for P0 x P0
-    } else if (G.cls == 2) {
+    } else if (cls == 2) {
         // cone triangles (u, p, q) with vertices on l(u,p,q) = 1
         const double V[6][3][3] = {
             {{0, 1, 0}, {1, 0, 0}, {1, 0, 1}},  {{0, 1, 0}, {1, 0, 1}, {0, 1, 1}},
             {{0, 0, 1}, {1, 0, 1}, {0, 1, 1}},  {{0, 1, 0}, {0, 1, 1}, {-1, 1, 0}},
             {{-1, 0, 0}, {0, 0, 1}, {0, 1, 1}}, {{-1, 0, 0}, {0, 1, 1}, {-1, 1, 0}}};
         int n3 = ng * ng * ng;
-        int tr = q / n3, r = q % n3, a = r / (ng * ng), b = (r / ng) % ng, c = r % ng;
-        double xi = gx[a], e1 = gx[b], e2 = gx[c];
-        double w3[3];
+        int tr = q / n3, r = q % n3, i = r / (ng * ng), b = (r / ng) % ng, c = r % ng;
+        double xi = gx[i], e1 = gx[b], e2 = gx[c];
         for (int k = 0; k < 3; ++k)
-            w3[k] = xi * (V[tr][0][k] + e1 * (V[tr][1][k] - V[tr][0][k]) +
-                          e1 * e2 * (V[tr][2][k] - V[tr][1][k]));
-        double u = w3[0], p = w3[1], qq = w3[2];
-        for (int k = 0; k < 3; ++k)
-            d[k] = u * (G.P[1][k] - G.P[0][k]) + qq * (G.Q[2][k] - G.Q[1][k]) -
-                   p * (G.P[2][k] - G.P[1][k]);
+            a[k] = xi * (V[tr][0][k] + e1 * (V[tr][1][k] - V[tr][0][k]) +
+                         e1 * e2 * (V[tr][2][k] - V[tr][1][k]));
+        double u = a[0], p = a[1], qq = a[2];
         // |det| is 1 for all six cone triangles
-        wgt = gw[a] * gw[b] * gw[c] * xi * xi * e1 * (1.0 - xi) * G.g;
+        wgt = gw[i] * gw[b] * gw[c] * xi * xi * e1 * (1.0 - xi);
         double tlo = p > qq - u ? p : qq - u;
         double thi = u > 0.0 ? 1.0 - u : 1.0;
         double tm = 0.5 * (tlo + thi);
@@ -401,28 +397,62 @@ TD_D void ss_point(const SingGeom &G, int q, int ng, const double *gx, const dou
     } else {
         int n4 = ng * ng * ng * ng;
         int reg = q / n4, r = q % n4;
-        int a = r / (ng * ng * ng), b = (r / (ng * ng)) % ng, c = (r / ng) % ng, e = r % ng;
-        double xi = gx[a], w = gx[b], e1 = gx[c], e2 = gx[e];
-        double x1, x2, y1, y2;
-        if (reg == 0) {
-            x1 = xi;
-            x2 = xi * w;
-            y1 = xi * e1;
-            y2 = xi * e1 * e2;
-        } else {
-            y1 = xi;
-            y2 = xi * w;
-            x1 = xi * e1;
-            x2 = xi * e1 * e2;
-        }
-        for (int k = 0; k < 3; ++k)
-            d[k] = y1 * (G.Q[1][k] - G.Q[0][k]) + y2 * (G.Q[2][k] - G.Q[1][k]) -
-                   x1 * (G.P[1][k] - G.P[0][k]) - x2 * (G.P[2][k] - G.P[1][k]);
-        wgt = gw[a] * gw[b] * gw[c] * gw[e] * xi * xi * xi * e1 * G.g;
-        lam[0] = 1.0 - y1;
-        lam[1] = y1 - y2;
-        lam[2] = y2;
+        int i = r / (ng * ng * ng), b = (r / (ng * ng)) % ng, c = (r / ng) % ng, e = r % ng;
+        double xi = gx[i], w = gx[b], e1 = gx[c], e2 = gx[e];
+        const int lead = reg == 0 ? 0 : 2;  // the triangle that reaches out to xi
+        a[lead] = xi;
+        a[lead + 1] = xi * w;
+        a[2 - lead] = xi * e1;
+        a[3 - lead] = xi * e1 * e2;
+        wgt = gw[i] * gw[b] * gw[c] * gw[e] * xi * xi * xi * e1;
+        lam[0] = 1.0 - a[2];
+        lam[1] = a[2] - a[3];
+        lam[2] = a[3];
     }
+}
+
+// The reference points of the three classes in one array: per class eight rows
+// (a0..a3, weight, lam0..lam2) of ss_npoints values, classes 1, 2, 3 in turn.
+TD_HD int64_t ss_rule_off(int cls, int ng) {
+    return (int64_t)8 * ((cls > 1 ? ss_npoints(1, ng) : 0) + (cls > 2 ? ss_npoints(2, ng) : 0));
+}
+
+// Edge vectors P1 - P0, P2 - P1, Q1 - Q0, Q2 - Q1 of a pair and the difference
+// d = y - x of a reference point.
+struct SsEdges {
+    double p0[3], p1[3], q0[3], q1[3];
+};
+TD_D void ss_edges(const SingGeom &G, SsEdges &E) {
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        E.p0[k] = G.P[1][k] - G.P[0][k];
+        E.p1[k] = G.P[2][k] - G.P[1][k];
+        E.q0[k] = G.Q[1][k] - G.Q[0][k];
+        E.q1[k] = G.Q[2][k] - G.Q[1][k];
+    }
+}
+TD_D void ss_diff(int cls, const double a[4], const SsEdges &E, double d[3]) {
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        if (cls == 3)
+            d[k] = a[2] * (a[0] * E.p0[k] + a[1] * E.p1[k]);
+        else if (cls == 2)
+            d[k] = a[0] * E.p0[k] + a[2] * E.q1[k] - a[1] * E.p1[k];
+        else
+            d[k] = a[2] * E.q0[k] + a[3] * E.q1[k] - a[0] * E.p0[k] - a[1] * E.p1[k];
+    }
+}
+
+// Quadrature point q of the transformed integral: difference vector d = y - x,
+// weight (including the Jacobian factor g) and trial barycentric weights lam.
+TD_D void ss_point(const SingGeom &G, int q, int ng, const double *gx, const double *gw,
+                   double d[3], double &wgt, double lam[3]) {
+    double a[4];
+    SsEdges E;
+    ss_ref(G.cls, q, ng, gx, gw, a, wgt, lam);
+    ss_edges(G, E);
+    ss_diff(G.cls, a, E, d);
+    wgt *= G.g;
 }
 
 // Signed normal factor of the double-layer kernels at difference d = y - x:
