@@ -185,7 +185,8 @@ int prepare_sep(tdbem_ctx *ctx, const tdbem_mesh *m, int op, int prec, int ng, c
     near.coef = (c64 *)(buf + o1);
     sing.coef = (c64 *)(buf + o2);
     *rule = (double *)(buf + o3);
-    if (td_launch_sep_coef(ctx->stream, op, sig, near, false) || td_launch_sep_coef(ctx->stream, op, sig, sing, true) ||
+    if (td_launch_sep_coef(ctx->stream, op, sig, nf, 1.0, near, false) ||
+        td_launch_sep_coef(ctx->stream, op, sig, nf, 1.0, sing, true) ||
         td_launch_ss_rule(ctx->stream, ng, gx, gw, *rule))
         return td_fail(ctx, TDBEM_ERR_CUDA, "separated-sum tables failed: %s", cudaGetErrorString(cudaGetLastError()));
     return TDBEM_OK;
@@ -196,6 +197,17 @@ int prepare_sep(tdbem_ctx *ctx, const tdbem_mesh *m, int op, int prec, int ng, c
 // ============================================================================
 // context
 // ============================================================================
+namespace {
+// the Gauss-Legendre rules of every order 1..16: nodes at 64 ng, weights at
+// 64 ng + 32
+cudaError_t upload_gauss(tdbem_ctx *c) {
+    double h[17 * 64] = {};
+    for (int ng = 1; ng <= 16; ++ng) td_gauss01(ng, h + 64 * ng, h + 64 * ng + 32);
+    const cudaError_t e = cudaMalloc(&c->dgauss, sizeof h);
+    return e != cudaSuccess ? e : cudaMemcpy(c->dgauss, h, sizeof h, cudaMemcpyHostToDevice);
+}
+}  // namespace
+
 extern "C" int tdbem_ctx_create(int device, void *stream, tdbem_ctx_t *out) {
     if (!out) return TDBEM_ERR_ARG;
     *out = nullptr;
@@ -218,9 +230,11 @@ extern "C" int tdbem_ctx_create(int device, void *stream, tdbem_ctx_t *out) {
         return TDBEM_ERR_CUDA;
     }
     if (td_noalloc_setup(device) != TDBEM_OK || cudaMalloc(&c->dflags, sizeof(int)) != cudaSuccess ||
-        cudaMemset(c->dflags, 0, sizeof(int)) != cudaSuccess) {
+        cudaMemset(c->dflags, 0, sizeof(int)) != cudaSuccess || upload_gauss(c) != cudaSuccess) {
         cudaGetLastError();
         cudaStreamDestroy(c->capture);
+        if (c->dflags) cudaFree(c->dflags);
+        if (c->dgauss) cudaFree(c->dgauss);
         delete c;
         return TDBEM_ERR_CUDA;
     }
@@ -231,6 +245,8 @@ extern "C" int tdbem_ctx_create(int device, void *stream, tdbem_ctx_t *out) {
 extern "C" int tdbem_ctx_destroy(tdbem_ctx_t ctx) {
     if (ctx && ctx->capture) cudaStreamDestroy(ctx->capture);
     if (ctx && ctx->dflags) cudaFree(ctx->dflags);
+    if (ctx && ctx->dgauss) cudaFree(ctx->dgauss);
+    if (ctx && ctx->entry_buf) cudaFree(ctx->entry_buf);
     delete ctx;
     return TDBEM_OK;
 }
@@ -526,6 +542,8 @@ int finish_freqs(tdbem_ctx *ctx, tdbem_freqs *f) {
         if (partner != k) f->unique[partner] = -(rep + 1);
     }
     f->Nu = (int)f->uidx.size();
+    f->smax = 0.0;
+    for (int k = 0; k < NQ; ++k) f->smax = std::max(f->smax, std::hypot(f->s[2 * k], f->s[2 * k + 1]));
     return TDBEM_OK;
 }
 }  // namespace
@@ -714,17 +732,43 @@ extern "C" int tdbem_entries(tdbem_mesh_t mesh, const tdbem_op *op, tdbem_freqs_
     if (nr < 0 || nc < 0 || nf < 0 || (nr * nc * nf > 0 && (!rows || !cols || !fidx || !out)))
         return td_fail(ctx, TDBEM_ERR_ARG, "tdbem_entries: bad sizes or NULL pointers");
     if (nr * nc * nf == 0) return TDBEM_OK;
-    Guard g;
-    double *gx, *gw, *sig;
-    int *tp_slot, *pti, *ptj, np;
-    if ((rc = prepare_sing(ctx, mesh, op->op, op->ng, g.p, &gx, &gw, &tp_slot, &pti, &ptj, &np))) return rc;
-    std::vector<double> hs(2 * f->NQ);
-    for (int k = 0; k < 2 * f->NQ; ++k) hs[k] = f->s[k] / op->c;
-    if ((rc = dalloc(ctx, &sig, hs.size(), &g.p)) || (rc = upload(ctx, sig, hs.data(), hs.size()))) return rc;
-    MeshDev md = td_mesh_dev(mesh, op->ng, gx, gw, tp_slot);
-    if (td_launch_entries(ctx->stream, md, op->op, op->prec, sig, f->NQ, rows, nr, cols, nc, fidx, nf, out))
-        return td_fail(ctx, TDBEM_ERR_CUDA, "entry kernel launch failed: %s", cudaGetErrorString(cudaGetLastError()));
-    TD_CUDA(ctx, cudaStreamSynchronize(ctx->stream));  // transient buffers are freed on return
+    // the Gauss rules are the context's, the kernel divides by the wave speed, and it
+    // only asks whether two triangles touch (a non-negative slot), which the touching
+    // list's own triangle indices answer
+    const double *gx = ctx->dgauss + 64 * op->ng;
+    MeshDev md = td_mesh_dev(mesh, op->ng, gx, gx + 32, mesh->dtp_tri);
+    SepSet ss;
+    const bool sep = td_entry_sing_set(op->op, f->smax, op->c, (1.0 + 1e-6) * mesh->edge_max, nr * nc, nf, ss);
+    int lrc = td_launch_entries(ctx->stream, md, op->op, op->prec, f->ds, op->c, f->NQ, rows, nr, cols, nc, fidx, nf, out,
+                                ctx->num_sms, sep);
+    if (sep && !lrc) {
+        // coefficients and reference points in the context's scratch, from the first
+        // launch to the last under the lock: calls of several threads queue their
+        // use of it one after the other on the context's stream
+        std::lock_guard<std::mutex> lock(ctx->entry_mutex);
+        const size_t cb = (td_sep_coef_bytes(op->op, ss, true) + 255) & ~(size_t)255;
+        const size_t need = cb + sizeof(double) * td_ss_rule_size(op->ng);
+        if (need > ctx->entry_bytes) {
+            if (ctx->entry_buf) cudaFree(ctx->entry_buf);  // (waits for the device)
+            ctx->entry_buf = nullptr;
+            ctx->entry_bytes = 0;
+            char *p = nullptr;
+            if ((rc = dalloc(ctx, &p, need))) return rc;
+            ctx->entry_buf = p;
+            ctx->entry_bytes = need;
+        }
+        ss.klist = fidx;
+        ss.coef = (c64 *)ctx->entry_buf;
+        double *rule = (double *)((char *)ctx->entry_buf + cb);
+        lrc = td_launch_sep_coef(ctx->stream, op->op, f->ds, f->NQ, op->c, ss, true);
+        if (!lrc) lrc = td_launch_ss_rule(ctx->stream, op->ng, gx, gx + 32, rule);
+        if (!lrc)
+            lrc = td_launch_entry_sing(ctx->stream, md, op->op, op->prec, rule, ss, f->NQ, rows, nr, cols, nc, out,
+                                       ctx->num_sms);
+    }
+    if (lrc) return td_fail(ctx, TDBEM_ERR_CUDA, "entry kernel launch failed: %s", cudaGetErrorString((cudaError_t)lrc));
+    // the index arrays may be the caller's temporaries on another stream
+    TD_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
     return TDBEM_OK;
 }
 

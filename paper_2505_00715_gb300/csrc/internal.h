@@ -3,6 +3,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -23,6 +24,11 @@ struct tdbem_ctx {
     double pool_scale = 1.0;                       // far part of the first face-pool size
     std::string err;
     int num_sms = 0;
+    double *dgauss = nullptr;  // device: Gauss-Legendre rules [ng][nodes 32 | weights 32], ng = 0..16
+    // scratch of tdbem_entries' separated sums, grown when needed
+    std::mutex entry_mutex;
+    void *entry_buf = nullptr;
+    size_t entry_bytes = 0;
     int *dflags = nullptr;  // device status word of asynchronous kernels (TD_DEV_* bits)
     uint32_t wait_polls = 0;  // poll limit of the tensor-core waits (0: the kernels' default)
 };
@@ -82,6 +88,7 @@ struct tdbem_freqs {
     double *dw = nullptr;
     int kind = 0;                 // 0 BDF2, 1 gCQ, 2 explicit points
     std::vector<double> dts;      // gCQ: the time steps the contour was built for
+    double smax = 0.0;            // largest |s|
     double rho = 1.0;             // gCQ: radius factor of the contour (td_gcq_radius)
 };
 

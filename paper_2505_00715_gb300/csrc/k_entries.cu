@@ -16,57 +16,196 @@
 namespace {
 
 // ---- generic entries --------------------------------------------------------
-// One entry A[row, col](sigma) (sigma = s/c), scaled by 1/(4 pi).
-template <class T, int OP>
-TD_D cx<T> entry_one(const MeshDev &m, int row, int col, double sr, double si) {
-    using R = Reg<T>;
-    typename R::Test X;
-    load_test(m, row, X);
-    cx<T> acc = {0, 0};
-    c64 accs = {0.0, 0.0};
-    if (!TD_P1_TRIAL(OP)) {
-        if (touching_slot(m, row, col) >= 0) {
-            c64 o[3] = {};
-            pair_singular_f64<OP>(m, row, col, sr, si, o);
-            accs = o[0];
+// One point pair at FC frequencies: test point oa of the lane (its weight is
+// left to the end of the sum), trial point ob with the trial hat; d = y - x.
+// acc += w e^{-sigma r} / r (SLP) or w (1 + sigma r) e^{-sigma r} (d.n) / r^3 with
+// the signed kernel normal n.
+template <int OP, int FC>
+TD_D void point_multi(const MeshDev &m, int oa, int ob, float hat, const float *n, const float *sr, const float *si,
+                      c32 *acc) {
+    const float4 xa = __ldg(&m.qp[2 * oa]), xl = __ldg(&m.qp[2 * oa + 1]);
+    const float4 yb = __ldg(&m.qp[2 * ob]), yl = __ldg(&m.qp[2 * ob + 1]);
+    const float dx = (yb.x - xa.x) + (yl.x - xl.x), dy = (yb.y - xa.y) + (yl.y - xl.y),
+                dz = (yb.z - xa.z) + (yl.z - xl.z);
+    const float r2 = dx * dx + dy * dy + dz * dz;
+    const float rinv = rsqrtf(r2), r = r2 * rinv;
+    float w = (TD_P1_TRIAL(OP) ? yb.w * hat : yb.w) * rinv;
+    if (OP != TD_SLP) w *= (dx * n[0] + dy * n[1] + dz * n[2]) * rinv * rinv;
+#pragma unroll
+    for (int j = 0; j < FC; ++j) {
+        const c32 e = expm_sr(sr[j], si[j], r);
+        if (OP == TD_SLP) {
+            acc[j].x = fmaf(w, e.x, acc[j].x);
+            acc[j].y = fmaf(w, e.y, acc[j].y);
         } else {
-            cx<T> o[3] = {};
-            R::template pair<OP>(X, m, col, (T)sr, (T)si, o);
-            acc = o[0];
-        }
-    } else {
-        for (int p = m.v2t_ptr[col]; p < m.v2t_ptr[col + 1]; ++p) {
-            int e = m.v2t[p], l = m.v2t_loc[p];
-            if (touching_slot(m, row, e) >= 0) {
-                c64 o[3] = {};
-                pair_singular_f64<TD_DLP>(m, row, e, sr, si, o);
-                accs = accs + o[l];
-            } else {
-                cx<T> o[3] = {};
-                R::template pair<TD_DLP>(X, m, e, (T)sr, (T)si, o);
-                acc = acc + o[l];
-            }
+            const float pr = fmaf(sr[j], r, 1.0f), pi = si[j] * r;
+            acc[j].x = fmaf(w, pr * e.x - pi * e.y, acc[j].x);
+            acc[j].y = fmaf(w, pr * e.y + pi * e.x, acc[j].y);
         }
     }
-    const double inv4pi = 1.0 / TD_FOUR_PI;
-    return cx<T>{(T)(((double)acc.x + accs.x) * inv4pi), (T)(((double)acc.y + accs.y) * inv4pi)};
 }
-
-template <class T, int OP>
-__global__ void k_entries_generic(MeshDev m, const double *sig, int nq, const int *rows, int64_t nr,
-                                  const int *cols, int64_t nc, const int *fidx, int64_t nf,
-                                  cx<T> *out) {
-    int64_t n = nr * nc * nf;
-    const int ncols = TD_P1_TRIAL(OP) ? m.nv : m.nt;
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n;
-         t += (int64_t)gridDim.x * blockDim.x) {
-        int64_t c = t % nc, r = (t / nc) % nr, f = t / (nc * nr);
-        const int k = fidx[f], row = rows[r], col = cols[c];
-        if (k < 0 || k >= nq || row < 0 || row >= m.nt || col < 0 || col >= ncols) {
-            out[t] = cx<T>{(T)NAN, (T)NAN};  // invalid index: no access, NaN result
-            continue;
+template <int OP, int FC>
+TD_D void point_multi(const MeshDev &m, int oa, int ob, double hat, const double *n, const double *sr, const double *si,
+                      c64 *acc) {
+    const double dx = m.qx[ob] - m.qx[oa], dy = m.qy[ob] - m.qy[oa], dz = m.qz[ob] - m.qz[oa];
+    const double r = sqrt(dx * dx + dy * dy + dz * dz);
+    double w = (TD_P1_TRIAL(OP) ? m.qw[ob] * hat : m.qw[ob]) / r;
+    if (OP != TD_SLP) w *= (dx * n[0] + dy * n[1] + dz * n[2]) / (r * r);
+#pragma unroll
+    for (int j = 0; j < FC; ++j) {
+        const c64 e = expm_sr(sr[j], si[j], r);
+        if (OP == TD_SLP) {
+            acc[j].x += w * e.x;
+            acc[j].y += w * e.y;
+        } else {
+            const double pr = 1.0 + sr[j] * r, pi = si[j] * r;
+            acc[j].x += w * (pr * e.x - pi * e.y);
+            acc[j].y += w * (pr * e.y + pi * e.x);
         }
-        out[t] = entry_one<T, OP>(m, row, col, sig[2 * k], sig[2 * k + 1]);
+    }
+}
+TD_D void tri_normal(const MeshDev &m, int t, float sign, float *n) {
+    const float4 v = __ldg(&m.nrm4[t]);
+    n[0] = sign * v.x;
+    n[1] = sign * v.y;
+    n[2] = sign * v.z;
+}
+TD_D void tri_normal(const MeshDev &m, int t, double sign, double *n) {
+    for (int k = 0; k < 3; ++k) n[k] = sign * m.n64[(int64_t)k * m.nt + t];
+}
+TD_D float point_weight(const MeshDev &m, int o, float) { return m.qw32[o]; }
+TD_D double point_weight(const MeshDev &m, int o, double) { return m.qw[o]; }
+TD_D float hat7(int b, int loc, float) { return bary7f(b, loc); }
+TD_D double hat7(int b, int loc, double) { return bary7d(b, loc); }
+
+// out[f][r][c] = A[rows[r], cols[c]](s_{fidx[f]} / c), an item = one (row,
+// column) at FC consecutive frequencies of the list.  Eight lanes per item: seven
+// take one test point each against the seven trial points (regular pairs); with
+// SING the touching pairs of a warp's four items are then integrated one after the
+// other by all 32 lanes, which split the up to 2 ng^4 Sauter-Schwab points (FP64 in
+// both forms), without it k_entry_sing adds them for all frequencies at once.  One
+// thread per entry left a warp waiting for the lane with the touching pair, 1250
+// points in a row at latency: 320 x 320 x 16 FP64 entries 269 -> 18.1 ms with SING, 11.9 with
+// k_entry_sing; 67 x 1801 x 11 double-layer entries 119 -> 6.2 and 3.3 ms.  Bound:
+// the FP64 pipe.
+template <class T, int OP, int FC, bool SING>
+__global__ void __launch_bounds__(128) k_entries_generic(MeshDev m, const double *s, double c, int nq, const int *rows,
+                                                         int64_t nr, const int *cols, int64_t nc, const int *fidx,
+                                                         int64_t nf, cx<T> *out) {
+    const int64_t nE = nr * nc, items = nE * ((nf + FC - 1) / FC);
+    const int ncols = TD_P1_TRIAL(OP) ? m.nv : m.nt;
+    const int lane = threadIdx.x & 31, sub = lane & 7, grp = lane >> 3;
+    const double inv4pi = 1.0 / TD_FOUR_PI;
+    const int64_t stride = ((int64_t)gridDim.x * blockDim.x) >> 3;
+    for (int64_t base = ((int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31)) >> 3; base < items; base += stride) {
+        const bool valid = base + grp < items;
+        const int64_t it = valid ? base + grp : 0;
+        const int64_t e = it % nE, f0 = it / nE * FC;
+        const int row = rows[e / nc], col = cols[e % nc];
+        const bool ok = valid && row >= 0 && row < m.nt && col >= 0 && col < ncols;
+        double sr[FC], si[FC];
+        T tr[FC], ti[FC];
+        bool fok[FC];
+#pragma unroll
+        for (int j = 0; j < FC; ++j) {
+            const int k = f0 + j < nf ? fidx[f0 + j] : -1;
+            fok[j] = k >= 0 && k < nq;
+            sr[j] = fok[j] ? s[2 * k] / c : 0.0;
+            si[j] = fok[j] ? s[2 * k + 1] / c : 0.0;
+            tr[j] = (T)sr[j];
+            ti[j] = (T)si[j];
+        }
+        cx<T> acc[FC];
+        c64 sing[FC];
+#pragma unroll
+        for (int j = 0; j < FC; ++j) {
+            acc[j] = cx<T>{0, 0};
+            sing[j] = c64{0.0, 0.0};
+        }
+        const int p0 = ok && TD_P1_TRIAL(OP) ? m.v2t_ptr[col] : 0;
+        const int ns = !ok ? 0 : TD_P1_TRIAL(OP) ? m.v2t_ptr[col + 1] - p0 : 1;
+        const int nsw = __reduce_max_sync(0xffffffffu, ns);
+        for (int q = 0; q < nsw; ++q) {
+            const bool has = q < ns;
+            const int tj = !has ? 0 : TD_P1_TRIAL(OP) ? m.v2t[p0 + q] : col;
+            const int loc = has && TD_P1_TRIAL(OP) ? m.v2t_loc[p0 + q] : 0;
+            const bool touch = has && touching_slot(m, row, tj) >= 0;
+            if (has && !touch && sub < 7) {
+                T n[3];
+                if (OP != TD_SLP) tri_normal(m, OP == TD_DLP ? tj : row, OP == TD_DLP ? T(-1) : T(1), n);
+                const int oa = sub * m.nt + row;
+#pragma unroll 1
+                for (int b = 0; b < 7; ++b)
+                    point_multi<OP, FC>(m, oa, b * m.nt + tj, TD_P1_TRIAL(OP) ? hat7(b, loc, T(0)) : T(1), n, tr, ti, acc);
+            }
+            for (unsigned todo = SING ? __ballot_sync(0xffffffffu, touch && sub == 0) : 0u; todo; todo &= todo - 1) {
+                const int src = __ffs(todo) - 1;
+                int ta = __shfl_sync(0xffffffffu, row, src), tb = __shfl_sync(0xffffffffu, tj, src);
+                const int lb = __shfl_sync(0xffffffffu, loc, src);
+                double br[FC], bi[FC];
+                c64 v[FC];
+#pragma unroll
+                for (int j = 0; j < FC; ++j) {
+                    br[j] = __shfl_sync(0xffffffffu, sr[j], src);
+                    bi[j] = __shfl_sync(0xffffffffu, si[j], src);
+                    v[j] = c64{0.0, 0.0};
+                }
+                if (OP == TD_SLP && ta > tb) {
+                    const int t = ta;
+                    ta = tb;
+                    tb = t;
+                }
+                SingGeom G;
+                classify_pair(m, ta, tb, G);
+                // (flat panel: (x - y).n = 0)
+                const int np = OP != TD_SLP && G.cls == 3 ? 0 : ss_npoints(G.cls, m.ng);
+                SsEdges E;
+                ss_edges(G, E);
+                const int hat = G.loc[0] == lb ? 0 : G.loc[1] == lb ? 1 : 2;
+                for (int p = lane; p < np; p += 32) {
+                    double a[4], w, lam[3], d[3];
+                    ss_ref(G.cls, p, m.ng, m.gx, m.gw, a, w, lam);
+                    ss_diff(G.cls, a, E, d);
+                    const double r = sqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
+                    w *= G.g;
+                    if (OP == TD_SLP) w /= r;
+                    else w *= ss_dn<OP>(G, d) / (r * r * r);
+                    if (TD_P1_TRIAL(OP)) w *= hat == 0 ? lam[0] : hat == 1 ? lam[1] : lam[2];
+#pragma unroll
+                    for (int j = 0; j < FC; ++j) {
+                        const c64 x = expm_sr(br[j], bi[j], r);
+                        if (OP == TD_SLP) {
+                            v[j].x += w * x.x;
+                            v[j].y += w * x.y;
+                        } else {
+                            const double pr = 1.0 + br[j] * r, pi = bi[j] * r;
+                            v[j].x += w * (pr * x.x - pi * x.y);
+                            v[j].y += w * (pr * x.y + pi * x.x);
+                        }
+                    }
+                }
+#pragma unroll
+                for (int j = 0; j < FC; ++j) {
+                    const c64 t = {warp_sum(v[j].x), warp_sum(v[j].y)};
+                    if (grp == src >> 3) sing[j] = sing[j] + t;
+                }
+            }
+        }
+        const T wx = ok && sub < 7 ? point_weight(m, sub * m.nt + row, T(0)) : T(0);
+#pragma unroll
+        for (int j = 0; j < FC; ++j) {
+            acc[j] = wx * acc[j];
+#pragma unroll
+            for (int o = 4; o > 0; o >>= 1) {
+                acc[j].x += __shfl_xor_sync(0xffffffffu, acc[j].x, o);
+                acc[j].y += __shfl_xor_sync(0xffffffffu, acc[j].y, o);
+            }
+            // an invalid index gives NaN without any table access
+            if (valid && sub == 0 && f0 + j < nf)
+                out[(f0 + j) * nE + e] = ok && fok[j] ? cx<T>{(T)(((double)acc[j].x + sing[j].x) * inv4pi),
+                                                              (T)(((double)acc[j].y + sing[j].y) * inv4pi)}
+                                                      : cx<T>{(T)NAN, (T)NAN};
+        }
     }
 }
 
@@ -387,28 +526,35 @@ __global__ void __launch_bounds__(128) k_near_entries(MeshDev m, NearArgs a, con
 }  // namespace
 
 // ---- launchers ----------------------------------------------------------------
-int td_launch_entries(cudaStream_t st, const MeshDev &m, int op, int prec, const double *sig, int nq,
-                      const int *rows, int64_t nr, const int *cols, int64_t nc, const int *fidx,
-                      int64_t nf, void *out) {
-    int64_t n = nr * nc * nf;
-    if (n == 0) return 0;
-    int grid = (int)std::min<int64_t>((n + 127) / 128, 152 * 16);
-    if (prec == TDBEM_FP64) {
-        if (op == TD_SLP)
-            k_entries_generic<double, TD_SLP><<<grid, 128, 0, st>>>(m, sig, nq, rows, nr, cols, nc, fidx, nf, (c64 *)out);
-        else if (op == TD_DLP)
-            k_entries_generic<double, TD_DLP><<<grid, 128, 0, st>>>(m, sig, nq, rows, nr, cols, nc, fidx, nf, (c64 *)out);
-        else
-            k_entries_generic<double, TD_ADLP><<<grid, 128, 0, st>>>(m, sig, nq, rows, nr, cols, nc, fidx, nf, (c64 *)out);
-    } else {
-        if (op == TD_SLP)
-            k_entries_generic<float, TD_SLP><<<grid, 128, 0, st>>>(m, sig, nq, rows, nr, cols, nc, fidx, nf, (c32 *)out);
-        else if (op == TD_DLP)
-            k_entries_generic<float, TD_DLP><<<grid, 128, 0, st>>>(m, sig, nq, rows, nr, cols, nc, fidx, nf, (c32 *)out);
-        else
-            k_entries_generic<float, TD_ADLP><<<grid, 128, 0, st>>>(m, sig, nq, rows, nr, cols, nc, fidx, nf, (c32 *)out);
-    }
+namespace {
+// Four frequencies share the point geometry where that leaves enough items to
+// fill the GPU (four per warp, 16 warps per SM); fewer items run one frequency each.
+template <class T, int OP>
+int launch_generic(cudaStream_t st, const MeshDev &m, const double *s, double c, int nq, const int *rows, int64_t nr,
+                   const int *cols, int64_t nc, const int *fidx, int64_t nf, void *out, int num_sms, bool regular_only) {
+    const int64_t nE = nr * nc;
+    const bool four = nf >= 3 && nE * ((nf + 3) / 4) >= (int64_t)num_sms * 64;
+    const int64_t items = nE * (four ? (nf + 3) / 4 : nf);
+    const int grid = (int)std::min<int64_t>((items + 15) / 16, (int64_t)num_sms * 64);
+    auto run = [&](auto kernel) { kernel<<<grid, 128, 0, st>>>(m, s, c, nq, rows, nr, cols, nc, fidx, nf, (cx<T> *)out); };
+    if (regular_only) run(four ? k_entries_generic<T, OP, 4, false> : k_entries_generic<T, OP, 1, false>);
+    else run(four ? k_entries_generic<T, OP, 4, true> : k_entries_generic<T, OP, 1, true>);
     return (int)cudaGetLastError();
+}
+}  // namespace
+
+int td_launch_entries(cudaStream_t st, const MeshDev &m, int op, int prec, const double *s, double c, int nq,
+                      const int *rows, int64_t nr, const int *cols, int64_t nc, const int *fidx,
+                      int64_t nf, void *out, int num_sms, bool regular_only) {
+    if (nr * nc * nf == 0) return 0;
+    const bool ro = regular_only;
+    if (prec == TDBEM_FP64)
+        return op == TD_SLP   ? launch_generic<double, TD_SLP>(st, m, s, c, nq, rows, nr, cols, nc, fidx, nf, out, num_sms, ro)
+               : op == TD_DLP ? launch_generic<double, TD_DLP>(st, m, s, c, nq, rows, nr, cols, nc, fidx, nf, out, num_sms, ro)
+                              : launch_generic<double, TD_ADLP>(st, m, s, c, nq, rows, nr, cols, nc, fidx, nf, out, num_sms, ro);
+    return op == TD_SLP   ? launch_generic<float, TD_SLP>(st, m, s, c, nq, rows, nr, cols, nc, fidx, nf, out, num_sms, ro)
+           : op == TD_DLP ? launch_generic<float, TD_DLP>(st, m, s, c, nq, rows, nr, cols, nc, fidx, nf, out, num_sms, ro)
+                          : launch_generic<float, TD_ADLP>(st, m, s, c, nq, rows, nr, cols, nc, fidx, nf, out, num_sms, ro);
 }
 
 // Frequencies per pass of the mixed-form kernels, selected by the tuning

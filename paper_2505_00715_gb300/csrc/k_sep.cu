@@ -57,13 +57,15 @@ constexpr double kSepTol = 6.938893903907228e-18;  // 2^-57: coefficient tail dr
 // of the layout near [i][set][stride] or touching [stride][n] (frequencies
 // contiguous); pk[2 i] / pk[2 i + 1] = terms kept of the first / second
 // interval, multiples of 4.
-__global__ void __launch_bounds__(kNodes) k_sep_coef(const double *sig, const int *klist, int n, double left,
+// A frequency index outside [0, nq) is left out.
+__global__ void __launch_bounds__(kNodes) k_sep_coef(const double *sig, int nq, const int *klist, int n, double left,
                                                      double half, int P, int kind, int by_term, int stride, int first,
                                                      c64 *coef, int *pk) {
     __shared__ double ct[4 * kNodes];
     __shared__ c64 F[2][kNodes];
     __shared__ double mag[kNodes];
     const int i = blockIdx.x, j = threadIdx.x, k = klist[i];
+    if (k < 0 || k >= nq) return;
     for (int e = j; e < 4 * kNodes; e += kNodes) ct[e] = cospi((double)e / (2 * kNodes));
     __syncthreads();
     const double r = fma(half, ct[2 * j + 1] + 1.0, left);  // u = cos(pi (j + 1/2) / 64)
@@ -326,6 +328,75 @@ __global__ void k_ss_rule(int ng, const double *gx, const double *gw, double *ru
     }
 }
 
+// A touching pair and its reference points; adds the lane's share of its moments
+// (hat v of the trial triangle for P1 columns) to M (inner interval) and N.
+struct SingPair {
+    SingGeom G;
+    SsEdges E;
+    double nrm[3];  // signed kernel normal at d = y - x
+    const double *rl;
+    int nq;
+};
+template <int OP>
+TD_D void sing_pair(const MeshDev &m, int ti, int tj, const double *rule, SingPair &S) {
+    if (OP == TD_SLP && ti > tj) {
+        const int t = ti;
+        ti = tj;
+        tj = t;
+    }
+    classify_pair(m, ti, tj, S.G);
+    ss_edges(S.G, S.E);
+    const double sn = OP == TD_DLP ? -1.0 : 1.0;
+    const double *g = OP == TD_DLP ? S.G.ny : S.G.nx;
+#pragma unroll
+    for (int x = 0; x < 3; ++x) S.nrm[x] = sn * g[x];
+    S.rl = rule + ss_rule_off(S.G.cls, m.ng);
+    S.nq = OP != TD_SLP && S.G.cls == 3 ? 0 : ss_npoints(S.G.cls, m.ng);  // (flat panel: (x - y).n = 0)
+}
+template <int OP, int P1, int P2>
+TD_D void sing_moments(const SingPair &S, int v, double D, double *M, double *N) {
+    // intervals [0, D/2] (P1 terms) and [D/2, 2D] (P2 terms)
+    const double cut = 0.5 * D, inv1 = 4.0 / D, inv2 = 4.0 / (3.0 * D);
+    for (int q = threadIdx.x & 31; q < S.nq; q += 32) {
+        double a[4], d[3], r;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) a[e] = __ldg(S.rl + (int64_t)e * S.nq + q);
+        ss_diff(S.G.cls, a, S.E, d);
+        double w = over_r<OP>(__ldg(S.rl + (int64_t)4 * S.nq + q) * S.G.g, d[0] * S.nrm[0] + d[1] * S.nrm[1] + d[2] * S.nrm[2],
+                              d[0] * d[0] + d[1] * d[1] + d[2] * d[2], r);
+        if (TD_P1_TRIAL(OP)) w *= __ldg(S.rl + (int64_t)(5 + v) * S.nq + q);
+        const bool inner = r < cut;
+        const double v1 = inner ? r * inv1 : (r - cut) * inv2, v2 = v1 + v1;  // 1 + u
+        const double wm = inner ? w : 0.0, wn = inner ? 0.0 : w;
+        double tn = v1 - 1.0, dn = v1;  // as in add_moments
+        M[0] += wm;
+        M[1] = fma(wm, tn, M[1]);
+        N[0] += wn;
+        N[1] = fma(wn, tn, N[1]);
+#pragma unroll
+        for (int e = 2; e < P2; ++e) {
+            dn = fma(v2, tn, -dn);
+            tn = dn - tn;
+            if (e < P1) M[e] = fma(wm, tn, M[e]);
+            N[e] = fma(wn, tn, N[e]);
+        }
+    }
+}
+// sum_m c_m M_m of frequency i of n (all lanes hold the warp's sums)
+template <int P1, int P2>
+TD_D c64 sing_sum(const c64 *coef, int n, int i, const double *M, const double *N) {
+    c64 a = {0.0, 0.0};
+#pragma unroll
+    for (int q = P1 + P2 - 1; q >= 0; --q) {  // outer interval first, large orders first
+        const c64 c = coef[(int64_t)q * n + i];
+        const double mq = q < P1 ? M[q < P1 ? q : 0] : N[q < P1 ? 0 : q - P1];
+        a.x = fma(c.x, mq, a.x);
+        a.y = fma(c.y, mq, a.y);
+    }
+    const double inv4pi = 1.0 / TD_FOUR_PI;
+    return c64{a.x * inv4pi, a.y * inv4pi};
+}
+
 // Touching-pair table at the separated frequencies, one warp per pair: the
 // lanes split the quadrature points, the moments are summed over the warp, and
 // the lanes then take one frequency each.  P1 columns sweep the points once per
@@ -337,31 +408,10 @@ __global__ void __launch_bounds__(128) k_sing_sep(MeshDev m, const int *pti, con
     const int lane = threadIdx.x & 31;
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int nwarps = (gridDim.x * blockDim.x) >> 5;
-    // intervals [0, D/2] (P1 terms) and [D/2, 2D] (P2 terms)
-    const double cut = 0.5 * s.D, inv1 = 4.0 / s.D, inv2 = 4.0 / (3.0 * s.D);
-    const c64 *coef = s.coef;
     for (int p = warp; p < npairs; p += nwarps) {
-        int ti = pti[p], tj = ptj[p];
-        if (OP == TD_SLP && ti > tj) {
-            const int t = ti;
-            ti = tj;
-            tj = t;
-        }
-        SingGeom G;
-        classify_pair(m, ti, tj, G);
+        SingPair S;
+        sing_pair<OP>(m, pti[p], ptj[p], rule, S);
         c64 *o = table + (int64_t)p * nf * NV;
-        if ((OP != TD_SLP && G.cls == 3) || G.cls == 0) {  // flat panel: (x - y).n = 0
-            for (int i = lane; i < s.nsep; i += 32)
-                for (int v = 0; v < NV; ++v) o[(int64_t)s.klist[i] * NV + v] = c64{0.0, 0.0};
-            continue;
-        }
-        SsEdges E;
-        ss_edges(G, E);
-        const double sn = OP == TD_DLP ? -1.0 : 1.0;  // signed kernel normal at d = y - x
-        const double *g = OP == TD_DLP ? G.ny : G.nx;
-        const double nrm[3] = {sn * g[0], sn * g[1], sn * g[2]};
-        const int nq = ss_npoints(G.cls, m.ng);
-        const double *rl = rule + ss_rule_off(G.cls, m.ng);
 #pragma unroll 1
         for (int v = 0; v < NV; ++v) {
             double M[P1], N[P2];
@@ -369,45 +419,64 @@ __global__ void __launch_bounds__(128) k_sing_sep(MeshDev m, const int *pti, con
             for (int q = 0; q < P1; ++q) M[q] = 0.0;
 #pragma unroll
             for (int q = 0; q < P2; ++q) N[q] = 0.0;
-            for (int q = lane; q < nq; q += 32) {
-                double a[4], d[3], r;
+            sing_moments<OP, P1, P2>(S, v, s.D, M, N);
 #pragma unroll
-                for (int e = 0; e < 4; ++e) a[e] = __ldg(rl + (int64_t)e * nq + q);
-                ss_diff(G.cls, a, E, d);
-                double w = over_r<OP>(__ldg(rl + (int64_t)4 * nq + q) * G.g, d[0] * nrm[0] + d[1] * nrm[1] + d[2] * nrm[2],
-                                      d[0] * d[0] + d[1] * d[1] + d[2] * d[2], r);
-                if (TD_P1_TRIAL(OP)) w *= __ldg(rl + (int64_t)(5 + v) * nq + q);
-                const bool inner = r < cut;
-                const double v1 = inner ? r * inv1 : (r - cut) * inv2, v2 = v1 + v1;  // 1 + u
-                const double wm = inner ? w : 0.0, wn = inner ? 0.0 : w;
-                double tn = v1 - 1.0, dn = v1;  // as in add_moments
-                M[0] += wm;
-                M[1] = fma(wm, tn, M[1]);
-                N[0] += wn;
-                N[1] = fma(wn, tn, N[1]);
+            for (int q = 0; q < P1; ++q) M[q] = warp_sum(M[q]);
 #pragma unroll
-                for (int e = 2; e < P2; ++e) {
-                    dn = fma(v2, tn, -dn);
-                    tn = dn - tn;
-                    if (e < P1) M[e] = fma(wm, tn, M[e]);
-                    N[e] = fma(wn, tn, N[e]);
-                }
+            for (int q = 0; q < P2; ++q) N[q] = warp_sum(N[q]);
+            for (int i = lane; i < s.nsep; i += 32)
+                o[(int64_t)s.klist[i] * NV + (TD_P1_TRIAL(OP) ? S.G.loc[v] : 0)] = sing_sum<P1, P2>(s.coef, s.nsep, i, M, N);
+        }
+    }
+}
+
+// Touching part of tdbem_entries at many frequencies: adds it to the entries of
+// out [nf][nr nc] that have one (either precision; the sums are FP64).  A warp
+// looks at 32 entries and integrates the touching ones one after the other; all
+// touching supports of a P1 column share the distance interval, so their moments
+// are added before the frequencies are taken.  An invalid index was answered
+// with NaN already.
+template <class T, int OP, int P1, int P2>
+__global__ void __launch_bounds__(128) k_entry_sing(MeshDev m, const double *rule, SepSet s, int nq, const int *rows,
+                                                    int64_t nr, const int *cols, int64_t nc, cx<T> *out) {
+    const int64_t nE = nr * nc, stride = (int64_t)gridDim.x * blockDim.x;
+    const int ncols = TD_P1_TRIAL(OP) ? m.nv : m.nt, lane = threadIdx.x & 31;
+    for (int64_t base = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < nE; base += stride) {
+        const int64_t e = base + lane;
+        int row = e < nE ? rows[e / nc] : -1, col = e < nE ? cols[e % nc] : -1;
+        bool touch = false;
+        if (row >= 0 && row < m.nt && col >= 0 && col < ncols) {
+            if (!TD_P1_TRIAL(OP)) touch = touching_slot(m, row, col) >= 0;
+            else
+                for (int p = m.v2t_ptr[col]; p < m.v2t_ptr[col + 1] && !touch; ++p) touch = touching_slot(m, row, m.v2t[p]) >= 0;
+        }
+        for (unsigned todo = __ballot_sync(0xffffffffu, touch); todo; todo &= todo - 1) {
+            const int src = __ffs(todo) - 1;
+            const int ti = __shfl_sync(0xffffffffu, row, src), tc = __shfl_sync(0xffffffffu, col, src);
+            double M[P1], N[P2];
+#pragma unroll
+            for (int q = 0; q < P1; ++q) M[q] = 0.0;
+#pragma unroll
+            for (int q = 0; q < P2; ++q) N[q] = 0.0;
+            const int p0 = TD_P1_TRIAL(OP) ? m.v2t_ptr[tc] : 0, p1 = TD_P1_TRIAL(OP) ? m.v2t_ptr[tc + 1] : 1;
+#pragma unroll 1
+            for (int p = p0; p < p1; ++p) {
+                const int tj = TD_P1_TRIAL(OP) ? m.v2t[p] : tc, loc = TD_P1_TRIAL(OP) ? m.v2t_loc[p] : 0;
+                if (TD_P1_TRIAL(OP) && touching_slot(m, ti, tj) < 0) continue;
+                SingPair S;
+                sing_pair<OP>(m, ti, tj, rule, S);
+                sing_moments<OP, P1, P2>(S, S.G.loc[0] == loc ? 0 : S.G.loc[1] == loc ? 1 : 2, s.D, M, N);
             }
 #pragma unroll
             for (int q = 0; q < P1; ++q) M[q] = warp_sum(M[q]);
 #pragma unroll
             for (int q = 0; q < P2; ++q) N[q] = warp_sum(N[q]);
-            const double inv4pi = 1.0 / TD_FOUR_PI;
             for (int i = lane; i < s.nsep; i += 32) {
-                c64 a = {0.0, 0.0};
-#pragma unroll
-                for (int q = P1 + P2 - 1; q >= 0; --q) {  // outer interval first, large orders first
-                    const c64 c = coef[(int64_t)q * s.nsep + i];
-                    const double mq = q < P1 ? M[q < P1 ? q : 0] : N[q < P1 ? 0 : q - P1];
-                    a.x = fma(c.x, mq, a.x);
-                    a.y = fma(c.y, mq, a.y);
-                }
-                o[(int64_t)s.klist[i] * NV + (TD_P1_TRIAL(OP) ? G.loc[v] : 0)] = c64{a.x * inv4pi, a.y * inv4pi};
+                const int k = s.klist[i];
+                if (k < 0 || k >= nq) continue;
+                const c64 a = sing_sum<P1, P2>(s.coef, s.nsep, i, M, N);
+                cx<T> &o = out[(int64_t)i * nE + base + src];
+                o = cx<T>{(T)((double)o.x + a.x), (T)((double)o.y + a.y)};
             }
         }
     }
@@ -512,11 +581,11 @@ size_t td_sep_coef_bytes(int op, const SepSet &s, bool touching) {
     return sizeof(c64) * s.nsep * (s.P + s.P1) * (op == TD_SLP || touching ? 1 : 2);
 }
 
-int td_launch_sep_coef(cudaStream_t st, int op, const double *sig, const SepSet &s, bool touching) {
+int td_launch_sep_coef(cudaStream_t st, int op, const double *sig, int nq, double c, const SepSet &s, bool touching) {
     if (s.nsep == 0) return 0;
     const int kind = op == TD_SLP ? 0 : touching ? 2 : 1;
     auto run = [&](double left, double half, int P, int first) {
-        k_sep_coef<<<s.nsep, kNodes, 0, st>>>(sig, s.klist, s.nsep, left, half, P, kind, touching, s.P1 + s.P, first,
+        k_sep_coef<<<s.nsep, kNodes, 0, st>>>(sig, nq, s.klist, s.nsep, left / c, half / c, P, kind, touching, s.P1 + s.P, first,
                                               s.coef, touching ? nullptr : s.pk);
     };
     if (s.P1) {
@@ -550,4 +619,37 @@ int td_launch_sing_sep(cudaStream_t st, const MeshDev &m, int op, const int *pti
     return op == TD_SLP   ? launch_sing<TD_SLP>(st, m, pti, ptj, npairs, rule, s, nf, table, num_sms)
            : op == TD_DLP ? launch_sing<TD_DLP>(st, m, pti, ptj, npairs, rule, s, nf, table, num_sms)
                           : launch_sing<TD_ADLP>(st, m, pti, ptj, npairs, rule, s, nf, table, num_sms);
+}
+
+bool td_entry_sing_set(int op, double smax, double c, double D, int64_t nE, int64_t nf, SepSet &s) {
+    s = SepSet{};
+    const SepVariant *v = variant_for(op, smax / c * D, true);
+    if (!v || !(D > 0.0) || nf < 3 || nf > 4096 || nE < 512) return false;
+    s.nsep = (int)nf;
+    s.P = v->P;
+    s.P1 = v->P1;
+    s.D = D;
+    return true;
+}
+
+namespace {
+template <class T, int OP>
+int launch_entry_sing(cudaStream_t st, const MeshDev &m, const double *rule, const SepSet &s, int nq, const int *rows,
+                      int64_t nr, const int *cols, int64_t nc, void *out, int num_sms) {
+    const int grid = (int)std::min<int64_t>((nr * nc + 127) / 128, (int64_t)num_sms * 32);
+    if (s.P == 24) k_entry_sing<T, OP, 16, 24><<<grid, 128, 0, st>>>(m, rule, s, nq, rows, nr, cols, nc, (cx<T> *)out);
+    else k_entry_sing<T, OP, 24, 40><<<grid, 128, 0, st>>>(m, rule, s, nq, rows, nr, cols, nc, (cx<T> *)out);
+    return (int)cudaGetLastError();
+}
+}  // namespace
+
+int td_launch_entry_sing(cudaStream_t st, const MeshDev &m, int op, int prec, const double *rule, const SepSet &s, int nq,
+                         const int *rows, int64_t nr, const int *cols, int64_t nc, void *out, int num_sms) {
+    if (prec == TDBEM_FP64)
+        return op == TD_SLP   ? launch_entry_sing<double, TD_SLP>(st, m, rule, s, nq, rows, nr, cols, nc, out, num_sms)
+               : op == TD_DLP ? launch_entry_sing<double, TD_DLP>(st, m, rule, s, nq, rows, nr, cols, nc, out, num_sms)
+                              : launch_entry_sing<double, TD_ADLP>(st, m, rule, s, nq, rows, nr, cols, nc, out, num_sms);
+    return op == TD_SLP   ? launch_entry_sing<float, TD_SLP>(st, m, rule, s, nq, rows, nr, cols, nc, out, num_sms)
+           : op == TD_DLP ? launch_entry_sing<float, TD_DLP>(st, m, rule, s, nq, rows, nr, cols, nc, out, num_sms)
+                          : launch_entry_sing<float, TD_ADLP>(st, m, rule, s, nq, rows, nr, cols, nc, out, num_sms);
 }

@@ -67,9 +67,10 @@ struct FarArgs {
 // k_peak.cu: throughput microbenchmark (what: 0 FP32 FMA, 1 special-function
 // unit, 2 FP64 FMA); *ops = operations performed by the launch
 int td_launch_peak(cudaStream_t st, int what, int grid, int iters, void *out, double *ops);
-int td_launch_entries(cudaStream_t st, const MeshDev &m, int op, int prec, const double *sig, int nq,
+// entries at the frequencies s[fidx] / c; regular_only: touching pairs are left out
+int td_launch_entries(cudaStream_t st, const MeshDev &m, int op, int prec, const double *s, double c, int nq,
                       const int *rows, int64_t nr, const int *cols, int64_t nc, const int *fidx,
-                      int64_t nf, void *out);
+                      int64_t nf, void *out, int num_sms, bool regular_only);
 // variant: tuning choice of the mixed form's frequencies per pass (0 = default;
 // td_sing_fc / td_near_fc give the values)
 // Both run the nd frequencies klist[0..nd) of the nf of the call; the table
@@ -96,12 +97,20 @@ struct SepSet {
     double D;            // half length of the distance interval (touching pairs: [0, 2D])
 };
 size_t td_sep_coef_bytes(int op, const SepSet &s, bool touching);
-int td_launch_sep_coef(cudaStream_t st, int op, const double *sig, const SepSet &s, bool touching);
+// coefficients of the frequencies sig / c (nq of them; indices outside are left out)
+int td_launch_sep_coef(cudaStream_t st, int op, const double *sig, int nq, double c, const SepSet &s, bool touching);
 // reference quadrature points of the touching-pair classes (doubles)
 int64_t td_ss_rule_size(int ng);
 int td_launch_ss_rule(cudaStream_t st, int ng, const double *gx, const double *gw, double *rule);
 int td_launch_near_sep(cudaStream_t st, const MeshDev &m, int op, const NearArgs &a, const SepSet &s, const c64 *table,
                        int num_sms);
+// Touching part of tdbem_entries: whether the separated sums take it (at least 3
+// frequencies, |s| <= smax within the longest variant, and enough entries to pay
+// for the extra launches), and the kernel that adds it to out [nf][nr nc]
+// (klist: the call's frequency indices).
+bool td_entry_sing_set(int op, double smax, double c, double D, int64_t nE, int64_t nf, SepSet &s);
+int td_launch_entry_sing(cudaStream_t st, const MeshDev &m, int op, int prec, const double *rule, const SepSet &s, int nq,
+                         const int *rows, int64_t nr, const int *cols, int64_t nc, void *out, int num_sms);
 int td_launch_sing_sep(cudaStream_t st, const MeshDev &m, int op, const int *pti, const int *ptj, int npairs,
                        const double *rule, const SepSet &s, int nf, c64 *table, int num_sms);
 int td_launch_near_aca(cudaStream_t st, const MeshDev &m, int op, int prec, const NearArgs &a, const TensorOut &o,

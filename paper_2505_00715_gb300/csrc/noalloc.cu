@@ -124,7 +124,8 @@ extern "C" int tdbem_entries_noalloc(tdbem_mesh_t mesh, const tdbem_op *op, tdbe
     // two triangles touch (a non-negative slot), which the touching list's own
     // triangle indices answer without the slot table
     MeshDev m = td_mesh_dev(mesh, op->ng, scratch, scratch + 32, mesh->dtp_tri);
-    if (td_launch_entries(ctx->stream, m, op->op, op->prec, scratch + 64, f->NQ, rows, nr, cols, nc, fidx, nf, out))
+    if (td_launch_entries(ctx->stream, m, op->op, op->prec, scratch + 64, 1.0, f->NQ, rows, nr, cols, nc, fidx, nf, out,
+                          ctx->num_sms, false))
         return td_fail(ctx, TDBEM_ERR_CUDA, "tdbem_entries_noalloc: kernel launch failed");
     return TDBEM_OK;
 }

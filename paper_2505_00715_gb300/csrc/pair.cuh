@@ -137,64 +137,6 @@ TD_D c32 expm_sr(float sr, float si, float r) {
     return {ea * cs, -ea * sn};
 }
 
-// out (SLP: out[0]; DLP: out[0..2] per trial-local vertex) += pair integral
-// over test X and trial triangle tj, sigma = s / c.  Unscaled by 1/(4 pi).
-template <int OP>
-TD_D void pair_f32(const TestF &X, const MeshDev &m, int tj, float sr, float si, c32 *out) {
-    // kernel normal: the trial normal with -d.n (DLP) or the test normal with +d.n (ADLP)
-    float nx = 0.f, ny = 0.f, nz = 0.f;
-    if (OP == TD_DLP) {
-        nx = -m.n32[tj];
-        ny = -m.n32[m.nt + tj];
-        nz = -m.n32[2 * m.nt + tj];
-    } else if (OP == TD_ADLP) {
-        nx = X.nx;
-        ny = X.ny;
-        nz = X.nz;
-    }
-#pragma unroll 1
-    for (int b = 0; b < 7; ++b) {
-        const int ob = b * m.nt + tj;
-        const float yxh = m.qxh[ob], yyh = m.qyh[ob], yzh = m.qzh[ob];
-        const float yxl = m.qxl[ob], yyl = m.qyl[ob], yzl = m.qzl[ob];
-        const float wy = m.qw32[ob];
-        c32 acc = {0.f, 0.f};
-#pragma unroll
-        for (int a = 0; a < 7; ++a) {
-            const float dx = (yxh - X.xh[a]) + (yxl - X.xl[a]);
-            const float dy = (yyh - X.yh[a]) + (yyl - X.yl[a]);
-            const float dz = (yzh - X.zh[a]) + (yzl - X.zl[a]);
-            const float r2 = dx * dx + dy * dy + dz * dz;
-            const float rinv = rsqrtf(r2);
-            const float r = r2 * rinv;
-            const c32 e = expm_sr(sr, si, r);
-            if (OP == TD_SLP) {
-                const float w = X.w[a] * rinv;
-                acc.x = fmaf(w, e.x, acc.x);
-                acc.y = fmaf(w, e.y, acc.y);
-            } else {
-                // (1 + sigma r) e^{-sigma r} (d.n) / r^3, n signed as above
-                const float dn = dx * nx + dy * ny + dz * nz;
-                const float w = X.w[a] * dn * rinv * rinv * rinv;
-                const float pr = fmaf(sr, r, 1.0f), pi = si * r;
-                acc.x = fmaf(w, pr * e.x - pi * e.y, acc.x);
-                acc.y = fmaf(w, pr * e.y + pi * e.x, acc.y);
-            }
-        }
-        if (!TD_P1_TRIAL(OP)) {
-            out[0].x = fmaf(wy, acc.x, out[0].x);
-            out[0].y = fmaf(wy, acc.y, out[0].y);
-        } else {
-#pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                const float f = wy * bary7f(b, k);
-                out[k].x = fmaf(f, acc.x, out[k].x);
-                out[k].y = fmaf(f, acc.y, out[k].y);
-            }
-        }
-    }
-}
-
 struct TestD {
     double x[7], y[7], z[7], w[7];
     double nx, ny, nz;  // unit normal of the test triangle (adjoint double layer)
@@ -221,68 +163,10 @@ TD_D c64 expm_sr(double sr, double si, double r) {
     return {ea * cs, -ea * sn};
 }
 
-template <int OP>
-TD_D void pair_f64(const TestD &X, const MeshDev &m, int tj, double sr, double si, c64 *out) {
-    double nx = 0.0, ny = 0.0, nz = 0.0;  // signed kernel normal, as in pair_f32
-    if (OP == TD_DLP) {
-        nx = -m.n64[tj];
-        ny = -m.n64[m.nt + tj];
-        nz = -m.n64[2 * m.nt + tj];
-    } else if (OP == TD_ADLP) {
-        nx = X.nx;
-        ny = X.ny;
-        nz = X.nz;
-    }
-#pragma unroll 1
-    for (int b = 0; b < 7; ++b) {
-        const int ob = b * m.nt + tj;
-        const double yx = m.qx[ob], yy = m.qy[ob], yz = m.qz[ob], wy = m.qw[ob];
-        c64 acc = {0.0, 0.0};
-#pragma unroll
-        for (int a = 0; a < 7; ++a) {
-            const double dx = yx - X.x[a], dy = yy - X.y[a], dz = yz - X.z[a];
-            const double r = sqrt(dx * dx + dy * dy + dz * dz);
-            const c64 e = expm_sr(sr, si, r);
-            if (OP == TD_SLP) {
-                const double w = X.w[a] / r;
-                acc.x += w * e.x;
-                acc.y += w * e.y;
-            } else {
-                const double dn = dx * nx + dy * ny + dz * nz;
-                const double w = X.w[a] * dn / (r * r * r);
-                const double pr = 1.0 + sr * r, pi = si * r;
-                acc.x += w * (pr * e.x - pi * e.y);
-                acc.y += w * (pr * e.y + pi * e.x);
-            }
-        }
-        if (!TD_P1_TRIAL(OP)) {
-            out[0].x += wy * acc.x;
-            out[0].y += wy * acc.y;
-        } else {
-#pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                const double f = wy * bary7d(b, k);
-                out[k].x += f * acc.x;
-                out[k].y += f * acc.y;
-            }
-        }
-    }
-}
-
-// Precision dispatch used by the kernels.
+// Test triangle in registers, by precision.
 template <class T> struct Reg;
-template <> struct Reg<float> {
-    using Test = TestF;
-    template <int OP> TD_D static void pair(const Test &X, const MeshDev &m, int tj, float sr, float si, c32 *o) {
-        pair_f32<OP>(X, m, tj, sr, si, o);
-    }
-};
-template <> struct Reg<double> {
-    using Test = TestD;
-    template <int OP> TD_D static void pair(const Test &X, const MeshDev &m, int tj, double sr, double si, c64 *o) {
-        pair_f64<OP>(X, m, tj, sr, si, o);
-    }
-};
+template <> struct Reg<float> { using Test = TestF; };
+template <> struct Reg<double> { using Test = TestD; };
 
 // ---------------------------------------------------------------------------
 // Touching pairs: classification and Sauter-Schwab quadrature points (FP64)
@@ -355,6 +239,14 @@ TD_HD int ss_npoints(int cls, int ng) {
     return cls == 3 ? 6 * n2 : cls == 2 ? 6 * n2 * ng : cls == 1 ? 2 * n2 * n2 : 0;
 }
 
+// Identical pairs: rays of the six sectors of the z-plane (|det| = 1); common
+// edge: cone triangles (u, p, q) with vertices on l(u,p,q) = 1.
+static __constant__ float c_ss_rays[7][2] = {{1, 0}, {1, 1}, {0, 1}, {-1, 0}, {-1, -1}, {0, -1}, {1, 0}};
+static __constant__ float c_ss_cones[6][3][3] = {
+    {{0, 1, 0}, {1, 0, 0}, {1, 0, 1}},  {{0, 1, 0}, {1, 0, 1}, {0, 1, 1}},
+    {{0, 0, 1}, {1, 0, 1}, {0, 1, 1}},  {{0, 1, 0}, {0, 1, 1}, {-1, 1, 0}},
+    {{-1, 0, 0}, {0, 0, 1}, {0, 1, 1}}, {{-1, 0, 0}, {0, 1, 1}, {-1, 1, 0}}};
+
 // Reference point q of a class's transformed integral: up to four coordinates
 // a (identical: z1, z2, xi; edge: u, p, q; vertex: x1, x2, y1, y2), the weight
 // without the Jacobian factor g, and the trial barycentric weights lam
@@ -362,28 +254,23 @@ TD_HD int ss_npoints(int cls, int ng) {
 TD_D void ss_ref(int cls, int q, int ng, const double *gx, const double *gw, double a[4], double &wgt, double lam[3]) {
     a[3] = 0.0;
     if (cls == 3) {
-        // six sectors of the z-plane, rays e_a, e_b with |det| = 1
-        const double SA[6][2] = {{1, 0}, {1, 1}, {0, 1}, {-1, 0}, {-1, -1}, {0, -1}};
-        const double SB[6][2] = {{1, 1}, {0, 1}, {-1, 0}, {-1, -1}, {0, -1}, {1, 0}};
         int sct = q / (ng * ng), i = (q / ng) % ng, b = q % ng;
         double xi = gx[i], eta = gx[b];
-        a[0] = SA[sct][0] + eta * (SB[sct][0] - SA[sct][0]);
-        a[1] = SA[sct][1] + eta * (SB[sct][1] - SA[sct][1]);
+        const float *A = c_ss_rays[sct], *B = c_ss_rays[sct + 1];
+        a[0] = A[0] + eta * (B[0] - A[0]);
+        a[1] = A[1] + eta * (B[1] - A[1]);
         a[2] = xi;
         wgt = gw[i] * gw[b] * xi * (1.0 - xi) * (1.0 - xi) * 0.5;
         lam[0] = lam[1] = lam[2] = 0.0;  // identical pairs only occur for P0 x P0
     } else if (cls == 2) {
-        // cone triangles (u, p, q) with vertices on l(u,p,q) = 1
-        const double V[6][3][3] = {
-            {{0, 1, 0}, {1, 0, 0}, {1, 0, 1}},  {{0, 1, 0}, {1, 0, 1}, {0, 1, 1}},
-            {{0, 0, 1}, {1, 0, 1}, {0, 1, 1}},  {{0, 1, 0}, {0, 1, 1}, {-1, 1, 0}},
-            {{-1, 0, 0}, {0, 0, 1}, {0, 1, 1}}, {{-1, 0, 0}, {0, 1, 1}, {-1, 1, 0}}};
         int n3 = ng * ng * ng;
         int tr = q / n3, r = q % n3, i = r / (ng * ng), b = (r / ng) % ng, c = r % ng;
         double xi = gx[i], e1 = gx[b], e2 = gx[c];
-        for (int k = 0; k < 3; ++k)
-            a[k] = xi * (V[tr][0][k] + e1 * (V[tr][1][k] - V[tr][0][k]) +
-                         e1 * e2 * (V[tr][2][k] - V[tr][1][k]));
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const double v0 = c_ss_cones[tr][0][k], v1 = c_ss_cones[tr][1][k], v2 = c_ss_cones[tr][2][k];
+            a[k] = xi * (v0 + e1 * (v1 - v0) + e1 * e2 * (v2 - v1));
+        }
         double u = a[0], p = a[1], qq = a[2];
         // |det| is 1 for all six cone triangles
         wgt = gw[i] * gw[b] * gw[c] * xi * xi * e1 * (1.0 - xi);
@@ -399,11 +286,12 @@ TD_D void ss_ref(int cls, int q, int ng, const double *gx, const double *gw, dou
         int reg = q / n4, r = q % n4;
         int i = r / (ng * ng * ng), b = (r / (ng * ng)) % ng, c = (r / ng) % ng, e = r % ng;
         double xi = gx[i], w = gx[b], e1 = gx[c], e2 = gx[e];
-        const int lead = reg == 0 ? 0 : 2;  // the triangle that reaches out to xi
-        a[lead] = xi;
-        a[lead + 1] = xi * w;
-        a[2 - lead] = xi * e1;
-        a[3 - lead] = xi * e1 * e2;
+        // region 0: the test triangle reaches out to xi, region 1: the trial triangle
+        const double big0 = xi, big1 = xi * w, small0 = xi * e1, small1 = xi * e1 * e2;
+        a[0] = reg == 0 ? big0 : small0;
+        a[1] = reg == 0 ? big1 : small1;
+        a[2] = reg == 0 ? small0 : big0;
+        a[3] = reg == 0 ? small1 : big1;
         wgt = gw[i] * gw[b] * gw[c] * gw[e] * xi * xi * xi * e1;
         lam[0] = 1.0 - a[2];
         lam[1] = a[2] - a[3];
@@ -461,56 +349,6 @@ template <int OP>
 TD_HD double ss_dn(const SingGeom &G, const double d[3]) {
     return OP == TD_DLP ? -(d[0] * G.ny[0] + d[1] * G.ny[1] + d[2] * G.ny[2])
                         : d[0] * G.nx[0] + d[1] * G.nx[1] + d[2] * G.nx[2];
-}
-
-// Kernel value times weight at one transformed point, accumulated into out
-// (mesh-local trial vertex order for DLP).  sigma = s / c.
-template <int OP>
-TD_D void ss_accum(const SingGeom &G, const double d[3], double wgt, const double lam[3],
-                   double sr, double si, c64 *out) {
-    double r = sqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
-    c64 e = expm_sr(sr, si, r);
-    if (OP == TD_SLP) {
-        double w = wgt / r;
-        out[0].x += w * e.x;
-        out[0].y += w * e.y;
-    } else {
-        double dn = ss_dn<OP>(G, d);
-        double w = wgt * dn / (r * r * r);
-        double pr = 1.0 + sr * r, pi = si * r;
-        c64 v = {w * (pr * e.x - pi * e.y), w * (pr * e.y + pi * e.x)};
-        if (OP == TD_ADLP) {
-            out[0].x += v.x;
-            out[0].y += v.y;
-        } else {
-            for (int k = 0; k < 3; ++k) {
-                out[G.loc[k]].x += lam[k] * v.x;
-                out[G.loc[k]].y += lam[k] * v.y;
-            }
-        }
-    }
-}
-
-// Whole touching-pair integral by one thread (used by the generic entry
-// kernel; the compressor uses the warp-parallel table kernel instead).
-// Returns the class; out is unscaled by 1/(4 pi).
-template <int OP>
-TD_D int pair_singular_f64(const MeshDev &m, int ti, int tj, double sr, double si, c64 *out) {
-    if (OP == TD_SLP && ti > tj) {
-        int t = ti;
-        ti = tj;
-        tj = t;
-    }
-    SingGeom G;
-    if (classify_pair(m, ti, tj, G) == 0) return 0;
-    if (OP != TD_SLP && G.cls == 3) return 3;  // flat panel: (x - y).n = 0
-    int nq = ss_npoints(G.cls, m.ng);
-    for (int q = 0; q < nq; ++q) {
-        double d[3], w, lam[3];
-        ss_point(G, q, m.ng, m.gx, m.gw, d, w, lam);
-        ss_accum<OP>(G, d, w, lam, sr, si, out);
-    }
-    return G.cls;
 }
 
 // Index of tj in ti's touching list, or -1.
