@@ -4,9 +4,9 @@
 // Parameter layout (FP32 master copy, same order for gradients):
 //   W1[64][6] b1[64] W2[64][64] b2[64] W3[16][64] b3[16]
 // Inference uses a BF16 copy of the weights with FP32 accumulation; training
-// runs forward and backward in FP32 from the master copy.  One thread per
-// sample; weights live in shared memory; gradients are reduced per CTA in
-// shared memory and then added to the global gradient.
+// runs forward and backward in FP32 from the master copy.  Weights live in
+// shared memory; inference takes one thread per sample, training tiles of 32
+// samples per CTA.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -24,10 +24,6 @@ constexpr int OW1 = 0, OB1 = OW1 + NH * NIN, OW2 = OB1 + NH, OB2 = OW2 + NH * NH
 static_assert(NP == TD_MLP_NPARAMS, "parameter count");
 
 TD_D float gelu(float x) { return 0.5f * x * (1.0f + erff(x * 0.70710678118654752f)); }
-TD_D float gelu_d(float x) {
-    return 0.5f * (1.0f + erff(x * 0.70710678118654752f)) + x * 0.39894228040143268f * expf(-0.5f * x * x);
-}
-
 __global__ void k_to_bf16(const float *p, __nv_bfloat16 *q, int n) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n) q[i] = __float2bfloat16(p[i]);
@@ -125,101 +121,212 @@ __global__ void __launch_bounds__(128) k_mlp_predict(const __nv_bfloat16 *P, con
 }
 
 // Mean softmax cross-entropy and its gradient (FP32).  grad and loss must be
-// zeroed by the caller; every CTA adds its partial sums.  Per-sample
-// contributions are summed over the warp with shuffles before one shared
-// atomic per warp, then once per CTA into global memory.
-TD_D float wsum(float v) {
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
+// zeroed by the caller; every CTA adds its sums once at the end.
+//
+// A CTA takes tiles of 32 samples through both passes with the weights and the
+// tile's activations in shared memory ([feature][sample], rows of kGS).  The
+// layers put one sample on each lane and eight outputs in registers: the weights
+// are broadcasts, W2 kept in both orders so that the eight weights of a step
+// are contiguous.  The weight gradients are outer products over the 32 samples,
+// 4 x 4 outputs per thread (W2), kept in registers over the CTA's tiles.  One
+// thread per sample with a warp sum per weight took 5648 x 5 shuffles a warp:
+// 4096 samples 989 -> 14 us.  Bound at that size: latency, one tile per SM.
+constexpr int kGT = 256, kGS = 36;
+struct GradSmem {
+    float w2[NH * NH], w2t[NH * NH], w3[NOUT * NH], w3t[NH * NOUT], w1[NH * NIN], b1[NH], b2[NH], b3[NOUT];
+    float in[NIN][kGS], h1[NH][kGS], g1[NH][kGS], h2[NH][kGS], g2[NH][kGS], d3[NOUT][kGS];
+};
+
+// GELU and its derivative
+TD_D void gelu_both(float x, float &h, float &g) {
+    const float c = 0.5f * (1.0f + erff(x * 0.70710678118654752f));
+    h = x * c;
+    g = c + x * 0.39894228040143268f * expf(-0.5f * x * x);
 }
 
-__global__ void __launch_bounds__(128) k_mlp_grad(const float *P, const float *x, const int *label, int64_t n,
+// a[q] += sum_k x[k][lane] w[k ld + q], q < 8 (w 16-byte aligned)
+template <int K>
+TD_D void layer8(const float (*x)[kGS], const float *w, int ld, int lane, float *a) {
+#pragma unroll 4
+    for (int k = 0; k < K; ++k) {
+        const float v = x[k][lane];
+        const float4 p = *reinterpret_cast<const float4 *>(w + k * ld), q = *reinterpret_cast<const float4 *>(w + k * ld + 4);
+        a[0] = fmaf(p.x, v, a[0]);
+        a[1] = fmaf(p.y, v, a[1]);
+        a[2] = fmaf(p.z, v, a[2]);
+        a[3] = fmaf(p.w, v, a[3]);
+        a[4] = fmaf(q.x, v, a[4]);
+        a[5] = fmaf(q.y, v, a[5]);
+        a[6] = fmaf(q.z, v, a[6]);
+        a[7] = fmaf(q.w, v, a[7]);
+    }
+}
+// sum over the 32 samples of two rows
+TD_D float row_dot(const float *x, const float *y, float a) {
+    float4 t = {0.0f, 0.0f, 0.0f, 0.0f};  // four chains: half the rounding of one
+#pragma unroll
+    for (int s = 0; s < 32; s += 4) {
+        const float4 p = *reinterpret_cast<const float4 *>(x + s), q = *reinterpret_cast<const float4 *>(y + s);
+        t = float4{fmaf(p.x, q.x, t.x), fmaf(p.y, q.y, t.y), fmaf(p.z, q.z, t.z), fmaf(p.w, q.w, t.w)};
+    }
+    return a + ((t.x + t.y) + (t.z + t.w));
+}
+TD_D float row_sum(const float *x, float a) {
+#pragma unroll
+    for (int s = 0; s < 32; s += 4) {
+        const float4 p = *reinterpret_cast<const float4 *>(x + s);
+        a += (p.x + p.y) + (p.z + p.w);
+    }
+    return a;
+}
+
+__global__ void __launch_bounds__(kGT) k_mlp_grad(const float *P, const float *x, const int *label, int64_t n,
                                                   float *grad, float *loss) {
-    __shared__ float w[NP];
-    __shared__ float g[NP];
-    __shared__ float sl;
-    for (int i = threadIdx.x; i < NP; i += blockDim.x) {
-        w[i] = P[i];
-        g[i] = 0.0f;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    GradSmem &S = *reinterpret_cast<GradSmem *>(smem_raw);
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, tx = tid & 15, ty = tid >> 4;
+    for (int i = tid; i < NH * NH; i += kGT) {
+        const float v = P[OW2 + i];
+        S.w2[i] = v;
+        S.w2t[(i % NH) * NH + i / NH] = v;
     }
-    if (threadIdx.x == 0) sl = 0.0f;
-    __syncthreads();
-    const int lane = threadIdx.x & 31;
+    for (int i = tid; i < NOUT * NH; i += kGT) {
+        const float v = P[OW3 + i];
+        S.w3[i] = v;
+        S.w3t[(i % NH) * NOUT + i / NH] = v;
+    }
+    for (int i = tid; i < NH * NIN; i += kGT) S.w1[i] = P[OW1 + i];
+    for (int i = tid; i < NH; i += kGT) {
+        S.b1[i] = P[OB1 + i];
+        S.b2[i] = P[OB2 + i];
+    }
+    if (tid < NOUT) S.b3[tid] = P[OB3 + tid];
+    float a2[4][4] = {}, a3[4] = {}, a1[2] = {}, ab = 0.0f, lsum = 0.0f;
     const float inv_n = 1.0f / (float)n;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    const int64_t iters = (n + stride - 1) / stride;
-    for (int64_t it = 0; it < iters; ++it) {
-        const int64_t s = it * stride + blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-        const bool valid = s < n;
-        float in[NIN], z1[NH], h1[NH], z2[NH], h2[NH], lg[NOUT];
+    const int64_t tiles = (n + 31) / 32;
+    const int o8 = wid * 8;  // this warp's eight outputs of a 64-wide layer
+    for (int64_t t = blockIdx.x; t < tiles; t += gridDim.x) {
+        const int64_t s0 = t * 32;
+        const bool valid = s0 + lane < n;
+        __syncthreads();  // weights loaded; the previous tile's sums are done
+        if (tid < 32 * NIN) {
+            const int i = tid % NIN, q = tid / NIN;
+            S.in[i][q] = s0 + q < n ? x[s0 * NIN + tid] : 0.0f;
+        }
+        __syncthreads();
+        // ---- forward
 #pragma unroll
-        for (int i = 0; i < NIN; ++i) in[i] = valid ? x[s * NIN + i] : 0.0f;
-        for (int o = 0; o < NH; ++o) {
-            float a = w[OB1 + o];
+        for (int q = 0; q < 8; ++q) {
+            float a = S.b1[o8 + q];
 #pragma unroll
-            for (int i = 0; i < NIN; ++i) a = fmaf(w[OW1 + o * NIN + i], in[i], a);
-            z1[o] = a;
-            h1[o] = gelu(a);
+            for (int i = 0; i < NIN; ++i) a = fmaf(S.w1[(o8 + q) * NIN + i], S.in[i][lane], a);
+            gelu_both(a, S.h1[o8 + q][lane], S.g1[o8 + q][lane]);
         }
-        for (int o = 0; o < NH; ++o) {
-            float a = w[OB2 + o];
-            for (int i = 0; i < NH; ++i) a = fmaf(w[OW2 + o * NH + i], h1[i], a);
-            z2[o] = a;
-            h2[o] = gelu(a);
+        __syncthreads();
+        {
+            float a[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) a[q] = S.b2[o8 + q];
+            layer8<NH>(S.h1, S.w2t + o8, NH, lane, a);
+#pragma unroll
+            for (int q = 0; q < 8; ++q) gelu_both(a[q], S.h2[o8 + q][lane], S.g2[o8 + q][lane]);
         }
-        float mx = -INFINITY;
-        for (int o = 0; o < NOUT; ++o) {
-            float a = w[OB3 + o];
-            for (int i = 0; i < NH; ++i) a = fmaf(w[OW3 + o * NH + i], h2[i], a);
-            lg[o] = a;
-            mx = fmaxf(mx, a);
-        }
-        float se = 0.0f;
-        for (int o = 0; o < NOUT; ++o) se += expf(lg[o] - mx);
-        const int lab = valid ? label[s] : 0;
-        const float ls = wsum(valid ? (logf(se) + mx - lg[lab]) * inv_n : 0.0f);
-        if (lane == 0) atomicAdd(&sl, ls);
-        // backward: d loss / d logits = (softmax - onehot) / n
-        float d3[NOUT];
-        for (int o = 0; o < NOUT; ++o) d3[o] = valid ? (expf(lg[o] - mx) / se - (o == lab ? 1.0f : 0.0f)) * inv_n : 0.0f;
-        for (int o = 0; o < NOUT; ++o) {
-            const float b = wsum(d3[o]);
-            if (lane == 0) atomicAdd(&g[OB3 + o], b);
+        __syncthreads();
+        {
+            const int o = wid * 2;
+            float a0 = S.b3[o], a1q = S.b3[o + 1];
+#pragma unroll 8
             for (int i = 0; i < NH; ++i) {
-                const float v = wsum(d3[o] * h2[i]);
-                if (lane == 0) atomicAdd(&g[OW3 + o * NH + i], v);
+                const float v = S.h2[i][lane];
+                const float2 w = *reinterpret_cast<const float2 *>(&S.w3t[i * NOUT + o]);
+                a0 = fmaf(w.x, v, a0);
+                a1q = fmaf(w.y, v, a1q);
             }
+            S.d3[o][lane] = a0;
+            S.d3[o + 1][lane] = a1q;
         }
-        float d2[NH];
-        for (int i = 0; i < NH; ++i) {
-            float a = 0.0f;
-            for (int o = 0; o < NOUT; ++o) a = fmaf(w[OW3 + o * NH + i], d3[o], a);
-            d2[i] = a * gelu_d(z2[i]);
-        }
-        for (int o = 0; o < NH; ++o) {
-            const float b = wsum(d2[o]);
-            if (lane == 0) atomicAdd(&g[OB2 + o], b);
-            for (int i = 0; i < NH; ++i) {
-                const float v = wsum(d2[o] * h1[i]);
-                if (lane == 0) atomicAdd(&g[OW2 + o * NH + i], v);
-            }
-        }
-        for (int i = 0; i < NH; ++i) {
-            float a = 0.0f;
-            for (int o = 0; o < NH; ++o) a = fmaf(w[OW2 + o * NH + i], d2[o], a);
-            const float d1 = a * gelu_d(z1[i]);
-            const float b = wsum(d1);
-            if (lane == 0) atomicAdd(&g[OB1 + i], b);
+        __syncthreads();
+        // ---- softmax cross-entropy: d loss / d logits = (softmax - onehot) / n
+        {
+            float lg[NOUT], mx = -INFINITY, se = 0.0f;
 #pragma unroll
-            for (int k = 0; k < NIN; ++k) {
-                const float v = wsum(d1 * in[k]);
-                if (lane == 0) atomicAdd(&g[OW1 + i * NIN + k], v);
+            for (int o = 0; o < NOUT; ++o) {
+                lg[o] = S.d3[o][lane];
+                mx = fmaxf(mx, lg[o]);
             }
+#pragma unroll
+            for (int o = 0; o < NOUT; ++o) se += expf(lg[o] - mx);
+            const int lab = valid ? label[s0 + lane] : 0;
+            const float l0 = S.d3[2 * wid][lane], l1 = S.d3[2 * wid + 1][lane];
+            if (wid == 0 && valid) lsum += (logf(se) + mx - S.d3[lab][lane]) * inv_n;
+            __syncthreads();
+            S.d3[2 * wid][lane] = valid ? (expf(l0 - mx) / se - (2 * wid == lab ? 1.0f : 0.0f)) * inv_n : 0.0f;
+            S.d3[2 * wid + 1][lane] = valid ? (expf(l1 - mx) / se - (2 * wid + 1 == lab ? 1.0f : 0.0f)) * inv_n : 0.0f;
         }
+        __syncthreads();
+        // ---- backward: g2 <- d2 = (W3^T d3) gelu'(z2), g1 <- d1 = (W2^T d2) gelu'(z1)
+        {
+            float a[8] = {};
+            layer8<NOUT>(S.d3, S.w3 + o8, NH, lane, a);
+#pragma unroll
+            for (int q = 0; q < 8; ++q) S.g2[o8 + q][lane] *= a[q];
+        }
+        __syncthreads();
+        {
+            float a[8] = {};
+            layer8<NH>(S.g2, S.w2 + o8, NH, lane, a);
+#pragma unroll
+            for (int q = 0; q < 8; ++q) S.g1[o8 + q][lane] *= a[q];
+        }
+        __syncthreads();
+        // ---- gradients over the tile's samples
+        float t2[4][4][2] = {};
+#pragma unroll 2
+        for (int q = 0; q < 32; q += 4) {
+            float4 d[4], h[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                d[e] = *reinterpret_cast<const float4 *>(&S.g2[ty + 16 * e][q]);
+                h[e] = *reinterpret_cast<const float4 *>(&S.h1[tx + 16 * e][q]);
+            }
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+#pragma unroll
+                for (int f = 0; f < 4; ++f) {
+                    t2[e][f][0] = fmaf(d[e].x, h[f].x, fmaf(d[e].y, h[f].y, t2[e][f][0]));
+                    t2[e][f][1] = fmaf(d[e].z, h[f].z, fmaf(d[e].w, h[f].w, t2[e][f][1]));
+                }
+        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+#pragma unroll
+            for (int f = 0; f < 4; ++f) a2[e][f] += t2[e][f][0] + t2[e][f][1];
+#pragma unroll
+        for (int f = 0; f < 4; ++f) a3[f] = row_dot(S.d3[ty], S.h2[tx + 16 * f], a3[f]);
+#pragma unroll
+        for (int f = 0; f < 2; ++f) {
+            const int e = tid + kGT * f;
+            if (e < NH * NIN) a1[f] = row_dot(S.g1[e / NIN], S.in[e % NIN], a1[f]);
+        }
+        if (tid < NH) ab = row_sum(S.g1[tid], ab);
+        else if (tid < 2 * NH) ab = row_sum(S.g2[tid - NH], ab);
+        else if (tid < 2 * NH + NOUT) ab = row_sum(S.d3[tid - 2 * NH], ab);
     }
-    __syncthreads();
-    for (int i = threadIdx.x; i < NP; i += blockDim.x) atomicAdd(&grad[i], g[i]);
-    if (threadIdx.x == 0) atomicAdd(loss, sl);
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+#pragma unroll
+        for (int f = 0; f < 4; ++f) atomicAdd(&grad[OW2 + (ty + 16 * e) * NH + tx + 16 * f], a2[e][f]);
+        atomicAdd(&grad[OW3 + ty * NH + tx + 16 * e], a3[e]);
+    }
+    for (int f = 0; f < 2; ++f)
+        if (tid + kGT * f < NH * NIN) atomicAdd(&grad[OW1 + tid + kGT * f], a1[f]);
+    if (tid < NH) atomicAdd(&grad[OB1 + tid], ab);
+    else if (tid < 2 * NH) atomicAdd(&grad[OB2 + tid - NH], ab);
+    else if (tid < 2 * NH + NOUT) atomicAdd(&grad[OB3 + tid - 2 * NH], ab);
+    if (wid == 0) {
+        lsum = warp_sum(lsum);
+        if (lane == 0) atomicAdd(loss, lsum);
+    }
 }
 
 // Adam: m = b1 m + (1-b1) g; v = b2 v + (1-b2) g^2;
@@ -294,8 +401,10 @@ int td_mlp_grad(cudaStream_t st, const float *P, const float *x, const int *labe
     cudaMemsetAsync(grad, 0, sizeof(float) * NP, st);
     cudaMemsetAsync(loss, 0, sizeof(float), st);
     if (n <= 0) return (int)cudaGetLastError();
-    const int grid = (int)std::min<int64_t>((n + 127) / 128, (int64_t)num_sms * 4);
-    k_mlp_grad<<<grid, 128, 0, st>>>(P, x, label, n, grad, loss);
+    const cudaError_t e = cudaFuncSetAttribute(k_mlp_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(GradSmem));
+    if (e != cudaSuccess) return (int)e;
+    const int grid = (int)std::min<int64_t>((n + 31) / 32, (int64_t)num_sms * 2);
+    k_mlp_grad<<<grid, kGT, sizeof(GradSmem), st>>>(P, x, label, n, grad, loss);
     return (int)cudaGetLastError();
 }
 
