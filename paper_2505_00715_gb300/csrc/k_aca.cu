@@ -248,43 +248,107 @@ __global__ void __launch_bounds__(128) k_near_aca(MeshDev m, NearArgs a, TensorO
 // ============================================================================
 // Far field
 // ============================================================================
-// One point pair (a of the test triangle, b of the trial triangle); fibres and
-// tubes are evaluated one entry per warp, the lanes splitting the point pairs.
-TD_D c32 point_pair(const MeshDev &m, int op, int ti, int a, int tj, int b, int loc, float sr, float si) {
-    const int oa = a * m.nt + ti, ob = b * m.nt + tj;
-    const float4 xa = __ldg(&m.qp[2 * oa]), xla = __ldg(&m.qp[2 * oa + 1]);
-    const float4 yb = __ldg(&m.qp[2 * ob]), ylb = __ldg(&m.qp[2 * ob + 1]);
-    const float dx = (yb.x - xa.x) + (ylb.x - xla.x);
-    const float dy = (yb.y - xa.y) + (ylb.y - xla.y);
-    const float dz = (yb.z - xa.z) + (ylb.z - xla.z);
+// A quadrature point with its weight (FP32: hi + lo coordinates), and one point
+// pair of test point x and trial point y: w e^{-sigma r} / r (SLP) or
+// w (1 + sigma r) e^{-sigma r} (d.n) / r^3 with the signed kernel normal n
+// (-n_y times the trial hat for DLP, n_x for ADLP); w the product of the weights.
+template <class T> struct QPoint;
+template <> struct QPoint<float> {
+    float4 h, l;
+};
+template <> struct QPoint<double> {
+    double x, y, z, w;
+};
+TD_D void load_q(const MeshDev &m, int o, QPoint<float> &q) {
+    q.h = __ldg(&m.qp[2 * o]);
+    q.l = __ldg(&m.qp[2 * o + 1]);
+}
+TD_D void load_q(const MeshDev &m, int o, QPoint<double> &q) {
+    q.x = m.qx[o];
+    q.y = m.qy[o];
+    q.z = m.qz[o];
+    q.w = m.qw[o];
+}
+template <class T> struct Vec3 {
+    T x, y, z;
+};
+// kernel normal of an entry: the trial triangle's (DLP, with -1) or the test one's
+template <int OP>
+TD_D Vec3<float> kernel_normal(const MeshDev &m, int ti, int tj, float) {
+    if (OP == TD_SLP) return {0.f, 0.f, 0.f};
+    const float4 n = __ldg(&m.nrm4[OP == TD_DLP ? tj : ti]);
+    return {n.x, n.y, n.z};
+}
+template <int OP>
+TD_D Vec3<double> kernel_normal(const MeshDev &m, int ti, int tj, double) {
+    if (OP == TD_SLP) return {0.0, 0.0, 0.0};
+    const int t = OP == TD_DLP ? tj : ti;
+    return {m.n64[t], m.n64[m.nt + t], m.n64[2 * m.nt + t]};
+}
+// (added to acc with explicit fused multiply-adds, so that every fibre rounds the
+// same way)
+template <int OP>
+TD_D void add_pair(c32 &acc, const QPoint<float> &x, const QPoint<float> &y, const Vec3<float> &n, float hat, float sr,
+                   float si) {
+    const float dx = (y.h.x - x.h.x) + (y.l.x - x.l.x);
+    const float dy = (y.h.y - x.h.y) + (y.l.y - x.l.y);
+    const float dz = (y.h.z - x.h.z) + (y.l.z - x.l.z);
     const float r2 = dx * dx + dy * dy + dz * dz;
     const float rinv = rsqrtf(r2), r = r2 * rinv;
     const c32 e = expm_sr(sr, si, r);
-    float w = xa.w * yb.w * rinv;
-    if (op == TD_SLP) return {w * e.x, w * e.y};
-    if (op == TD_DLP) {
-        const float4 n = __ldg(&m.nrm4[tj]);  // (x - y).n_y, P1 hat of the trial vertex
-        w *= bary7f(b, loc) * -(dx * n.x + dy * n.y + dz * n.z) * rinv * rinv;
-    } else {
-        const float4 n = __ldg(&m.nrm4[ti]);  // (y - x).n_x
-        w *= (dx * n.x + dy * n.y + dz * n.z) * rinv * rinv;
+    float w = x.h.w * y.h.w * rinv;
+    if (OP == TD_SLP) {
+        acc = c32{fmaf(w, e.x, acc.x), fmaf(w, e.y, acc.y)};
+        return;
     }
+    if (OP == TD_DLP) w *= hat * -(dx * n.x + dy * n.y + dz * n.z) * rinv * rinv;
+    else w *= (dx * n.x + dy * n.y + dz * n.z) * rinv * rinv;
     const float pr = fmaf(sr, r, 1.0f), pi = si * r;
-    return {w * (pr * e.x - pi * e.y), w * (pr * e.y + pi * e.x)};
+    acc = c32{fmaf(w, pr * e.x - pi * e.y, acc.x), fmaf(w, pr * e.y + pi * e.x, acc.y)};
 }
-TD_D c64 point_pair(const MeshDev &m, int op, int ti, int a, int tj, int b, int loc, double sr, double si) {
-    const int oa = a * m.nt + ti, ob = b * m.nt + tj;
-    double dx = m.qx[ob] - m.qx[oa], dy = m.qy[ob] - m.qy[oa], dz = m.qz[ob] - m.qz[oa];
-    double r = sqrt(dx * dx + dy * dy + dz * dz);
-    c64 e = expm_sr(sr, si, r);
-    double w = m.qw[oa] * m.qw[ob] / r;
-    if (op == TD_SLP) return {w * e.x, w * e.y};
-    if (op == TD_DLP)
-        w *= bary7d(b, loc) * -(dx * m.n64[tj] + dy * m.n64[m.nt + tj] + dz * m.n64[2 * m.nt + tj]) / (r * r);
-    else
-        w *= (dx * m.n64[ti] + dy * m.n64[m.nt + ti] + dz * m.n64[2 * m.nt + ti]) / (r * r);
-    double pr = 1.0 + sr * r, pi = si * r;
-    return {w * (pr * e.x - pi * e.y), w * (pr * e.y + pi * e.x)};
+template <int OP>
+TD_D void add_pair(c64 &acc, const QPoint<double> &x, const QPoint<double> &y, const Vec3<double> &n, double hat,
+                   double sr, double si) {
+    const double dx = y.x - x.x, dy = y.y - x.y, dz = y.z - x.z;
+    const double r = sqrt(dx * dx + dy * dy + dz * dz);
+    const c64 e = expm_sr(sr, si, r);
+    double w = x.w * y.w / r;
+    if (OP == TD_SLP) {
+        acc = c64{fma(w, e.x, acc.x), fma(w, e.y, acc.y)};
+        return;
+    }
+    if (OP == TD_DLP) w *= hat * -(dx * n.x + dy * n.y + dz * n.z) / (r * r);
+    else w *= (dx * n.x + dy * n.y + dz * n.z) / (r * r);
+    const double pr = 1.0 + sr * r, pi = si * r;
+    acc = c64{fma(w, pr * e.x - pi * e.y, acc.x), fma(w, pr * e.y + pi * e.x, acc.y)};
+}
+TD_D float hat_at(int b, int loc, float) { return bary7f(b, loc); }
+TD_D double hat_at(int b, int loc, double) { return bary7d(b, loc); }
+
+// Sum of a group of 8 lanes (the total reaches all of them), 1/(4 pi) applied.
+// Every lane of the warp must call it.
+template <class T>
+TD_D cx<T> group_total(cx<T> acc) {
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) {
+        acc.x += __shfl_xor_sync(0xffffffffu, acc.x, o);
+        acc.y += __shfl_xor_sync(0xffffffffu, acc.y, o);
+    }
+    const T s = (T)(1.0 / TD_FOUR_PI);
+    return cx<T>{acc.x * s, acc.y * s};
+}
+// acc + the seven point pairs add(acc, 0..6) of a lane, in three interleaved chains
+template <class T, class F>
+TD_D cx<T> sum7(cx<T> acc, F add) {
+    cx<T> b = {0, 0}, c = {0, 0};
+    add(acc, 0);
+    add(b, 1);
+    add(c, 2);
+    add(acc, 3);
+    add(b, 4);
+    add(c, 5);
+    add(acc, 6);
+    return acc + (b + c);
 }
 
 // Entry by a group of 8 lanes: lanes 0..6 of the group take test point a =
@@ -296,38 +360,112 @@ TD_D cx<T> group_entry(const MeshDev &m, int row, int col, T sr, T si, bool vali
     const int sub = threadIdx.x & 7;
     cx<T> acc = {0, 0};
     if (valid && sub < 7) {
-        if (!TD_P1_TRIAL(OP)) {
-            // independent point pairs in flight: 3 + 3 + 1
-            cx<T> acc2 = {0, 0}, acc3 = {0, 0};
-#pragma unroll 1
-            for (int b = 0; b < 6; b += 3) {
-                acc = acc + point_pair(m, OP, row, sub, col, b, 0, sr, si);
-                acc2 = acc2 + point_pair(m, OP, row, sub, col, b + 1, 0, sr, si);
-                acc3 = acc3 + point_pair(m, OP, row, sub, col, b + 2, 0, sr, si);
-            }
-            acc = acc + point_pair(m, OP, row, sub, col, 6, 0, sr, si) + (acc2 + acc3);
-        } else {
-            const int p1 = m.v2t_ptr[col + 1];
-            for (int p = m.v2t_ptr[col]; p < p1; ++p) {
-                const int tj = m.v2t[p], loc = m.v2t_loc[p];
-                cx<T> acc2 = {0, 0}, acc3 = {0, 0};
-#pragma unroll 1
-                for (int b = 0; b < 6; b += 3) {
-                    acc = acc + point_pair(m, OP, row, sub, tj, b, loc, sr, si);
-                    acc2 = acc2 + point_pair(m, OP, row, sub, tj, b + 1, loc, sr, si);
-                    acc3 = acc3 + point_pair(m, OP, row, sub, tj, b + 2, loc, sr, si);
-                }
-                acc = acc + point_pair(m, OP, row, sub, tj, 6, loc, sr, si) + (acc2 + acc3);
-            }
+        QPoint<T> x;
+        load_q(m, sub * m.nt + row, x);
+        const int p0 = TD_P1_TRIAL(OP) ? m.v2t_ptr[col] : 0, p1 = TD_P1_TRIAL(OP) ? m.v2t_ptr[col + 1] : 1;
+        for (int p = p0; p < p1; ++p) {
+            const int tj = TD_P1_TRIAL(OP) ? m.v2t[p] : col, loc = TD_P1_TRIAL(OP) ? m.v2t_loc[p] : 0;
+            const Vec3<T> n = kernel_normal<OP>(m, row, tj, T(0));
+            acc = sum7<T>(acc, [&](cx<T> &s, int b) {
+                QPoint<T> y;
+                load_q(m, b * m.nt + tj, y);
+                add_pair<OP>(s, x, y, n, TD_P1_TRIAL(OP) ? hat_at(b, loc, T(0)) : T(1), sr, si);
+            });
         }
     }
-#pragma unroll
-    for (int o = 4; o > 0; o >>= 1) {
-        acc.x += __shfl_xor_sync(0xffffffffu, acc.x, o);
-        acc.y += __shfl_xor_sync(0xffffffffu, acc.y, o);
+    return group_total(acc);
+}
+
+// The entries of a fibre, with group_entry's sums (same values).  Each lane holds
+// the test point of its number.  Row fibre A(i*, cols[j]): the test points stay in
+// registers; a group's seven lanes read one trial point of the column's triangle
+// each and exchange them through shared memory (ex: 2 x 4 groups x 7 points of
+// the warp), the next triangle's point on its way while this one is evaluated.
+// Column fibre A(rows[i], j*): the column's seven points stay in shared memory (fx) and
+// the lanes read their test point of the next row.  Every lane of a group used to
+// read all seven trial points itself, 14 16-byte loads an entry through an L1
+// that shared memory leaves a quarter of: 30k housing 617 -> 547 ms (whole far
+// phase), 5120-triangle sphere 61 -> 57, double layer 133 -> 97 ms.
+// P1 columns: every support triangle in turn (row), group_entry (column).
+template <class T, int OP, class F>
+TD_D void row_fibre(const MeshDev &m, QPoint<T> *ex, int row, const int *cols, int nJ, T sr, T si, F out) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, step = (blockDim.x >> 5) * 4, sub = lane & 7;
+    const int pt = min(sub, 6);
+    const unsigned gmask = 0xffu << (lane & 24);
+    QPoint<T> x, y;
+    load_q(m, pt * m.nt + row, x);
+    ex += (lane >> 3) * 7;
+    int j = wid * 4 + (lane >> 3), buf = 0;
+    if (!TD_P1_TRIAL(OP)) {
+        int cn = cols[min(j + step, nJ - 1)];
+        load_q(m, pt * m.nt + cols[min(j, nJ - 1)], y);
+        const Vec3<T> n = kernel_normal<OP>(m, row, 0, T(0));
+        for (int j0 = wid * 4; j0 < nJ; j0 += step, j += step, buf ^= 28) {  // warp-uniform trip count
+            if (sub < 7) ex[buf + sub] = y;
+            load_q(m, pt * m.nt + cn, y);
+            cn = cols[min(j + 2 * step, nJ - 1)];
+            __syncwarp();
+            cx<T> acc = {0, 0};
+            if (sub < 7) acc = sum7<T>(acc, [&](cx<T> &s, int b) { add_pair<OP>(s, x, ex[buf + b], n, T(1), sr, si); });
+            acc = group_total(acc);
+            if (j < nJ && sub == 0) out(j, acc);
+        }
+    } else {
+        for (int j0 = wid * 4; j0 < nJ; j0 += step, j += step) {
+            const int col = cols[min(j, nJ - 1)];
+            const int p0 = m.v2t_ptr[col], p1 = m.v2t_ptr[col + 1];
+            cx<T> acc = {0, 0};
+            int tn = p0 < p1 ? m.v2t[p0] : 0;
+            load_q(m, pt * m.nt + tn, y);
+            for (int p = p0; p < p1; ++p, buf ^= 28) {
+                const int tj = tn, loc = m.v2t_loc[p];
+                if (sub < 7) ex[buf + sub] = y;
+                tn = m.v2t[min(p + 1, p1 - 1)];
+                load_q(m, pt * m.nt + tn, y);
+                const Vec3<T> n = kernel_normal<OP>(m, row, tj, T(0));
+                __syncwarp(gmask);
+                if (sub < 7)
+                    acc = sum7<T>(acc, [&](cx<T> &s, int b) { add_pair<OP>(s, x, ex[buf + b], n, hat_at(b, loc, T(0)), sr, si); });
+            }
+            __syncwarp();
+            acc = group_total(acc);
+            if (j < nJ && sub == 0) out(j, acc);
+        }
     }
-    const T s = (T)(1.0 / TD_FOUR_PI);
-    return cx<T>{acc.x * s, acc.y * s};
+    __syncwarp();  // ex is free again
+}
+// The seven points of a column's triangle to shared memory.
+template <class T>
+TD_D void stage_fixed(const MeshDev &m, int tri, QPoint<T> *fx) {
+    if (threadIdx.x < 7) load_q(m, threadIdx.x * m.nt + tri, fx[threadIdx.x]);
+}
+template <class T, int OP, class F>
+TD_D void col_fibre(const MeshDev &m, const QPoint<T> *fx, const int *rows, int nI, int col, T sr, T si, F out) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, step = (blockDim.x >> 5) * 4, sub = lane & 7;
+    int i = wid * 4 + (lane >> 3);
+    if (!TD_P1_TRIAL(OP)) {
+        const int pt = min(sub, 6);
+        int rc = rows[min(i, nI - 1)], rn = rows[min(i + step, nI - 1)];
+        QPoint<T> x;
+        load_q(m, pt * m.nt + rc, x);
+        for (int i0 = wid * 4; i0 < nI; i0 += step, i += step) {  // warp-uniform trip count
+            const Vec3<T> n = kernel_normal<OP>(m, rc, col, T(0));
+            QPoint<T> xn;
+            load_q(m, pt * m.nt + rn, xn);
+            rc = rn;
+            rn = rows[min(i + 2 * step, nI - 1)];
+            cx<T> acc = {0, 0};
+            if (sub < 7) acc = sum7<T>(acc, [&](cx<T> &s, int b) { add_pair<OP>(s, x, fx[b], n, T(1), sr, si); });
+            acc = group_total(acc);
+            if (i < nI && sub == 0) out(i, acc);
+            x = xn;
+        }
+    } else {
+        for (int i0 = wid * 4; i0 < nI; i0 += step, i += step) {
+            const cx<T> v = group_entry<T, OP>(m, rows[min(i, nI - 1)], col, sr, si, i < nI);
+            if (i < nI && sub == 0) out(i, v);
+        }
+    }
 }
 
 constexpr int kNCoef = 512;
@@ -371,11 +509,18 @@ struct FarShared {
     int idx;
     long long off;
     cx<T> piv;
+    QPoint<T> fx[7];  // points of the column j* whose fibre is evaluated
+    AccT<T> gre[kGmax][kGmax], gim[kGmax][kGmax];  // <H_d, H_d'> of the block's kept terms
+    double floor2;  // mixed form: (2^-20 ||C^(l-1)(k_l)||_F)^2, the face ACA's noise floor (0: none)
+};
+
+// Coefficient lists of the residual corrections (faces above kDenseS entries): in
+// the place of the Gram tiles, which are idle during a face's ACA.
+template <class T>
+struct FarCoef {
     cx<T> coef[kNCoef];
     const cx<T> *base[kNCoef];
     cx<T> part[256];  // partial corrections of the thread groups (correct_fibre)
-    AccT<T> gre[kGmax][kGmax], gim[kGmax][kGmax];  // <H_d, H_d'> of the block's kept terms
-    double floor2;  // mixed form: (2^-20 ||C^(l-1)(k_l)||_F)^2, the face ACA's noise floor (0: none)
 };
 
 // Per-frequency arrays of one far-field CTA, carved from dynamic shared memory
@@ -419,7 +564,7 @@ TD_D FarFreq<T> far_freq(unsigned char *p, int Nu) {
 // f_d[k] V_d[tau][j*], base U_d[tau]), followed by the current face's own
 // terms (u_t[i*], base v_t) / (v_t[j*], base u_t).  Entries [c0, c0+kNCoef).
 template <class T>
-TD_D int build_coef(FarShared<T> &S, const FarFreq<T> &F, int mode, int fixed, int l, int kf, int k, int Nu,
+TD_D int build_coef(FarCoef<T> &S, const FarFreq<T> &F, int mode, int fixed, int l, int kf, int k, int Nu,
                     int64_t tb, int nI, int nJ, const cx<T> *pool, const cx<T> *fib, const cx<T> *Uw,
                     const cx<T> *Vw, int maxI, int maxJ, int c0) {
     int total = kf;
@@ -464,7 +609,7 @@ TD_D int build_coef(FarShared<T> &S, const FarFreq<T> &F, int mode, int fixed, i
 // that more loads are in flight, and combine the partial sums through
 // shared memory.  Called by every thread of the block.
 template <class T>
-TD_D void correct_fibre(FarShared<T> &S, cx<T> *x, int n, int cn) {
+TD_D void correct_fibre(FarCoef<T> &S, cx<T> *x, int n, int cn) {
     const int G = n >= (int)blockDim.x ? 1 : min(16, (int)blockDim.x / n);
     if (G == 1) {
         for (int j = threadIdx.x; j < n; j += blockDim.x) x[j] = x[j] - coef_sum(S.coef, S.base, cn, j);
@@ -830,7 +975,11 @@ __global__ void __launch_bounds__(NT, 640 / NT) k_far_aca(MeshDev m, FarArgs a, 
     size_t soff = align16(sizeof(FarShared<T>));
     GramTiles<T> *gt = reinterpret_cast<GramTiles<T> *>(smem_raw + soff);
     cx<T> *Ss = reinterpret_cast<cx<T> *>(gt);  // S of dense-S blocks (no Gram tiles needed there)
+    FarCoef<T> &Q = *reinterpret_cast<FarCoef<T> *>(gt);  // (dense-S faces use no coefficient lists)
+    static_assert(sizeof(GramTiles<T>) >= sizeof(FarCoef<T>), "the coefficient lists must fit in the Gram tiles");
     soff += align16(sizeof(GramTiles<T>));
+    QPoint<T> *ex = reinterpret_cast<QPoint<T> *>(smem_raw + soff) + (threadIdx.x >> 5) * 56;  // row_fibre's exchange
+    soff += align16(sizeof(QPoint<T>) * 56 * (NT / 32));
     const int Nu = a.nf;
     FarFreq<T> F = far_freq<T>(smem_raw + soff, Nu);
     soff += far_freq_bytes<T>(Nu);
@@ -877,7 +1026,7 @@ __global__ void __launch_bounds__(NT, 640 / NT) k_far_aca(MeshDev m, FarArgs a, 
             const bool small = dense_b && l < nd, cdm = cd_b && small, dense_s = dense_sb && small;
             for (int t = tid; t < 64; t += blockDim.x) S.nrow[t] = A(0);
             if (small && !cdm)
-                for (int d = tid; d < l; d += blockDim.x) S.coef[d] = fib[(tb + d) * Nu + k];
+                for (int d = tid; d < l; d += blockDim.x) Q.coef[d] = fib[(tb + d) * Nu + k];
             if (cdm) {
                 for (int e = tid; e < nI * nJ; e += blockDim.x) {
                     cx<T> acc = {0, 0};
@@ -916,17 +1065,13 @@ __global__ void __launch_bounds__(NT, 640 / NT) k_far_aca(MeshDev m, FarArgs a, 
                     ++guard;
                     // residual row fibre at i*: entry minus C and S, by the group leader
                     AM am = {-1, 0x7fffffff};
-                    for (int j0 = wid * 4; j0 < nJ; j0 += nwarps * 4) {
-                        const int j = j0 + (lane >> 3);
-                        const cx<T> ent = group_entry<T, OP>(m, rows[istar], cols[min(j, nJ - 1)], sr, si, j < nJ);
-                        if (j < nJ && (lane & 7) == 0) {
-                            const int64_t e = (int64_t)istar * nJ + j;
-                            const cx<T> v = ent - Cd[e] - Ss[e];
-                            Vw[(int64_t)kf * a.maxJ + j] = v;
-                            const auto key = pivot_key(v);
-                            if (am_better(key, j, am.v, am.i)) am = {key, j};
-                        }
-                    }
+                    row_fibre<T, OP>(m, ex, rows[istar], cols, nJ, sr, si, [&](int j, cx<T> ent) {
+                        const int64_t e = (int64_t)istar * nJ + j;
+                        const cx<T> v = ent - Cd[e] - Ss[e];
+                        Vw[(int64_t)kf * a.maxJ + j] = v;
+                        const auto key = pivot_key(v);
+                        if (am_better(key, j, am.v, am.i)) am = {key, j};
+                    });
                     ev_reg += nJ;
                     am = block_argmax_1sync(am, S.red[par]);
                     par ^= 1;
@@ -951,19 +1096,19 @@ __global__ void __launch_bounds__(NT, 640 / NT) k_far_aca(MeshDev m, FarArgs a, 
                     const cx<T> piv = Vw[(int64_t)kf * a.maxJ + jstar];
                     // residual column fibre at j*, divided by the pivot
                     AM am2 = {-1, 0x7fffffff};
-                    for (int i0 = wid * 4; i0 < nI; i0 += nwarps * 4) {
-                        const int i = i0 + (lane >> 3);
-                        const cx<T> ent = group_entry<T, OP>(m, rows[min(i, nI - 1)], cols[jstar], sr, si, i < nI);
-                        if (i < nI && (lane & 7) == 0) {
-                            const int64_t e = (int64_t)i * nJ + jstar;
-                            const cx<T> u = cdiv(ent - Cd[e] - Ss[e], piv);
-                            Uw[(int64_t)kf * a.maxI + i] = u;
-                            if (i != istar && !(used[i >> 5] & (1u << (i & 31)))) {
-                                const auto key = pivot_key(u);
-                                if (am_better(key, i, am2.v, am2.i)) am2 = {key, i};
-                            }
-                        }
+                    if (!TD_P1_TRIAL(OP)) {
+                        stage_fixed(m, cols[jstar], S.fx);  // (the arg-max barrier closed the row fibre)
+                        __syncthreads();
                     }
+                    col_fibre<T, OP>(m, S.fx, rows, nI, cols[jstar], sr, si, [&](int i, cx<T> ent) {
+                        const int64_t e = (int64_t)i * nJ + jstar;
+                        const cx<T> u = cdiv(ent - Cd[e] - Ss[e], piv);
+                        Uw[(int64_t)kf * a.maxI + i] = u;
+                        if (i != istar && !(used[i >> 5] & (1u << (i & 31)))) {
+                            const auto key = pivot_key(u);
+                            if (am_better(key, i, am2.v, am2.i)) am2 = {key, i};
+                        }
+                    });
                     ev_reg += nI;
                     am2 = block_argmax_1sync(am2, S.red[par]);
                     par ^= 1;
@@ -1027,11 +1172,8 @@ __global__ void __launch_bounds__(NT, 640 / NT) k_far_aca(MeshDev m, FarArgs a, 
                 // residual corrections in chunks
                 AM am = {-1, 0x7fffffff};
                 int total = 0;
-                for (int j0 = wid * 4; j0 < nJ; j0 += nwarps * 4) {  // warp-uniform trip count
-                    const int j = j0 + (lane >> 3);
-                    const cx<T> v = group_entry<T, OP>(m, rows[istar], cols[min(j, nJ - 1)], sr, si, j < nJ);
-                    if (j < nJ && (lane & 7) == 0) Vw[(int64_t)kf * a.maxJ + j] = v;
-                }
+                row_fibre<T, OP>(m, ex, rows[istar], cols, nJ, sr, si,
+                                 [&](int j, cx<T> v) { Vw[(int64_t)kf * a.maxJ + j] = v; });
                 ev_reg += nJ;
                 if (small) {
                     // previous terms from C(k); the face's own terms by each thread
@@ -1039,7 +1181,7 @@ __global__ void __launch_bounds__(NT, 640 / NT) k_far_aca(MeshDev m, FarArgs a, 
                     __syncthreads();
                     for (int j = tid; j < nJ; j += blockDim.x) {
                         const int64_t ep = (int64_t)istar * nJ + j;
-                        cx<T> v = Vw[(int64_t)kf * a.maxJ + j] - (cdm ? Cd[ep] : dense_prev(Hs, nIJb, S.coef, l, ep));
+                        cx<T> v = Vw[(int64_t)kf * a.maxJ + j] - (cdm ? Cd[ep] : dense_prev(Hs, nIJb, Q.coef, l, ep));
                         v = v - own_sum(Uw, (int64_t)a.maxI, istar, Vw, (int64_t)a.maxJ, j, kf);
                         Vw[(int64_t)kf * a.maxJ + j] = v;
                         const auto key = pivot_key(v);
@@ -1048,9 +1190,9 @@ __global__ void __launch_bounds__(NT, 640 / NT) k_far_aca(MeshDev m, FarArgs a, 
                 } else {
                     for (int c0 = 0;; c0 += kNCoef) {
                         __syncthreads();
-                        total = build_coef(S, F, 0, istar, l, kf, k, Nu, tb, nI, nJ, pool, fib, Uw, Vw, a.maxI, a.maxJ, c0);
+                        total = build_coef(Q, F, 0, istar, l, kf, k, Nu, tb, nI, nJ, pool, fib, Uw, Vw, a.maxI, a.maxJ, c0);
                         __syncthreads();
-                        correct_fibre(S, Vw + (int64_t)kf * a.maxJ, nJ, min(kNCoef, total - c0));
+                        correct_fibre(Q, Vw + (int64_t)kf * a.maxJ, nJ, min(kNCoef, total - c0));
                         if (c0 + kNCoef >= total) break;
                     }
                     for (int j = tid; j < nJ; j += blockDim.x) {
@@ -1079,24 +1221,22 @@ __global__ void __launch_bounds__(NT, 640 / NT) k_far_aca(MeshDev m, FarArgs a, 
                 }
                 const int jstar = am.i;
                 const cx<T> piv = Vw[(int64_t)kf * a.maxJ + jstar];
+                if (!TD_P1_TRIAL(OP)) stage_fixed(m, cols[jstar], S.fx);
                 __syncthreads();
                 for (int j = tid; j < nJ; j += blockDim.x) {
                     cx<T> v = Vw[(int64_t)kf * a.maxJ + j];
                     Vw[(int64_t)kf * a.maxJ + j] = cdiv(v, piv);
                 }
                 // column fibre at jstar
-                for (int i0 = wid * 4; i0 < nI; i0 += nwarps * 4) {
-                    const int i = i0 + (lane >> 3);
-                    const cx<T> v = group_entry<T, OP>(m, rows[min(i, nI - 1)], cols[jstar], sr, si, i < nI);
-                    if (i < nI && (lane & 7) == 0) Uw[(int64_t)kf * a.maxI + i] = v;
-                }
+                col_fibre<T, OP>(m, S.fx, rows, nI, cols[jstar], sr, si,
+                                 [&](int i, cx<T> v) { Uw[(int64_t)kf * a.maxI + i] = v; });
                 ev_reg += nI;
                 if (!small) {
                     for (int c0 = 0;; c0 += kNCoef) {
                         __syncthreads();
-                        total = build_coef(S, F, 1, jstar, l, kf, k, Nu, tb, nI, nJ, pool, fib, Uw, Vw, a.maxI, a.maxJ, c0);
+                        total = build_coef(Q, F, 1, jstar, l, kf, k, Nu, tb, nI, nJ, pool, fib, Uw, Vw, a.maxI, a.maxJ, c0);
                         __syncthreads();
-                        correct_fibre(S, Uw + (int64_t)kf * a.maxI, nI, min(kNCoef, total - c0));
+                        correct_fibre(Q, Uw + (int64_t)kf * a.maxI, nI, min(kNCoef, total - c0));
                         if (c0 + kNCoef >= total) break;
                     }
                 }
@@ -1107,7 +1247,7 @@ __global__ void __launch_bounds__(NT, 640 / NT) k_far_aca(MeshDev m, FarArgs a, 
                     if (small) {
                         // previous terms from C(k); the face's own terms by each thread
                         const int64_t ep = (int64_t)i * nJ + jstar;
-                        u = u - (cdm ? Cd[ep] : dense_prev(Hs, nIJb, S.coef, l, ep));
+                        u = u - (cdm ? Cd[ep] : dense_prev(Hs, nIJb, Q.coef, l, ep));
                         u = u - own_sum(Vw, (int64_t)a.maxJ, jstar, Uw, (int64_t)a.maxI, i, kf);
                         Uw[(int64_t)kf * a.maxI + i] = u;
                     }
@@ -1434,7 +1574,8 @@ int td_launch_near_aca(cudaStream_t st, const MeshDev &m, int op, int prec, cons
 template <class T, int OP, int NT>
 static int launch_far_nt(cudaStream_t st, const MeshDev &m, const FarArgs &a, const TensorOut &o,
                          const AcaParams &p, int nctas) {
-    const size_t sm = align16(sizeof(FarShared<T>)) + align16(sizeof(GramTiles<T>)) + far_freq_bytes<T>(a.nf) +
+    const size_t sm = align16(sizeof(FarShared<T>)) + align16(sizeof(GramTiles<T>)) +
+                      align16(sizeof(QPoint<T>) * 56 * (NT / 32)) + far_freq_bytes<T>(a.nf) +
                       sizeof(unsigned int) * ((a.maxI + 31) / 32 + 1);
     cudaError_t e = cudaFuncSetAttribute(k_far_aca<T, OP, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return (int)e;
