@@ -381,7 +381,7 @@ int tdbem_measure_peak(tdbem_ctx_t ctx, int32_t what, double *ops_per_s);
 /* ---- per-frequency solve (Sec. 2, the Laplace-domain systems of the gCQ
  * step; Sec. 5 solves them iteratively) --------------------------------------
  * Solves A(s_fidx) x = b for nrhs right-hand sides with restarted GMRES
- * (modified Gram-Schmidt Arnoldi, complex Givens rotations, FP64 inner
+ * (Arnoldi by classical Gram-Schmidt applied twice, complex Givens rotations, FP64 inner
  * products; every operator application is tdbem_apply_freq on the compressed
  * tensor).  The paper uses BiCGstab; GMRES reaches the same solution and
  * its residual decreases monotonically.  Square operators only (SLP).

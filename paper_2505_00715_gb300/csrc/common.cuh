@@ -48,6 +48,33 @@ TD_D float warp_sum(float v) {
     return v;
 }
 
+// Sums N values (a power of two <= 32) over the warp: a lane gives away half of its
+// values at each step until one is left, so that N values take N - 1 + 5 - log2 N
+// exchanges instead of 5 N (the additions are warp_sum's, in its order).  Returns the
+// total of value many_index<N>(lane).
+template <int N>
+TD_D int many_index(int lane) {
+    int idx = 0;
+#pragma unroll
+    for (int n = N / 2, o = 16; n >= 1; n /= 2, o /= 2) idx += (lane & o) ? n : 0;
+    return idx;
+}
+template <int N, class T>
+TD_D T warp_sum_many(T *v, int lane) {
+    int o = 16;
+#pragma unroll
+    for (int n = N / 2; n >= 1; n /= 2, o /= 2) {
+        const bool up = lane & o;
+#pragma unroll
+        for (int q = 0; q < n; ++q) {
+            const T send = up ? v[q] : v[q + n], keep = up ? v[q + n] : v[q];
+            v[q] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+        }
+    }
+    for (; o > 0; o /= 2) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+    return v[0];
+}
+
 // arg-max over (value, index) pairs: larger value wins, ties -> lower index.
 struct ArgMax {
     float v;

@@ -8,33 +8,34 @@
 // columns, all NQ frequencies) through shared memory, the frequency
 // contraction of every term is done on the tile, then contracted with the
 // face (near) or V (far); results are added to y with atomics.
+#include <algorithm>
+
 #include "internal.h"
 #include "kernels.h"
 
 namespace {
 
-template <class T>
-TD_D void atomic_add_c(cx<T> *p, cx<T> v) {
+TD_D void atomic_add_c(c64 *p, c64 v) {
     atomicAdd(&p->x, v.x);
     atomicAdd(&p->y, v.y);
 }
+TD_D void atomic_add_c(c32 *p, c32 v) { atomicAdd(reinterpret_cast<float2 *>(p), make_float2(v.x, v.y)); }
 
-// dynamic shared memory layout (complex T units):
+// FP64 weighted apply.  Dynamic shared memory layout (complex units):
 //   Wt [NQ][TJ][nrhs] | z [RC][2][TJ][nrhs] | acc: near [nI][nrhs] or far [sumk][2][nrhs]
-template <class T>
 __global__ void __launch_bounds__(256) k_apply(ApplyArgs a, TensorOut o, int TJ, int RC) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    cx<T> *sm = reinterpret_cast<cx<T> *>(smem_raw);
-    const int NQ = a.single_f >= 0 ? 1 : a.NQ;
+    c64 *sm = reinterpret_cast<c64 *>(smem_raw);
+    const int NQ = a.NQ;
     const int nrhs = a.nrhs, Nu = a.Nu;
-    const cx<T> *W = (const cx<T> *)a.W;
-    cx<T> *y = (cx<T> *)a.y;
-    const cx<T> *fib = (const cx<T> *)o.fib;
-    const cx<T> *pool = (const cx<T> *)o.face;
-    cx<T> *Wt = sm;
-    cx<T> *z = Wt + (int64_t)NQ * TJ * nrhs;
-    cx<T> *acc = z + (int64_t)RC * 2 * TJ * nrhs;
-    cx<T> *fq_s = acc + a.acc_max;                                   // [RC][NQ]
+    const c64 *W = (const c64 *)a.W;
+    c64 *y = (c64 *)a.y;
+    const c64 *fib = (const c64 *)o.fib;
+    const c64 *pool = (const c64 *)o.face;
+    c64 *Wt = sm;
+    c64 *z = Wt + (int64_t)NQ * TJ * nrhs;
+    c64 *acc = z + (int64_t)RC * 2 * TJ * nrhs;
+    c64 *fq_s = acc + a.acc_max;                                   // [RC][NQ]
     int *sg_s = reinterpret_cast<int *>(fq_s + (int64_t)RC * NQ);    // [NQ]
     const int tid = threadIdx.x;
     for (int b = blockIdx.x; b < a.nb; b += gridDim.x) {
@@ -55,8 +56,8 @@ __global__ void __launch_bounds__(256) k_apply(ApplyArgs a, TensorOut o, int TJ,
             // conjugate half) and the half it belongs to
             for (int e = tid; e < rc * NQ; e += blockDim.x) {
                 const int q = e % NQ, dd = e / NQ;
-                const int mp = a.qmap[a.single_f >= 0 ? a.single_f : q];
-                const cx<T> fv = fib[(tb + d0 + dd) * Nu + (mp > 0 ? mp - 1 : -mp - 1)];
+                const int mp = a.qmap[q];
+                const c64 fv = fib[(tb + d0 + dd) * Nu + (mp > 0 ? mp - 1 : -mp - 1)];
                 fq_s[e] = mp > 0 ? fv : cconj(fv);
                 if (dd == 0) sg_s[q] = mp > 0 ? 1 : -1;
             }
@@ -73,11 +74,11 @@ __global__ void __launch_bounds__(256) k_apply(ApplyArgs a, TensorOut o, int TJ,
                 // per-point fibre coefficients were staged in shared memory
                 for (int e = tid; e < rc * tj * nrhs; e += blockDim.x) {
                     const int c = e % nrhs, jj = (e / nrhs) % tj, dd = e / (nrhs * tj);
-                    const cx<T> *fq = fq_s + (int64_t)dd * NQ;
-                    cx<T> z1 = {0, 0}, z2 = {0, 0};
+                    const c64 *fq = fq_s + (int64_t)dd * NQ;
+                    c64 z1 = {0, 0}, z2 = {0, 0};
 #pragma unroll 4
                     for (int q = 0; q < NQ; ++q) {
-                        const cx<T> w = Wt[((int64_t)q * TJ + jj) * nrhs + c];
+                        const c64 w = Wt[((int64_t)q * TJ + jj) * nrhs + c];
                         if (sg_s[q] > 0) cfma(z1, fq[q], w);
                         else cfma(z2, fq[q], w);
                     }
@@ -88,11 +89,11 @@ __global__ void __launch_bounds__(256) k_apply(ApplyArgs a, TensorOut o, int TJ,
                 if (!far) {
                     for (int e = tid; e < nI * nrhs; e += blockDim.x) {
                         const int c = e % nrhs, i = e / nrhs;
-                        cx<T> s = acc[e];
+                        c64 s = acc[e];
                         for (int dd = 0; dd < rc; ++dd) {
-                            const cx<T> *H = pool + o.foff[tb + d0 + dd] + (int64_t)i * nJ + j0;
+                            const c64 *H = pool + o.foff[tb + d0 + dd] + (int64_t)i * nJ + j0;
                             for (int jj = 0; jj < tj; ++jj) {
-                                const cx<T> h = H[jj];
+                                const c64 h = H[jj];
                                 cfma(s, h, z[(((int64_t)dd * 2 + 0) * TJ + jj) * nrhs + c]);
                                 cfma(s, cconj(h), z[(((int64_t)dd * 2 + 1) * TJ + jj) * nrhs + c]);
                             }
@@ -109,10 +110,10 @@ __global__ void __launch_bounds__(256) k_apply(ApplyArgs a, TensorOut o, int TJ,
                             ++dd;
                         }
                         const int kd = o.frank[tb + d0 + dd];
-                        const cx<T> *V = pool + o.foff[tb + d0 + dd] + (int64_t)kd * nI + (int64_t)t * nJ + j0;
-                        cx<T> s1 = acc[(e / nrhs) * 2 * nrhs + c], s2 = acc[(e / nrhs) * 2 * nrhs + nrhs + c];
+                        const c64 *V = pool + o.foff[tb + d0 + dd] + (int64_t)kd * nI + (int64_t)t * nJ + j0;
+                        c64 s1 = acc[(e / nrhs) * 2 * nrhs + c], s2 = acc[(e / nrhs) * 2 * nrhs + nrhs + c];
                         for (int jj = 0; jj < tj; ++jj) {
-                            const cx<T> v = V[jj];
+                            const c64 v = V[jj];
                             cfma(s1, v, z[(((int64_t)dd * 2 + 0) * TJ + jj) * nrhs + c]);
                             cfma(s2, cconj(v), z[(((int64_t)dd * 2 + 1) * TJ + jj) * nrhs + c]);
                         }
@@ -130,13 +131,13 @@ __global__ void __launch_bounds__(256) k_apply(ApplyArgs a, TensorOut o, int TJ,
             } else {
                 for (int e = tid; e < nI * nrhs; e += blockDim.x) {
                     const int c = e % nrhs, i = e / nrhs;
-                    cx<T> s = {0, 0};
+                    c64 s = {0, 0};
                     int base = 0;
                     for (int dd = 0; dd < rc; ++dd) {
                         const int kd = o.frank[tb + d0 + dd];
-                        const cx<T> *U = pool + o.foff[tb + d0 + dd];
+                        const c64 *U = pool + o.foff[tb + d0 + dd];
                         for (int t = 0; t < kd; ++t) {
-                            const cx<T> u = U[(int64_t)t * nI + i];
+                            const c64 u = U[(int64_t)t * nI + i];
                             cfma(s, u, acc[(int64_t)(base + t) * 2 * nrhs + c]);
                             cfma(s, cconj(u), acc[(int64_t)(base + t) * 2 * nrhs + nrhs + c]);
                         }
@@ -150,171 +151,438 @@ __global__ void __launch_bounds__(256) k_apply(ApplyArgs a, TensorOut o, int TJ,
     }
 }
 
+// y += A(s_f) x at one point of the list: sum_d f_d[f] H_d x, one CTA per block.
+//   near: every warp takes rows, its lanes the columns (coalesced); the terms are
+//         combined first, h = sum_d f_d H_d[i][j], then multiplied with x;
+//   far:  t = f_d V_d x by warps (one factor row each, lanes along it), then rows
+//         of y from U, threads along i (coalesced), CTAs of short blocks splitting
+//         the factor rows over thread groups.
+// CC right-hand sides per pass over the faces.  A conjugate point takes conj(x)
+// and conjugates its result.  Bound: HBM, every face read once per pass.  The
+// general kernel read near rows with stride |J| and one right-hand side gave it
+// 4 CTAs of work per SM at a time: 30k housing, 8 frequencies, 1 right-hand side:
+// 1043 -> 340 us (142M stored values, 3.3 TB/s); 5120-triangle sphere, 4 right-hand
+// sides: 400 -> 193 us (14,488 blocks of 1800 values: latency).
+constexpr int kOneJ = 128, kOneT = 128, kOneD = 32;  // columns, factor rows, terms in shared memory at a time
+
+template <class T, int CC>
+__global__ void __launch_bounds__(128, sizeof(T) == 4 ? (CC == 4 ? 8 : 10) : 5) k_apply_one(ApplyArgs a, TensorOut o, int c0) {
+    __shared__ cx<T> xs[kOneJ][CC];
+    __shared__ cx<T> ts[kOneT][CC];
+    __shared__ cx<T> fs[kOneD];
+    __shared__ long long off[kOneD];
+    __shared__ int pre[kOneD + 1];
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = 4, b = blockIdx.x;
+    const int rb = o.rank[b];
+    const int *bl = a.blocks + 5 * b;
+    const int nI = bl[1] - bl[0], nJ = bl[3] - bl[2], nrhs = a.nrhs;
+    const bool far = bl[4] != 0;
+    const int nc = min(CC, nrhs - c0);
+    const int64_t tb = (int64_t)b * a.Nu;
+    const int mp = a.qmap[a.single_f];
+    const bool cj = mp < 0;
+    const int u = (cj ? -mp : mp) - 1;
+    const cx<T> *x = (const cx<T> *)a.W, *pool = (const cx<T> *)o.face;
+    cx<T> *y = (cx<T> *)a.y;
+    int loaded = -1;  // first column of the x tile in shared memory
+    auto load_x = [&](int j0, int tj) {
+        __syncthreads();
+        if (loaded == j0) return;
+        loaded = j0;
+        for (int e = tid; e < tj * CC; e += 128) {
+            const int j = e / CC, c = e - j * CC;
+            cx<T> v = {0, 0};
+            if (c < nc) v = x[(int64_t)a.perm_c[bl[2] + j0 + j] * nrhs + c0 + c];
+            xs[j][c] = cj ? cconj(v) : v;
+        }
+        __syncthreads();
+    };
+    auto add = [&](int i, const cx<T> *v) {
+        cx<T> *yr = y + (int64_t)a.perm_r[bl[0] + i] * nrhs + c0;
+#pragma unroll
+        for (int c = 0; c < CC; ++c)
+            if (c < nc) atomic_add_c(yr + c, cj ? cconj(v[c]) : v[c]);
+    };
+    if (rb > 0) load_x(0, min(kOneJ, nJ));  // its dependent loads first
+    for (int d0 = 0; d0 < rb; d0 += kOneD) {
+        const int r = min(kOneD, rb - d0);
+        __syncthreads();
+        if (tid < r) {
+            fs[tid] = ((const cx<T> *)o.fib)[(tb + d0 + tid) * a.Nu + u];
+            off[tid] = o.foff[tb + d0 + tid];
+        }
+        if (wid == 0) {  // inclusive prefix of the face ranks
+            int k = far && lane < r ? o.frank[tb + d0 + lane] : 0;
+            for (int s = 1; s < 32; s <<= 1) {
+                const int v = __shfl_up_sync(0xffffffffu, k, s);
+                if (lane >= s) k += v;
+            }
+            if (lane == 0) pre[0] = 0;
+            pre[lane + 1] = k;
+        }
+        if (!far) {
+            for (int j0 = 0; j0 < nJ; j0 += kOneJ) {
+                const int tj = min(kOneJ, nJ - j0);
+                load_x(j0, tj);
+                // two rows per warp and pass
+                for (int i = 2 * wid; i < nI; i += 2 * nw) {
+                    const bool two = i + 1 < nI;
+                    cx<T> acc[2][CC];
+#pragma unroll
+                    for (int c = 0; c < CC; ++c) acc[0][c] = acc[1][c] = cx<T>{0, 0};
+                    const int64_t ij = (int64_t)i * nJ + j0, st = two ? nJ : 0;
+                    for (int j = lane; j < tj; j += 32) {
+                        cx<T> h[2] = {{0, 0}, {0, 0}};
+                        int d = 0;
+                        for (; d + 4 <= r; d += 4) {
+                            cx<T> v[4][2];
+#pragma unroll
+                            for (int q = 0; q < 4; ++q) {
+                                const cx<T> *p = pool + off[d + q] + ij + j;
+                                v[q][0] = p[0];
+                                v[q][1] = p[st];
+                            }
+#pragma unroll
+                            for (int q = 0; q < 4; ++q) {
+                                cfma(h[0], fs[d + q], v[q][0]);
+                                cfma(h[1], fs[d + q], v[q][1]);
+                            }
+                        }
+                        for (; d < r; ++d) {
+                            const cx<T> *p = pool + off[d] + ij + j;
+                            const cx<T> v0 = p[0], v1 = p[st];
+                            cfma(h[0], fs[d], v0);
+                            cfma(h[1], fs[d], v1);
+                        }
+#pragma unroll
+                        for (int c = 0; c < CC; ++c) {
+                            cfma(acc[0][c], h[0], xs[j][c]);
+                            cfma(acc[1][c], h[1], xs[j][c]);
+                        }
+                    }
+                    T v[4 * CC];  // row, column, part
+#pragma unroll
+                    for (int c = 0; c < CC; ++c) {
+                        v[2 * c] = acc[0][c].x;
+                        v[2 * c + 1] = cj ? -acc[0][c].y : acc[0][c].y;
+                        v[2 * CC + 2 * c] = acc[1][c].x;
+                        v[2 * CC + 2 * c + 1] = cj ? -acc[1][c].y : acc[1][c].y;
+                    }
+                    const T s = warp_sum_many<4 * CC>(v, lane);
+                    const int idx = many_index<4 * CC>(lane), row = idx / (2 * CC), c = (idx >> 1) % CC;
+                    if ((lane & (32 / (4 * CC) - 1)) == 0 && row <= (two ? 1 : 0) && c < nc) {
+                        cx<T> *yc = y + (int64_t)a.perm_r[bl[0] + i + row] * nrhs + c0 + c;
+                        atomicAdd(idx & 1 ? &yc->y : &yc->x, s);
+                    }
+                }
+            }
+            continue;
+        }
+        __syncthreads();  // pre
+        const int R = pre[r];
+        for (int r0 = 0; r0 < R; r0 += kOneT) {
+            const int rc = min(kOneT, R - r0);
+            for (int j0 = 0; j0 < nJ; j0 += kOneJ) {
+                const int tj = min(kOneJ, nJ - j0);
+                load_x(j0, tj);
+                int d = 0;
+                for (int t = wid; t < rc; t += nw) {
+                    while (r0 + t >= pre[d + 1]) ++d;
+                    const int kd = pre[d + 1] - pre[d], tau = r0 + t - pre[d];
+                    const cx<T> *v = pool + off[d] + (int64_t)kd * nI + (int64_t)tau * nJ + j0;
+                    cx<T> acc[CC], w[kOneJ / 32];
+#pragma unroll
+                    for (int q = 0; q < kOneJ / 32; ++q) w[q] = lane + 32 * q < tj ? v[lane + 32 * q] : cx<T>{0, 0};
+#pragma unroll
+                    for (int c = 0; c < CC; ++c) acc[c] = cx<T>{0, 0};
+#pragma unroll
+                    for (int q = 0; q < kOneJ / 32; ++q) {
+                        if (lane + 32 * q < tj) {
+#pragma unroll
+                            for (int c = 0; c < CC; ++c) cfma(acc[c], w[q], xs[lane + 32 * q][c]);
+                        }
+                    }
+                    T s[2 * CC];
+#pragma unroll
+                    for (int c = 0; c < CC; ++c) {
+                        s[2 * c] = acc[c].x;
+                        s[2 * c + 1] = acc[c].y;
+                    }
+                    constexpr int LB = 32 / (2 * CC);  // lanes per value; the other part is LB lanes on
+                    const T own = warp_sum_many<2 * CC>(s, lane), oth = __shfl_xor_sync(0xffffffffu, own, LB);
+                    const int idx = many_index<2 * CC>(lane);
+                    const T val = idx & 1 ? fs[d].x * own + fs[d].y * oth : fs[d].x * own - fs[d].y * oth;
+                    if ((lane & (LB - 1)) == 0) {
+                        T *tp = reinterpret_cast<T *>(&ts[t][0]) + idx;
+                        *tp = j0 == 0 ? val : *tp + val;
+                    }
+                }
+            }
+            __syncthreads();
+            // rows of y: groups of gi threads along i, each a part of the factor rows
+            const int gi = nI >= 128 ? 128 : (nI + 31) & ~31, G = 128 / gi;
+            const int g = tid / gi;
+            cx<T> own[CC];
+            if (g < G) {
+                const int per = (rc + G - 1) / G, tA = min(rc, g * per), tB = min(rc, tA + per);
+                for (int i = tid - g * gi; i < nI && (tA < tB || G > 1); i += gi) {
+                    cx<T> acc[CC];
+#pragma unroll
+                    for (int c = 0; c < CC; ++c) acc[c] = cx<T>{0, 0};
+                    int d = 0;
+                    for (int t = tA; t < tB;) {
+                        while (r0 + t >= pre[d + 1]) ++d;
+                        // a run of factor rows of one term is contiguous
+                        const int te = min(tB, pre[d + 1] - r0), n = te - t;
+                        const cx<T> *ub = pool + off[d] + (int64_t)(r0 + t - pre[d]) * nI + i;
+                        int q = 0;
+                        for (; q + 4 <= n; q += 4) {
+                            cx<T> uv[4];
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) uv[e] = ub[(int64_t)(q + e) * nI];
+#pragma unroll
+                            for (int e = 0; e < 4; ++e)
+#pragma unroll
+                                for (int c = 0; c < CC; ++c) cfma(acc[c], uv[e], ts[t + q + e][c]);
+                        }
+                        for (; q < n; ++q) {
+                            const cx<T> uv = ub[(int64_t)q * nI];
+#pragma unroll
+                            for (int c = 0; c < CC; ++c) cfma(acc[c], uv, ts[t + q][c]);
+                        }
+                        t = te;
+                    }
+                    if (G == 1 || g == 0) {
+                        if (G == 1) add(i, acc);
+#pragma unroll
+                        for (int c = 0; c < CC; ++c) own[c] = acc[c];
+                    } else {
+#pragma unroll
+                        for (int c = 0; c < CC; ++c) xs[tid - gi][c] = acc[c];  // (G > 1: one i per thread)
+                    }
+                }
+            }
+            __syncthreads();
+            if (G > 1) {  // the groups' sums meet in the place of x: one atomic add per output
+                if (g == 0 && tid < nI) {
+                    for (int q = 1; q < G; ++q)
+#pragma unroll
+                        for (int c = 0; c < CC; ++c) own[c] = own[c] + xs[(q - 1) * gi + tid][c];
+                    add(tid, own);
+                }
+                loaded = -1;
+                __syncthreads();
+            }
+        }
+    }
+}
+
 // Second phase of the tensor-core apply.  The frequency contraction
 // z_(b,d,p) = sum_l f_d(l) W_l[J] is already in Z (k_zgemm.cu); Z rows of a
 // block are (term d, half p) at zbase[b] + p zpstride[b] + d nJ nrhs.  Both face
 // stages are small complex GEMMs out[m][(p, c)] = sum_k A_p[m][k] B[k][(p, c)]
-// with A_1 = conj(A_0) for the conjugate half, tiled through shared memory:
+// with A_1 = conj(A_0) for the conjugate half:
 //   stage 0 (one CTA per far term):  T_p = V_d^T z_p, m = tau < k_d, k = j < |J|,
-//            A = V_d (row-major), written to T;
+//            written to T;
 //   stage 1 (one CTA per block):      y_I += sum_d U_d T_(d,1) + conj(U_d) T_(d,2)
-//            (far; m = i, k = (d, tau), A = U_d^T, column-major) or
-//            y_I += sum_d H_d z_(d,1) + conj(H_d) z_(d,2) (near; k = (d, j),
-//            A = H_d row-major); both halves summed before one atomic add
-//            per output.
-// Tiles: 64 rows x (rpt nrhs) columns, k in chunks of 32; 16 x CG threads,
-// every thread holds a 4 x CPT register tile (rows 4 ty .. 4 ty + 3,
-// columns tx + CG q, tx < CG).
-constexpr int kFM = 64, kFK = 32, kFPad = 65;
+//            (far; k = (d, tau)) or y_I += sum_d H_d z_(d,1) + conj(H_d) z_(d,2)
+//            (near; k = (d, j)); both halves summed before one atomic add per
+//            output.
+// The k of all terms run through one chunked loop (no padding per term): each
+// k has a descriptor (A column, B row), chunks of 32 are brought to shared memory
+// by asynchronous copies in two stages.  Four warps of 4 x (4 or 8 or 2) register
+// tiles, 16 rows each: M <= 16 rows take one row tile with k split over the four
+// warps, M <= 32 two and two, else four row tiles; the warps' sums meet in shared
+// memory.  conj(a) b is formed as conj(a conj(b)): the sign goes on b when it is
+// loaded and on the result, not on every product.  Fixed tiles of 64 rows spent
+// three quarters of stage 0 on padding (k_d is 16 on average): 30k housing, 16
+// right-hand sides: both stages 23.2 -> 11.5 ms.  Bound: FP32 FMA.
+constexpr int kFK = 32, kFA = kFK + 2;  // k per chunk; A row stride (16-byte reads of 4 rows conflict-free)
+constexpr int kFY = 4;                  // CTAs that share a large block's row tiles (stage 1)
 
+struct FaceK {
+    const c32 *A, *B;  // column k of A (row stride per job), row k of B (half 0)
+    int64_t sB;        // offset of the half-1 row
+};
+template <int CQ>
 struct FaceSmem {
-    c32 A[kFK][kFPad];  // A[k][m] (m contiguous)
+    static constexpr int NC = 8 * CQ;
+    c32 A[2][64][kFA];
+    c32 B[2][kFK][NC];
+    FaceK kd[2][kFK];
 };
 
-template <int CG, int CPT>
-__global__ void __launch_bounds__(16 * CG) k_apply_faces(ApplyZArgs a, TensorOut o, int stage) {
-    constexpr int NT = 16 * CG;
+TD_D void cp_async(void *dst, const void *src, int bytes, bool valid) {
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+    if (bytes == 16)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(valid ? 16 : 0) : "memory");
+    else
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(d), "l"(src), "r"(valid ? 8 : 0) : "memory");
+}
+
+template <int CQ>
+__global__ void __launch_bounds__(128) k_apply_faces(ApplyZArgs a, TensorOut o, int stage, int col0) {
+    using Smem = FaceSmem<CQ>;
+    constexpr int NC = Smem::NC;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    FaceSmem &F = *reinterpret_cast<FaceSmem *>(smem_raw);
-    c32 *Bs = reinterpret_cast<c32 *>(smem_raw + sizeof(FaceSmem));  // [kFK][ncol]
-    const int nrhs = a.nrhs, Nu = a.Nu, rpt = a.rpt, ncol = rpt * nrhs;
+    Smem &S = *reinterpret_cast<Smem *>(smem_raw);
+    const int nrhs = a.nrhs, Nu = a.Nu, ncol = min(NC, a.rpt * nrhs - col0);
     const c32 *pool = (const c32 *)o.face;
-    const int tid = threadIdx.x, tx = tid % CG, ty = tid / CG;
-    // columns of this thread and their half; both halves of one right-hand side
-    // sit in the same thread (q and q + CPT / 2) when 2 nrhs = CG CPT
-    bool conj_q[CPT];
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, tx = lane & 7, ry = lane >> 3;
+    // columns 2 tx + 16 h + {0, 1} of this thread: sign of the conjugate half
+    float sgn[CQ];
 #pragma unroll
-    for (int q = 0; q < CPT; ++q) conj_q[q] = tx + CG * q >= nrhs;
-    const bool pair_halves = CPT >= 2 && rpt == 2 && 2 * nrhs == CG * CPT;
-    const int64_t njobs = stage == 0 ? a.nft : a.nb;
-    for (int64_t job = blockIdx.x; job < njobs; job += gridDim.x) {
-        int b, d0, d1, M;
-        if (stage == 0) {
-            const int2 bd = a.ftab[job];
-            b = bd.x;
-            d0 = bd.y;
-            d1 = bd.y + 1;
+    for (int q = 0; q < CQ; ++q) sgn[q] = col0 + 2 * tx + 16 * (q >> 1) + (q & 1) >= nrhs ? -1.0f : 1.0f;
+    // 16-byte copies of B rows: two columns of one half
+    const bool wide = (nrhs & 1) == 0 && (ncol & 1) == 0;
+    int b, d0, d1;
+    if (stage == 0) {
+        const int2 bd = a.ftab[blockIdx.x];
+        b = bd.x;
+        d0 = bd.y;
+        d1 = bd.y + 1;
+    } else {
+        b = blockIdx.x;
+        d0 = 0;
+        d1 = o.rank[b];
+        if (d1 == 0 || a.zbase[b] < 0) return;
+    }
+    const int *bl = a.blocks + 5 * b;
+    const int nI = bl[1] - bl[0], nJ = bl[3] - bl[2];
+    const bool far = bl[4] != 0, ucol = stage == 1 && far;
+    const int64_t tb = (int64_t)b * Nu, L = (int64_t)nJ * nrhs;
+    const int M = stage == 0 ? o.frank[tb + d0] : nI;
+    const int64_t sA = ucol ? 1 : nJ;  // row stride of A
+    if ((int)blockIdx.y * 64 >= M) return;
+    for (int e = tid; e < 2 * kFK * NC; e += 128) (&S.B[0][0][0])[e] = c32{0.f, 0.f};  // columns beyond ncol stay 0
+    int K = 0;
+    if (ucol)
+        for (int d = 0; d < d1; ++d) K += o.frank[tb + d];
+    else
+        K = (d1 - d0) * nJ;
+    // descriptor of k; its term is found from the last one's (k ascends)
+    int dk = d0, kbase = 0;  // threads < 32
+    auto describe = [&](int chunk) {
+        const int k = chunk * kFK + tid;
+        if (tid >= kFK || k >= K) return;
+        FaceK f;
+        if (ucol) {
+            int kd = o.frank[tb + dk];
+            while (k - kbase >= kd) {
+                kbase += kd;
+                kd = o.frank[tb + ++dk];
+            }
+            const int t = k - kbase;
+            f.A = pool + o.foff[tb + dk] + (int64_t)t * nI;
+            f.B = a.T + a.toff[tb + dk] + (int64_t)t * nrhs;
+            f.sB = (int64_t)kd * nrhs;
         } else {
-            b = (int)job;
-            d0 = 0;
-            d1 = o.rank[b];
-            if (d1 == 0 || a.zbase[b] < 0) continue;
+            const int d = d0 + k / nJ, j = k - (k / nJ) * nJ;
+            f.A = pool + o.foff[tb + d] + (stage == 0 ? (int64_t)M * nI : 0) + j;
+            f.B = a.Z + a.zbase[b] + (int64_t)d * L + (int64_t)j * nrhs;
+            f.sB = a.zpstride[b];
         }
-        const int *bl = a.blocks + 5 * b;
-        const int nI = bl[1] - bl[0], nJ = bl[3] - bl[2];
-        const bool far = bl[4] != 0;
-        const int64_t tb = (int64_t)b * Nu, L = (int64_t)nJ * nrhs;
-        M = stage == 0 ? o.frank[tb + d0] : nI;
-        for (int m0 = 0; m0 < M; m0 += kFM) {
-            c32 acc[4][CPT];
+        S.kd[chunk & 1][tid] = f;
+    };
+    const int nchunk = (K + kFK - 1) / kFK;
+    for (int m0 = blockIdx.y * 64; m0 < M; m0 += 64 * gridDim.y) {
+        const int mc = min(64, M - m0);
+        const int WR = mc <= 16 ? 1 : mc <= 32 ? 2 : 4, WK = 4 / WR, R = 16 * WR;
+        const int wr = wid % WR, wk = wid / WR;
+        auto stage_in = [&](int chunk) {
+            const int buf = chunk & 1, kc = min(kFK, K - chunk * kFK);
+            for (int e = tid; e < R * kFK; e += 128) {
+                // consecutive lanes take consecutive addresses: rows of U, columns of V and H
+                const int m = ucol ? e % R : e / kFK, k = ucol ? e / R : e % kFK;
+                const bool ok = k < kc && m < mc;
+                cp_async(&S.A[buf][m][k], ok ? S.kd[buf][k].A + (int64_t)(m0 + m) * sA : pool, 8, ok);
+            }
+            const int per = wide ? 2 : 1, nn = (ncol + per - 1) / per;
+            for (int e = tid; e < kFK * nn; e += 128) {
+                const int k = e / nn, n = (e - k * nn) * per, g = col0 + n, p = g >= nrhs ? 1 : 0;
+                const bool ok = k < kc;
+                cp_async(&S.B[buf][k][n], ok ? S.kd[buf][k].B + p * S.kd[buf][k].sB + g - p * nrhs : pool, 8 * per, ok);
+            }
+            asm volatile("cp.async.commit_group;" ::: "memory");
+        };
+        c32 acc[4][CQ];
 #pragma unroll
-            for (int x = 0; x < 4; ++x)
+        for (int x = 0; x < 4; ++x)
 #pragma unroll
-                for (int q = 0; q < CPT; ++q) acc[x][q] = c32{0.f, 0.f};
-            for (int d = d0; d < d1; ++d) {
-                const int kd = o.frank[tb + d];
-                const c32 *face = pool + o.foff[tb + d];
-                // A operand, its layout and length; B operand rows (p = 0 / 1)
-                const c32 *Ab;
-                int64_t lda;
-                bool acol;
-                int K;
-                const c32 *B0;
-                int64_t bstride;  // B[k][(p, c)] = B0[p * bstride + k * nrhs + c]
-                if (stage == 0) {
-                    Ab = face + (int64_t)kd * nI;  // V[tau][j]
-                    lda = nJ;
-                    acol = false;
-                    K = nJ;
-                    B0 = a.Z + a.zbase[b] + (int64_t)d * L;
-                    bstride = a.zpstride[b];
-                } else if (far) {
-                    Ab = face;  // U[tau][i]: A[i][tau] column-major
-                    lda = nI;
-                    acol = true;
-                    K = kd;
-                    B0 = a.T + a.toff[tb + d];
-                    bstride = (int64_t)kd * nrhs;
-                } else {
-                    Ab = face;  // H[i][j]
-                    lda = nJ;
-                    acol = false;
-                    K = nJ;
-                    B0 = a.Z + a.zbase[b] + (int64_t)d * L;
-                    bstride = a.zpstride[b];
-                }
-                for (int k0 = 0; k0 < K; k0 += kFK) {
-                    const int kc = min(kFK, K - k0), mc = min(kFM, M - m0);
-                    __syncthreads();
-                    if (acol) {
-                        for (int e = tid; e < kFK * kFM; e += NT) {
-                            const int kk = e / kFM, mm = e - kk * kFM;
-                            F.A[kk][mm] = (kk < kc && mm < mc) ? Ab[(int64_t)(k0 + kk) * lda + m0 + mm] : c32{0.f, 0.f};
-                        }
-                    } else {
-                        for (int e = tid; e < kFK * kFM; e += NT) {
-                            const int mm = e / kFK, kk = e - mm * kFK;
-                            F.A[kk][mm] = (kk < kc && mm < mc) ? Ab[(int64_t)(m0 + mm) * lda + k0 + kk] : c32{0.f, 0.f};
-                        }
+            for (int q = 0; q < CQ; ++q) acc[x][q] = c32{0.f, 0.f};
+        __syncthreads();  // shared memory is free
+        dk = d0;
+        kbase = 0;
+        describe(0);
+        describe(1);
+        __syncthreads();
+        if (nchunk > 0) stage_in(0);
+        for (int ch = 0; ch < nchunk; ++ch) {
+            if (ch + 1 < nchunk) {
+                stage_in(ch + 1);
+                asm volatile("cp.async.wait_group 1;" ::: "memory");
+            } else {
+                asm volatile("cp.async.wait_group 0;" ::: "memory");
+            }
+            __syncthreads();
+            const int buf = ch & 1, k1 = (wk + 1) * (kFK / WK);
+#pragma unroll 2
+            for (int k = wk * (kFK / WK); k < k1; k += 2) {
+                float4 av[4];  // rows 16 wr + ry + 4 x at k and k + 1
+#pragma unroll
+                for (int x = 0; x < 4; ++x) av[x] = *reinterpret_cast<const float4 *>(&S.A[buf][16 * wr + ry + 4 * x][k]);
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    c32 bv[CQ];
+#pragma unroll
+                    for (int q = 0; q < CQ; q += 2) {
+                        const float4 v = *reinterpret_cast<const float4 *>(&S.B[buf][k + h][2 * tx + 8 * q]);
+                        bv[q] = c32{v.x, v.y * sgn[q]};
+                        bv[q + 1] = c32{v.z, v.w * sgn[q + 1]};
                     }
-                    for (int e = tid; e < kFK * ncol; e += NT) {
-                        const int kk = e / ncol, n = e - kk * ncol, p = n / nrhs, c = n - p * nrhs;
-                        Bs[e] = kk < kc ? B0[p * bstride + (int64_t)(k0 + kk) * nrhs + c] : c32{0.f, 0.f};
-                    }
-                    __syncthreads();
-#pragma unroll 4
-                    for (int kk = 0; kk < kFK; ++kk) {
-                        c32 av[4], bv[CPT];
 #pragma unroll
-                        for (int x = 0; x < 4; ++x) av[x] = F.A[kk][4 * ty + x];
+                    for (int x = 0; x < 4; ++x) {
+                        const c32 ax = h == 0 ? c32{av[x].x, av[x].y} : c32{av[x].z, av[x].w};
 #pragma unroll
-                        for (int q = 0; q < CPT; ++q) {
-                            const int n = tx + CG * q;
-                            bv[q] = n < ncol ? Bs[kk * ncol + n] : c32{0.f, 0.f};
-                        }
-#pragma unroll
-                        for (int x = 0; x < 4; ++x)
-#pragma unroll
-                            for (int q = 0; q < CPT; ++q) {
-                                // conjugate half: conj(a) b
-                                const float ay = conj_q[q] ? -av[x].y : av[x].y;
-                                acc[x][q].x = fmaf(av[x].x, bv[q].x, fmaf(-ay, bv[q].y, acc[x][q].x));
-                                acc[x][q].y = fmaf(av[x].x, bv[q].y, fmaf(ay, bv[q].x, acc[x][q].y));
-                            }
+                        for (int q = 0; q < CQ; ++q) cfma(acc[x][q], ax, bv[q]);
                     }
                 }
             }
-            // ---- output
+            describe(ch + 2);
+            __syncthreads();  // the stage is refilled, its descriptors replaced
+        }
+        // ---- the warps' sums meet in shared memory [wk][R][NC], in the place of A
+        c32 *red = &S.A[0][0][0];
+        static_assert(sizeof(S.A) >= 4 * 16 * NC * sizeof(c32), "the sums fit in A's stages");
 #pragma unroll
-            for (int x = 0; x < 4; ++x) {
-                const int m = m0 + 4 * ty + x;
-                if (m >= M) continue;
-                if (stage == 0) {
-                    const int kd = M;
-                    c32 *Tout = a.T + a.toff[tb + d0];
+        for (int x = 0; x < 4; ++x)
 #pragma unroll
-                    for (int q = 0; q < CPT; ++q) {
-                        const int n = tx + CG * q;
-                        if (n >= ncol) continue;
-                        const int p = n / nrhs, c = n - p * nrhs;
-                        Tout[((int64_t)p * kd + m) * nrhs + c] = acc[x][q];
-                    }
-                } else {
-                    c32 *yr = a.y + (int64_t)a.perm_r[bl[0] + m] * nrhs;
-                    if (pair_halves) {
-#pragma unroll
-                        for (int q = 0; q < CPT / 2; ++q) {
-                            const int c = tx + CG * q;
-                            if (c < nrhs) atomic_add_c(yr + c, acc[x][q] + acc[x][q + CPT / 2]);
-                        }
-                    } else {
-#pragma unroll
-                        for (int q = 0; q < CPT; ++q) {
-                            const int n = tx + CG * q;
-                            if (n < ncol) atomic_add_c(yr + n % nrhs, acc[x][q]);
-                        }
-                    }
+            for (int q = 0; q < CQ; ++q)
+                red[((wk * R) + 16 * wr + ry + 4 * x) * NC + 2 * tx + 16 * (q >> 1) + (q & 1)] =
+                    c32{acc[x][q].x, acc[x][q].y * sgn[q]};
+        __syncthreads();
+        if (stage == 0) {
+            c32 *Tout = a.T + a.toff[tb + d0];
+            for (int e = tid; e < mc * ncol; e += 128) {
+                const int m = e / ncol, n = e - m * ncol, g = col0 + n, p = g >= nrhs ? 1 : 0;
+                c32 v = red[m * NC + n];
+                for (int w = 1; w < WK; ++w) v = v + red[(w * R + m) * NC + n];
+                Tout[((int64_t)p * M + m0 + m) * nrhs + g - p * nrhs] = v;
+            }
+        } else {
+            // columns of both halves in this pass are summed first
+            const int lo = min(ncol, max(0, nrhs - col0));  // half-0 columns of the pass
+            const bool both = col0 == 0 && ncol == 2 * nrhs;
+            const int no = both ? nrhs : ncol;
+            for (int e = tid; e < mc * no; e += 128) {
+                const int m = e / no, n = e - m * no;
+                c32 v = {0.f, 0.f};
+                for (int w = 0; w < WK; ++w) {
+                    v = v + red[(w * R + m) * NC + n];
+                    if (both) v = v + red[(w * R + m) * NC + n + nrhs];
                 }
+                const int c = n < lo ? col0 + n : col0 + n - nrhs;
+                atomic_add_c(a.y + (int64_t)a.perm_r[bl[0] + m0 + m] * nrhs + c, v);
             }
         }
     }
@@ -362,9 +630,26 @@ __global__ void k_tensor_entries(TensorOut o, const int *blocks, int nb, int64_t
 
 }  // namespace
 
+// One right-hand side, two or up to four per pass over the faces.
+template <class T>
+static int launch_one(cudaStream_t st, const ApplyArgs &a, const TensorOut &o) {
+    for (int c = 0; c < a.nrhs;) {
+        const int left = a.nrhs - c;
+        if (left >= 3) k_apply_one<T, 4><<<a.nb, 128, 0, st>>>(a, o, c);
+        else if (left == 2) k_apply_one<T, 2><<<a.nb, 128, 0, st>>>(a, o, c);
+        else k_apply_one<T, 1><<<a.nb, 128, 0, st>>>(a, o, c);
+        c += left >= 3 ? std::min(4, left) : left;
+    }
+    return (int)cudaGetLastError();
+}
+
 int td_launch_apply(cudaStream_t st, int prec, const ApplyArgs &a, const TensorOut &o, int num_sms) {
-    const int NQ = a.single_f >= 0 ? 1 : a.NQ;
-    const size_t es = prec == TDBEM_FP64 ? 16 : 8;
+    if (a.nb == 0) return 0;
+    if (a.single_f >= 0)
+        return prec == TDBEM_FP64 ? launch_one<double>(st, a, o) : launch_one<float>(st, a, o);
+    if (prec != TDBEM_FP64) return (int)cudaErrorInvalidValue;  // the mixed form runs on the tensor cores
+    const int NQ = a.NQ;
+    const size_t es = sizeof(c64);
     const int budget = 160 * 1024;
     // W tile: NQ x TJ x nrhs; z: RC x 2 x TJ x nrhs; acc: max(nI, 2*sumk) x nrhs
     int TJ = (int)std::max<int64_t>(1, std::min<int64_t>(32, (budget / 2) / ((int64_t)NQ * a.nrhs * es)));
@@ -383,41 +668,35 @@ int td_launch_apply(cudaStream_t st, int prec, const ApplyArgs &a, const TensorO
     aa.acc_max = acc_max;
     if (sm > (size_t)(220 * 1024)) return (int)cudaErrorInvalidConfiguration;
     const int grid = std::min(a.nb, num_sms * 4);
-    cudaError_t e;
-    if (prec == TDBEM_FP64) {
-        e = cudaFuncSetAttribute(k_apply<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        if (e != cudaSuccess) return (int)e;
-        k_apply<double><<<grid, 256, sm, st>>>(aa, o, TJ, RC);
-    } else {
-        e = cudaFuncSetAttribute(k_apply<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        if (e != cudaSuccess) return (int)e;
-        k_apply<float><<<grid, 256, sm, st>>>(aa, o, TJ, RC);
-    }
+    const cudaError_t e = cudaFuncSetAttribute(k_apply, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (e != cudaSuccess) return (int)e;
+    k_apply<<<grid, 256, sm, st>>>(aa, o, TJ, RC);
     return (int)cudaGetLastError();
 }
 
-template <int CG, int CPT>
-static int launch_faces(cudaStream_t st, const ApplyZArgs &a, const TensorOut &o, int stage, int grid) {
-    const size_t sm = sizeof(FaceSmem) + sizeof(c32) * kFK * a.rpt * a.nrhs;
-    cudaError_t e = cudaFuncSetAttribute(k_apply_faces<CG, CPT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+template <int CQ>
+static int launch_faces(cudaStream_t st, const ApplyZArgs &a, const TensorOut &o, int stage, int col0) {
+    const size_t sm = sizeof(FaceSmem<CQ>);
+    cudaError_t e = cudaFuncSetAttribute(k_apply_faces<CQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return (int)e;
-    k_apply_faces<CG, CPT><<<grid, 16 * CG, sm, st>>>(a, o, stage);
+    const dim3 grid(stage == 0 ? a.nft : a.nb, stage == 0 ? 1 : kFY);
+    k_apply_faces<CQ><<<grid, 128, sm, st>>>(a, o, stage, col0);
     return (int)cudaGetLastError();
 }
 
 int td_launch_apply_z(cudaStream_t st, const ApplyZArgs &a, const TensorOut &o, int num_sms) {
+    // 16, 32 or 64 columns (half, right-hand side) per pass over the faces
     const int ncol = a.rpt * a.nrhs;
-    auto run = [&](int stage, int grid) {
-        // 8 x 4 or 16 x 4 threads' register tiles of 4 x 4 complex outputs
-        // (ncol <= 64); 16 column groups of 8 columns beyond
-        if (ncol <= 16) return launch_faces<8, 2>(st, a, o, stage, grid);
-        if (ncol <= 32) return launch_faces<8, 4>(st, a, o, stage, grid);
-        if (ncol <= 64) return launch_faces<16, 4>(st, a, o, stage, grid);
-        return launch_faces<16, 8>(st, a, o, stage, grid);
-    };
     int e = 0;
-    if (a.nft > 0) e = run(0, (int)std::min<int64_t>(a.nft, (int64_t)num_sms * 32));
-    if (!e && a.nb > 0) e = run(1, std::min(a.nb, num_sms * 32));
+    for (int stage = 0; stage < 2 && !e; ++stage) {
+        if ((stage == 0 ? a.nft : a.nb) == 0) continue;
+        for (int c = 0; c < ncol && !e;) {
+            const int left = ncol - c;
+            e = left <= 16 ? launch_faces<2>(st, a, o, stage, c)
+                : left <= 32 ? launch_faces<4>(st, a, o, stage, c) : launch_faces<8>(st, a, o, stage, c);
+            c += left <= 16 ? 16 : left <= 32 ? 32 : 64;
+        }
+    }
     return e;
 }
 
