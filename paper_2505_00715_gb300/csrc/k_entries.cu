@@ -308,16 +308,21 @@ __global__ void k_sing_table(MeshDev m, const int *pti, const int *ptj, int npai
 // reused by every frequency, FC frequencies per pass; each pass's lane sums
 // are reduced over the warp and added to the pair's table rows.  The reference
 // points come from an array formed once per call (k_ss_rule): a point then takes
-// 18 FP64 operations instead of about 100 (30k housing: 65 -> 43 ms; bound by FP32
-// issue, 24 instructions per point and frequency, and by the FP64 pipe).
+// 18 FP64 operations instead of about 100, and the chunk sums meet in shared memory
+// (the table was read and written once per pass, a memory latency each).  30k
+// housing: 65 -> 43 -> 33 ms; 5120-triangle sphere, double layer: 15.7 -> 6.4 ms.
+// Bound by FP32 issue, 24 instructions per point and frequency, and by the FP64 pipe.
 template <int OP, int FC>
-__global__ void k_sing_table_mixed(MeshDev m, const int *pti, const int *ptj, int npairs, const double *rule,
+__global__ void __launch_bounds__(128, 4) k_sing_table_mixed(MeshDev m, const int *pti, const int *ptj, int npairs, const double *rule,
                                    const double *sig, int nf, const int *klist, int nd, c64 *table) {
     const int lane = threadIdx.x & 31;
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int nwarps = (gridDim.x * blockDim.x) >> 5;
     constexpr int NV = TD_P1_TRIAL(OP) ? 3 : 1;
     constexpr int P = TD_P1_TRIAL(OP) ? 8 : 16;  // points per lane and chunk
+    // the warp's table rows, FP64 (dynamic: 4 warps x nd x NV)
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    double *rows = reinterpret_cast<double *>(smem_raw) + (int64_t)(threadIdx.x >> 5) * nd * NV * 2;
     // s / c of every frequency in shared memory (nd <= nf <= 256, checked by the caller)
     __shared__ float2 s_sig[256];
     for (int k = threadIdx.x; k < nd; k += blockDim.x)
@@ -336,9 +341,13 @@ __global__ void k_sing_table_mixed(MeshDev m, const int *pti, const int *ptj, in
         const int nq = ss_npoints(G.cls, m.ng);
         const bool zero = (OP != TD_SLP && G.cls == 3) || G.cls == 0;
         c64 *o = table + (int64_t)p * nf * NV;
-        for (int e = lane; e < nd * NV; e += 32) o[(int64_t)klist[e / NV] * NV + e % NV] = c64{0.0, 0.0};
+        if (zero) {
+            for (int e = lane; e < nd * NV; e += 32) o[(int64_t)klist[e / NV] * NV + e % NV] = c64{0.0, 0.0};
+            continue;
+        }
         __syncwarp();
-        if (zero) continue;
+        for (int e = lane; e < nd * NV * 2; e += 32) rows[e] = 0.0;
+        __syncwarp();
         SsEdges E;
         ss_edges(G, E);
         const double *rl = rule + ss_rule_off(G.cls, m.ng);
@@ -395,20 +404,28 @@ __global__ void k_sing_table_mixed(MeshDev m, const int *pti, const int *ptj, in
                         }
                     }
                 }
-                // lane sums over the warp in FP32, chunk sums into the FP64 table
+                // lane sums over the warp in FP32 (NS sums, padded to a power of two), chunk
+                // sums into the FP64 rows by the lanes that hold them
+                constexpr int NS = FC * NV * 2, NP = NS <= 4 ? 4 : NS <= 8 ? 8 : NS <= 16 ? 16 : 32;
 #pragma unroll
-                for (int j = 0; j < FC; ++j) {
+                for (int c0 = 0; c0 < NS; c0 += NP) {
+                    float v[NP];
 #pragma unroll
-                    for (int k = 0; k < NV; ++k) {
-                        const float sx = warp_sum(acc[j][k].x), sy = warp_sum(acc[j][k].y);
-                        if (lane == 0 && f0 + j < nd) {
-                            c64 &t = o[(int64_t)klist[f0 + j] * NV + (TD_P1_TRIAL(OP) ? G.loc[k] : 0)];
-                            t.x += (double)sx * inv4pi;
-                            t.y += (double)sy * inv4pi;
-                        }
+                    for (int q = 0; q < NP; ++q) {
+                        const int t = c0 + q, j = t / (2 * NV), kk = t / 2 % NV;
+                        v[q] = t >= NS ? 0.0f : t & 1 ? acc[j][kk].y : acc[j][kk].x;
                     }
+                    const float sum = warp_sum_many<NP>(v, lane);
+                    const int t = c0 + many_index<NP>(lane), j = t / (2 * NV);
+                    if ((lane & (32 / NP - 1)) == 0 && t < NS && f0 + j < nd)
+                        rows[(f0 + j) * NV * 2 + t % (2 * NV)] += (double)sum * inv4pi;
                 }
             }
+        }
+        __syncwarp();
+        for (int e = lane; e < nd * NV; e += 32) {
+            const int v = e % NV;
+            o[(int64_t)klist[e / NV] * NV + (TD_P1_TRIAL(OP) ? G.loc[v] : 0)] = c64{rows[2 * e], rows[2 * e + 1]};
         }
     }
 }
@@ -575,20 +592,19 @@ int td_launch_sing_table(cudaStream_t st, const MeshDev &m, int op, int prec, co
     int grid = std::min((npairs + 3) / 4, num_sms * 8);
     if (prec == TDBEM_MIXED) {
         const int v = variant % 3;
-        if (op == TD_SLP) {
-            if (v == 1) k_sing_table_mixed<TD_SLP, 8><<<grid, 128, 0, st>>>(m, pti, ptj, npairs, rule, sig, nf, klist, nd, table);
-            else if (v == 2) k_sing_table_mixed<TD_SLP, 16><<<grid, 128, 0, st>>>(m, pti, ptj, npairs, rule, sig, nf, klist, nd, table);
-            else k_sing_table_mixed<TD_SLP, 4><<<grid, 128, 0, st>>>(m, pti, ptj, npairs, rule, sig, nf, klist, nd, table);
-        } else if (op == TD_DLP) {
-            if (v == 1) k_sing_table_mixed<TD_DLP, 4><<<grid, 128, 0, st>>>(m, pti, ptj, npairs, rule, sig, nf, klist, nd, table);
-            else if (v == 2) k_sing_table_mixed<TD_DLP, 8><<<grid, 128, 0, st>>>(m, pti, ptj, npairs, rule, sig, nf, klist, nd, table);
-            else k_sing_table_mixed<TD_DLP, 2><<<grid, 128, 0, st>>>(m, pti, ptj, npairs, rule, sig, nf, klist, nd, table);
-        } else {
-            if (v == 1) k_sing_table_mixed<TD_ADLP, 8><<<grid, 128, 0, st>>>(m, pti, ptj, npairs, rule, sig, nf, klist, nd, table);
-            else if (v == 2) k_sing_table_mixed<TD_ADLP, 16><<<grid, 128, 0, st>>>(m, pti, ptj, npairs, rule, sig, nf, klist, nd, table);
-            else k_sing_table_mixed<TD_ADLP, 4><<<grid, 128, 0, st>>>(m, pti, ptj, npairs, rule, sig, nf, klist, nd, table);
-        }
-        return (int)cudaGetLastError();
+        const size_t sm = sizeof(c64) * 4 * nd * (op == TD_DLP ? 3 : 1);
+        cudaError_t e = cudaSuccess;
+        auto run = [&](auto kernel) {
+            e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+            if (e == cudaSuccess) kernel<<<grid, 128, sm, st>>>(m, pti, ptj, npairs, rule, sig, nf, klist, nd, table);
+        };
+        if (op == TD_SLP)
+            run(v == 1 ? k_sing_table_mixed<TD_SLP, 8> : v == 2 ? k_sing_table_mixed<TD_SLP, 16> : k_sing_table_mixed<TD_SLP, 4>);
+        else if (op == TD_DLP)
+            run(v == 1 ? k_sing_table_mixed<TD_DLP, 4> : v == 2 ? k_sing_table_mixed<TD_DLP, 8> : k_sing_table_mixed<TD_DLP, 2>);
+        else
+            run(v == 1 ? k_sing_table_mixed<TD_ADLP, 8> : v == 2 ? k_sing_table_mixed<TD_ADLP, 16> : k_sing_table_mixed<TD_ADLP, 4>);
+        return e != cudaSuccess ? (int)e : (int)cudaGetLastError();
     }
     if (op == TD_SLP)
         k_sing_table<TD_SLP, 8><<<grid, 128, 0, st>>>(m, pti, ptj, npairs, sig, nf, klist, nd, table);
