@@ -40,7 +40,23 @@ TD_D cx<T> coef_sum(const cx<T> *coef, const cx<T> *const *base, int cn, int idx
 #pragma unroll
         for (int q = 0; q < 8; ++q) cfma(acc[q & 3], coef[c + q], b[q]);
     }
-    for (; c < cn; ++c) cfma(acc[0], coef[c], base[c][idx]);
+    if (c + 4 <= cn) {  // the remainder's loads in flight together as well
+        cx<T> b[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) b[q] = base[c + q][idx];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) cfma(acc[0], coef[c + q], b[q]);
+        c += 4;
+    }
+    if (c < cn) {
+        cx<T> b[3] = {};
+#pragma unroll
+        for (int q = 0; q < 3; ++q)
+            if (c + q < cn) b[q] = base[c + q][idx];
+#pragma unroll
+        for (int q = 0; q < 3; ++q)
+            if (c + q < cn) cfma(acc[0], coef[c + q], b[q]);
+    }
     return (acc[0] + acc[1]) + (acc[2] + acc[3]);
 }
 template <class T>
@@ -770,8 +786,8 @@ TD_D void cp_async_wait() {
 // of KC factor columns are staged in shared memory (the Gram tiles' space)
 // in two stages, the next chunk's asynchronous copies in flight while the
 // current one is multiplied; every thread accumulates a 4 x 4 register tile:
-// rows 4*ty .. 4*ty+3 and columns tx, tx+16, tx+32, tx+48 (8 shared loads
-// per 16 complex MACs, conflict-free).  Entries are summed over t in the
+// rows 4*ty .. 4*ty+3 and columns 2 tx, 2 tx + 1, 2 tx + 32, 2 tx + 33 (four 16-byte
+// shared loads per 16 complex MACs, conflict-free).  Entries are summed over t in the
 // same order as the plain rebuild.  Dense-face blocks also store the face to
 // Sd.
 template <int NT>
@@ -823,9 +839,14 @@ TD_D void rebuild_tiled(void *smem, const c32 *Uw, const c32 *Vw, int64_t maxI, 
                 for (int t = 0; t < kc; ++t) {
                     c32 u[4], v[4];
 #pragma unroll
-                    for (int x = 0; x < 4; ++x) u[x] = su[t * TI + 4 * ty + x];
-#pragma unroll
-                    for (int y = 0; y < 4; ++y) v[y] = sv[t * TJ + tx + 16 * y];
+                    for (int x = 0; x < 4; x += 2) {
+                        const float4 p = *reinterpret_cast<const float4 *>(su + t * TI + 4 * ty + x);
+                        const float4 q = *reinterpret_cast<const float4 *>(sv + t * TJ + 2 * tx + 16 * x);
+                        u[x] = c32{p.x, p.y};
+                        u[x + 1] = c32{p.z, p.w};
+                        v[x] = c32{q.x, q.y};
+                        v[x + 1] = c32{q.z, q.w};
+                    }
 #pragma unroll
                     for (int x = 0; x < 4; ++x)
 #pragma unroll
@@ -838,7 +859,7 @@ TD_D void rebuild_tiled(void *smem, const c32 *Uw, const c32 *Vw, int64_t maxI, 
                 const int i = i0 + 4 * ty + x;
 #pragma unroll
                 for (int y = 0; y < 4; ++y) {
-                    const int j = j0 + tx + 16 * y;
+                    const int j = j0 + 2 * tx + 32 * (y >> 1) + (y & 1);
                     if (i >= nI || j >= nJ) continue;
                     const int e = i * nJ + j;
                     if (Sd) Sd[e] = h[x][y];
@@ -879,7 +900,24 @@ TD_D cx<T> dense_prev(const cx<T> *Hs, int64_t ds, const cx<T> *coef, int l, int
 #pragma unroll
         for (int q = 0; q < 8; ++q) cfma(a4[q & 3], coef[d + q], h[q]);
     }
-    for (; d < l; ++d) cfma(a4[d & 3], coef[d], Hs[(int64_t)d * ds + e]);
+    // the remainder's loads in flight together as well
+    if (d + 4 <= l) {
+        cx<T> h[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) h[q] = Hs[(int64_t)(d + q) * ds + e];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) cfma(a4[q], coef[d + q], h[q]);
+        d += 4;
+    }
+    if (d < l) {
+        cx<T> h[3] = {};
+#pragma unroll
+        for (int q = 0; q < 3; ++q)
+            if (d + q < l) h[q] = Hs[(int64_t)(d + q) * ds + e];
+#pragma unroll
+        for (int q = 0; q < 3; ++q)
+            if (d + q < l) cfma(a4[q], coef[d + q], h[q]);
+    }
     return (a4[0] + a4[1]) + (a4[2] + a4[3]);
 }
 
@@ -900,32 +938,71 @@ TD_D cx<T> own_sum(const cx<T> *X, int64_t sx, int fixed, const cx<T> *Y, int64_
 #pragma unroll
         for (int q = 0; q < 8; ++q) cfma(a4[q & 3], xv[q], yv[q]);
     }
-    for (; t < kf; ++t) cfma(a4[t & 3], X[(int64_t)t * sx + fixed], Y[(int64_t)t * sy + idx]);
+    // the remainder's loads in flight together as well
+    if (t + 4 <= kf) {
+        cx<T> xv[4], yv[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            xv[q] = X[(int64_t)(t + q) * sx + fixed];
+            yv[q] = Y[(int64_t)(t + q) * sy + idx];
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) cfma(a4[q], xv[q], yv[q]);
+        t += 4;
+    }
+    if (t < kf) {
+        cx<T> xv[3] = {}, yv[3] = {};
+#pragma unroll
+        for (int q = 0; q < 3; ++q)
+            if (t + q < kf) {
+                xv[q] = X[(int64_t)(t + q) * sx + fixed];
+                yv[q] = Y[(int64_t)(t + q) * sy + idx];
+            }
+#pragma unroll
+        for (int q = 0; q < 3; ++q)
+            if (t + q < kf) cfma(a4[q], xv[q], yv[q]);
+    }
     return (a4[0] + a4[1]) + (a4[2] + a4[3]);
 }
 
-// sum_{i < n} x[i] conj(y[i]) over the lanes of a warp (each lane its part;
-// the caller sums over the warp), four pairs of loads in flight per lane.
+// out[q] = sum_{i < n} x[i] conj(y_q[i]) over the lanes of a warp (each lane its
+// part; the caller sums over the warp) for two vectors y_0, y_1, four elements of
+// each in flight per lane.
 template <class T>
-TD_D DotAcc<T> lane_dot(const cx<T> *x, const cx<T> *y, int n, int lane) {
-    DotAcc<T> a, b;
+TD_D void lane_dot2(const cx<T> *x, const cx<T> *y0, const cx<T> *y1, int n, int lane, DotAcc<T> *out) {
+    DotAcc<T> s0, s1;
     int i = lane;
     for (; i + 96 < n; i += 128) {
-        cx<T> xv[4], yv[4];
+        cx<T> xv[4], u[4], v[4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            xv[u] = x[i + 32 * u];
-            yv[u] = y[i + 32 * u];
+        for (int q = 0; q < 4; ++q) {
+            xv[q] = x[i + 32 * q];
+            u[q] = y0[i + 32 * q];
+            v[q] = y1[i + 32 * q];
         }
-        a.add(xv[0], yv[0]);
-        b.add(xv[1], yv[1]);
-        a.add(xv[2], yv[2]);
-        b.add(xv[3], yv[3]);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            s0.add(xv[q], u[q]);
+            s1.add(xv[q], v[q]);
+        }
     }
-    for (; i < n; i += 32) a.add(x[i], y[i]);
-    a.re += b.re;
-    a.im += b.im;
-    return a;
+    if (i < n) {
+        cx<T> xv[4], u[4], v[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const bool ok = i + 32 * q < n;
+            xv[q] = ok ? x[i + 32 * q] : cx<T>{0, 0};
+            u[q] = ok ? y0[i + 32 * q] : cx<T>{0, 0};
+            v[q] = ok ? y1[i + 32 * q] : cx<T>{0, 0};
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            s0.add(xv[q], u[q]);
+            s1.add(xv[q], v[q]);
+        }
+    }
+    out[0] = s0;
+    out[1] = s1;
 }
 
 // eq. norm's <H_l, H_d> for every d <= l (< kDenseTerms) from the dense
@@ -936,19 +1013,24 @@ TD_D void dense_grams(const cx<T> *Hs, int l, int64_t nIJ, AccT<T> *gH) {
     DotAcc<T> acc[kDenseTerms];
     const cx<T> *Hl = Hs + (int64_t)l * nIJ;
     const int64_t st = blockDim.x;
-    // four entries per thread and pass: four loads in flight per face
+    // four entries per thread and pass, two faces at a time: eight loads in flight
     for (int64_t e0 = threadIdx.x; e0 < nIJ; e0 += 4 * st) {
         cx<T> h[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) h[u] = e0 + u * st < nIJ ? Hl[e0 + u * st] : cx<T>{0, 0};
 #pragma unroll
-        for (int d = 0; d < kDenseTerms; ++d) {
+        for (int d = 0; d < kDenseTerms; d += 2) {
             if (d > l) break;
-            cx<T> g[4];
+            cx<T> g[2][4];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) g[u] = e0 + u * st < nIJ ? Hs[(int64_t)d * nIJ + e0 + u * st] : cx<T>{0, 0};
+            for (int v = 0; v < 2; ++v)
 #pragma unroll
-            for (int u = 0; u < 4; ++u) acc[d].add(h[u], g[u]);
+                for (int u = 0; u < 4; ++u)
+                    g[v][u] = d + v <= l && e0 + u * st < nIJ ? Hs[(int64_t)(d + v) * nIJ + e0 + u * st] : cx<T>{0, 0};
+#pragma unroll
+            for (int v = 0; v < 2; ++v)
+#pragma unroll
+                for (int u = 0; u < 4; ++u) acc[d + v].add(h[u], g[v][u]);
         }
     }
 #pragma unroll
@@ -1028,9 +1110,19 @@ __global__ void __launch_bounds__(NT, 640 / NT) k_far_aca(MeshDev m, FarArgs a, 
             if (small && !cdm)
                 for (int d = tid; d < l; d += blockDim.x) Q.coef[d] = fib[(tb + d) * Nu + k];
             if (cdm) {
+                for (int d = tid; d < l; d += blockDim.x) F.hd[d] = fib[(tb + d) * Nu + k];
+                __syncthreads();
                 for (int e = tid; e < nI * nJ; e += blockDim.x) {
                     cx<T> acc = {0, 0};
-                    for (int d = 0; d < l; ++d) cfma(acc, fib[(tb + d) * Nu + k], Hs[(int64_t)d * nIJb + e]);
+                    for (int d = 0; d < l; d += 4) {  // four faces' loads in flight
+                        cx<T> h[4] = {};
+#pragma unroll
+                        for (int q = 0; q < 4; ++q)
+                            if (d + q < l) h[q] = Hs[(int64_t)(d + q) * nIJb + e];
+#pragma unroll
+                        for (int q = 0; q < 4; ++q)
+                            if (d + q < l) cfma(acc, F.hd[d + q], h[q]);
+                    }
                     Cd[e] = acc;
                     if (dense_s) Ss[e] = cx<T>{0, 0};
                 }
@@ -1274,25 +1366,31 @@ __global__ void __launch_bounds__(NT, 640 / NT) k_far_aca(MeshDev m, FarArgs a, 
                 ++ev_tests;
                 __syncthreads();
                 {
-                    int npairs = 0;
-                    for (int t = pend0; t <= kf; ++t) npairs += t + 1;
-                    for (int pr = wid; pr < npairs; pr += nwarps) {
-                        int t = pend0, rem = pr;
-                        while (rem >= t + 1) {
-                            rem -= t + 1;
+                    // one warp per pair (t, t2 <= t), two pairs of one t at a time
+                    int t = pend0, t2 = 2 * wid;
+                    for (;;) {
+                        while (t <= kf && t2 > t) {
+                            t2 -= (t + 2) & ~1;
                             ++t;
                         }
-                        const int t2 = rem;
-                        const DotAcc<T> au = lane_dot(Uw + (int64_t)t * a.maxI, Uw + (int64_t)t2 * a.maxI, nI, lane);
-                        const DotAcc<T> av = lane_dot(Vw + (int64_t)t * a.maxJ, Vw + (int64_t)t2 * a.maxJ, nJ, lane);
-                        const A ur = au.warp_re(), vr = av.warp_re();
-                        if (t2 < t) {
-                            const A ui = au.warp_im(), vi = av.warp_im();
-                            if (lane == 0) atomicAdd(&S.nrow[t], ur * vr - ui * vi);
-                        } else if (lane == 0) {
-                            S.nu[t] = ur;
-                            S.nv[t] = vr;
+                        if (t > kf) break;
+                        const int tb2 = min(t2 + 1, t);
+                        DotAcc<T> au[2], av[2];
+                        lane_dot2(Uw + (int64_t)t * a.maxI, Uw + (int64_t)t2 * a.maxI, Uw + (int64_t)tb2 * a.maxI, nI, lane, au);
+                        lane_dot2(Vw + (int64_t)t * a.maxJ, Vw + (int64_t)t2 * a.maxJ, Vw + (int64_t)tb2 * a.maxJ, nJ, lane, av);
+#pragma unroll
+                        for (int q = 0; q < 2; ++q) {
+                            if (t2 + q > t) continue;
+                            const A ur = au[q].warp_re(), vr = av[q].warp_re();
+                            if (t2 + q < t) {
+                                const A ui = au[q].warp_im(), vi = av[q].warp_im();
+                                if (lane == 0) atomicAdd(&S.nrow[t], ur * vr - ui * vi);
+                            } else if (lane == 0) {
+                                S.nu[t] = ur;
+                                S.nv[t] = vr;
+                            }
                         }
+                        t2 += 2 * nwarps;
                     }
                 }
                 __syncthreads();
