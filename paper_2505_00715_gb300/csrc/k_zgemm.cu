@@ -19,8 +19,14 @@
 // (256 FP32 TMEM columns); K is consumed in chunks of 32 complex values
 // (64 real = 4 MMAs of K = 16 per split term).  Two CTAs of 256 threads per
 // SM (the operand tiles take 96 KB of shared memory and 256 TMEM columns per
-// CTA), so that one CTA's operand loads overlap the other's MMAs; tiles are
-// taken from a job list in a persistent loop.  Used by the weighted apply (the
+// CTA), so that one CTA's operand splitting overlaps the other's MMAs, and a
+// CTA loads the next chunk to registers while its own MMAs run; tiles are
+// taken from a job list in a persistent loop.  Bound by moving the operands
+// (a load, a split and two shared stores per value) and writing D, not by the
+// MMAs.  Stage 1 of the apply of a 30k-element SLP operator (16 right-hand
+// sides): 11.3 -> 5.1 ms, of 5120 elements 1.77 -> 0.52 ms, of 1280 elements
+// 55 -> 28 us, against loads between the MMAs and rows of D stored 8 bytes a
+// lane.  Used by the weighted apply (the
 // frequency contraction of eq. product) and exposed for testing as
 // tdbem_zgemm.
 #include <cuda_bf16.h>
@@ -153,92 +159,87 @@ __global__ void __launch_bounds__(kThreads, 2) k_zgemm(Ops ops, const ZJob *jobs
         const int mr = ops.rows(job), nc = ops.cols(job);
         int kb, ke;
         ops.krange(job, K, kb, ke);
-        for (int k0 = kb; k0 < ke && !failed; k0 += kTK) {
+        // Operand items of a chunk (8 consecutive complex k of one row of A or column of
+        // B), two of each per thread, loaded to registers while the MMAs of the chunk
+        // before run.  Real item it of the canonical layout is at byte 16 * it: A item ci
+        // -> (kstep ci >> 8, row group (ci >> 4) & 15, core matrix (ci >> 3) & 1, row
+        // ci & 7), B item ci -> (kstep ci >> 8, row group (ci >> 3) & 31, core matrix
+        // (ci >> 2) & 1, column ci & 3 of the group's four).
+        constexpr int kAItems = kTM * kTK / 8, kBItems = kTN * kTK / 8;
+        static_assert(kAItems == 2 * kThreads && kBItems == 2 * kThreads, "two items of each operand per thread");
+        c32 xa[2][8], xb[2][8];
+        auto load_chunk = [&](int k0) {
             const int kc = min(kTK, ke - k0);
-            // ---- A tile.  Real item it -> (kstep s, row group g, core matrix kh, row
-            // rr), its 16 bytes at byte offset 16 * it of the canonical layout.  One
-            // complex item (8 consecutive complex k of one row) gives the real item of
-            // its real parts (real k < kTK) and the one of its imaginary parts (real
-            // k + kTK, kTK / 16 ksteps = kTK * 16 items further): each value is loaded
-            // once.  Two complex items per thread and pass, loads issued first.
-            constexpr int kAItems = kTM * kTK / 8, kAImag = kTK * 16;
-            for (int c0 = tid; c0 < kAItems; c0 += 2 * kThreads) {
-                c32 x[2][8];
 #pragma unroll
-                for (int u = 0; u < 2; ++u) {
-                    const int ci = c0 + u * kThreads;
-                    const int rr = ci & 7, kh = (ci >> 3) & 1, g = (ci >> 4) & 15, sk = ci >> 8;
-                    const int r = g * 8 + rr, k = sk * 16 + kh * 8;  // complex k of the first element
-                    if (ci < kAItems && r < mr) {
-                        ops.a8(job, job.m0 + r, k0 + k, k0 + kc, x[u]);
-                    } else {
+            for (int u = 0; u < 2; ++u) {
+                const int ci = tid + u * kThreads;
+                const int r = ((ci >> 4) & 15) * 8 + (ci & 7), ka = (ci >> 8) * 16 + ((ci >> 3) & 1) * 8;
+                if (r < mr) {
+                    ops.a8(job, job.m0 + r, k0 + ka, k0 + kc, xa[u]);
+                } else {
 #pragma unroll
-                        for (int e = 0; e < 8; ++e) x[u][e] = c32{0.f, 0.f};
-                    }
-                }
-#pragma unroll
-                for (int u = 0; u < 2; ++u) {
-                    const int ci = c0 + u * kThreads;
-                    if (ci >= kAItems) continue;
-                    float v[8];
-#pragma unroll
-                    for (int e = 0; e < 8; ++e) v[e] = x[u][e].x;
-                    SplitPack p = split8(v);
-                    *reinterpret_cast<uint4 *>(Ah + 16 * ci) = p.hi;
-                    *reinterpret_cast<uint4 *>(Al + 16 * ci) = p.lo;
-#pragma unroll
-                    for (int e = 0; e < 8; ++e) v[e] = x[u][e].y;
-                    p = split8(v);
-                    *reinterpret_cast<uint4 *>(Ah + 16 * (ci + kAImag)) = p.hi;
-                    *reinterpret_cast<uint4 *>(Al + 16 * (ci + kAImag)) = p.lo;
+                    for (int e = 0; e < 8; ++e) xa[u][e] = c32{0.f, 0.f};
                 }
             }
-            // ---- B tile: 2 kTN real rows (re / im row of every complex column).
-            // Real item it -> (kstep s = it >> 9, row group g, kh, row rr).  One
-            // complex item (8 consecutive k of complex column n) gives four real
-            // items: rows 2n / 2n + 1 (rr = 2 (n & 3), + 1) in the first K half
-            // (Re B, Im B) and in the second (-Im B, Re B, kTK / 16 ksteps further).
-            constexpr int kBItems = kTN * kTK / 8, kBSecond = kTK * 32;
-            for (int c0 = tid; c0 < kBItems; c0 += 2 * kThreads) {
-                c32 x[2][8];
 #pragma unroll
-                for (int u = 0; u < 2; ++u) {
-                    const int ci = c0 + u * kThreads;
-                    const int n4 = ci & 3, kh = (ci >> 2) & 1, g = (ci >> 3) & 31, sk = ci >> 8;
-                    const int n = g * 4 + n4, k = sk * 16 + kh * 8;
-                    if (ci < kBItems && n < nc) {
-                        ops.b8(job, k0 + k, k0 + kc, job.n0 + n, x[u]);
-                    } else {
+            for (int u = 0; u < 2; ++u) {
+                const int ci = tid + u * kThreads;
+                const int n = ((ci >> 3) & 31) * 4 + (ci & 3), kk = (ci >> 8) * 16 + ((ci >> 2) & 1) * 8;
+                if (n < nc) {
+                    ops.b8(job, k0 + kk, k0 + kc, job.n0 + n, xb[u]);
+                } else {
 #pragma unroll
-                        for (int e = 0; e < 8; ++e) x[u][e] = c32{0.f, 0.f};
-                    }
+                    for (int e = 0; e < 8; ++e) xb[u][e] = c32{0.f, 0.f};
                 }
+            }
+        };
+        if (kb < ke) load_chunk(kb);
+        for (int k0 = kb; k0 < ke && !failed; k0 += kTK) {
+            // ---- A tile: the item's real parts (real k < kTK) and its imaginary parts
+            // (kTK / 16 ksteps = kTK * 16 items further)
+            constexpr int kAImag = kTK * 16;
 #pragma unroll
-                for (int u = 0; u < 2; ++u) {
-                    const int ci = c0 + u * kThreads;
-                    if (ci >= kBItems) continue;
-                    const int n4 = ci & 3, kh = (ci >> 2) & 1, g = (ci >> 3) & 31, sk = ci >> 8;
-                    const int it = sk * 512 + g * 16 + kh * 8 + 2 * n4;
-                    float v[8];
-                    SplitPack p;
+            for (int u = 0; u < 2; ++u) {
+                const int ci = tid + u * kThreads;
+                float v[8];
 #pragma unroll
-                    for (int e = 0; e < 8; ++e) v[e] = x[u][e].x;  // row 2n, first half; row 2n + 1, second
-                    p = split8(v);
-                    *reinterpret_cast<uint4 *>(Bh + 16 * it) = p.hi;
-                    *reinterpret_cast<uint4 *>(Bl + 16 * it) = p.lo;
-                    *reinterpret_cast<uint4 *>(Bh + 16 * (it + kBSecond + 1)) = p.hi;
-                    *reinterpret_cast<uint4 *>(Bl + 16 * (it + kBSecond + 1)) = p.lo;
+                for (int e = 0; e < 8; ++e) v[e] = xa[u][e].x;
+                SplitPack p = split8(v);
+                *reinterpret_cast<uint4 *>(Ah + 16 * ci) = p.hi;
+                *reinterpret_cast<uint4 *>(Al + 16 * ci) = p.lo;
 #pragma unroll
-                    for (int e = 0; e < 8; ++e) v[e] = x[u][e].y;  // row 2n + 1, first half
-                    p = split8(v);
-                    *reinterpret_cast<uint4 *>(Bh + 16 * (it + 1)) = p.hi;
-                    *reinterpret_cast<uint4 *>(Bl + 16 * (it + 1)) = p.lo;
+                for (int e = 0; e < 8; ++e) v[e] = xa[u][e].y;
+                p = split8(v);
+                *reinterpret_cast<uint4 *>(Ah + 16 * (ci + kAImag)) = p.hi;
+                *reinterpret_cast<uint4 *>(Al + 16 * (ci + kAImag)) = p.lo;
+            }
+            // ---- B tile: 2 kTN real rows (re / im row of every complex column).  One
+            // complex item gives four real items: rows 2n / 2n + 1 (row 2 (n & 3), + 1 of
+            // the group) in the first K half (Re B, Im B) and in the second (-Im B, Re B,
+            // kTK / 16 ksteps further); a sign change of both parts of the split is exact.
+            constexpr int kBSecond = kTK * 32;
 #pragma unroll
-                    for (int e = 0; e < 8; ++e) v[e] = -x[u][e].y;  // row 2n, second half
-                    p = split8(v);
-                    *reinterpret_cast<uint4 *>(Bh + 16 * (it + kBSecond)) = p.hi;
-                    *reinterpret_cast<uint4 *>(Bl + 16 * (it + kBSecond)) = p.lo;
-                }
+            for (int u = 0; u < 2; ++u) {
+                const int ci = tid + u * kThreads;
+                const int it = (ci >> 8) * 512 + ((ci >> 3) & 31) * 16 + ((ci >> 2) & 1) * 8 + 2 * (ci & 3);
+                float v[8];
+#pragma unroll
+                for (int e = 0; e < 8; ++e) v[e] = xb[u][e].x;  // row 2n, first half; row 2n + 1, second
+                SplitPack p = split8(v);
+                *reinterpret_cast<uint4 *>(Bh + 16 * it) = p.hi;
+                *reinterpret_cast<uint4 *>(Bl + 16 * it) = p.lo;
+                *reinterpret_cast<uint4 *>(Bh + 16 * (it + kBSecond + 1)) = p.hi;
+                *reinterpret_cast<uint4 *>(Bl + 16 * (it + kBSecond + 1)) = p.lo;
+#pragma unroll
+                for (int e = 0; e < 8; ++e) v[e] = xb[u][e].y;  // row 2n + 1, first half; row 2n, second, negated
+                p = split8(v);
+                *reinterpret_cast<uint4 *>(Bh + 16 * (it + 1)) = p.hi;
+                *reinterpret_cast<uint4 *>(Bl + 16 * (it + 1)) = p.lo;
+                const uint32_t sg = 0x80008000u;
+                p.hi = make_uint4(p.hi.x ^ sg, p.hi.y ^ sg, p.hi.z ^ sg, p.hi.w ^ sg);
+                p.lo = make_uint4(p.lo.x ^ sg, p.lo.y ^ sg, p.lo.z ^ sg, p.lo.w ^ sg);
+                *reinterpret_cast<uint4 *>(Bh + 16 * (it + kBSecond)) = p.hi;
+                *reinterpret_cast<uint4 *>(Bl + 16 * (it + kBSecond)) = p.lo;
             }
             fence_async_shared();
             __syncthreads();
@@ -255,6 +256,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_zgemm(Ops ops, const ZJob *jobs
                 }
                 tc_commit(bar);
             }
+            if (k0 + kTK < ke) load_chunk(k0 + kTK);
             // a limit below the default counts non-blocking tests (a blocking
             // try_wait may itself wait until the MMAs are done)
             const bool ok = max_polls < kMaxPolls ? mbar_test(bar, phase, max_polls) : mbar_wait(bar, phase, max_polls);
@@ -263,22 +265,30 @@ __global__ void __launch_bounds__(kThreads, 2) k_zgemm(Ops ops, const ZJob *jobs
             tc_fence_after();
         }
         if (failed) break;
-        // ---- epilogue: warp w reads TMEM lanes 32 (w % 4) .. +31 (tile rows),
-        // real columns 128 (w / 4) .. +127
+        // ---- epilogue: warp w reads TMEM lanes 32 (w % 4) .. +31 (tile rows), real
+        // columns 128 (w / 4) .. +127, 32 complex columns at a time through its part
+        // of the (idle) operand space, so that a row's 256 bytes are stored at once:
+        // a lane per row stored 8 bytes at a time, each a write of its own to L2
         const int q = warp & 3, h = warp >> 2;
-        const int r = 32 * q + lane;
-        c32 *drow = r < mr ? ops.drow(job, job.m0 + r) : nullptr;
+        c32 *buf = reinterpret_cast<c32 *>(base) + warp * 32 * 33;
+        static_assert(8 * 32 * 33 * sizeof(c32) <= 2 * kABytes + 2 * kBBytes, "the epilogue's buffers fit");
 #pragma unroll 1
-        for (int c16 = 0; c16 < 8; ++c16) {
-            const int col = 128 * h + 16 * c16;  // real column of the first value
-            float v[16];
-            tmem_ld16(tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)col, v);
-            const int n0 = col >> 1;  // complex column
-            if (drow) {
+        for (int p = 0; p < 2; ++p) {
+#pragma unroll 1
+            for (int c16 = 0; c16 < 4; ++c16) {
+                const int col = 128 * h + 64 * p + 16 * c16;  // real column of the first value
+                float v[16];
+                tmem_ld16(tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)col, v);
 #pragma unroll
-                for (int e = 0; e < 8; ++e)
-                    if (n0 + e < nc) drow[job.n0 + n0 + e] = c32{v[2 * e], v[2 * e + 1]};
+                for (int e = 0; e < 8; ++e) buf[lane * 33 + 8 * c16 + e] = c32{v[2 * e], v[2 * e + 1]};
             }
+            __syncwarp();
+            const int n = 64 * h + 32 * p + lane, rows = min(32, mr - 32 * q);  // complex column
+            if (n < nc) {
+#pragma unroll 4
+                for (int r = 0; r < rows; ++r) ops.drow(job, job.m0 + 32 * q + r)[job.n0 + n] = buf[r * 33 + lane];
+            }
+            __syncwarp();
         }
         tc_fence_before();
         __syncthreads();
