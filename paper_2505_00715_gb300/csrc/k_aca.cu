@@ -326,17 +326,19 @@ template <int OP>
 TD_D void add_pair(c64 &acc, const QPoint<double> &x, const QPoint<double> &y, const Vec3<double> &n, double hat,
                    double sr, double si) {
     const double dx = y.x - x.x, dy = y.y - x.y, dz = y.z - x.z;
-    const double r = sqrt(dx * dx + dy * dy + dz * dz);
-    const c64 e = expm_sr(sr, si, r);
-    double w = x.w * y.w / r;
+    double ri;
+    const double r = sqrt_inv(dx * dx + dy * dy + dz * dz, ri), px = sr * r, pi = si * r;
+    const ExpParts e = exp_parts(px, pi);
+    double w = x.w * y.w * ri;
+    if (OP == TD_DLP) w *= hat * -(dx * n.x + dy * n.y + dz * n.z) * ri * ri;
+    if (OP == TD_ADLP) w *= (dx * n.x + dy * n.y + dz * n.z) * ri * ri;
+    w *= e.ea;
     if (OP == TD_SLP) {
-        acc = c64{fma(w, e.x, acc.x), fma(w, e.y, acc.y)};
+        acc = c64{fma(w, e.c, acc.x), fma(-w, e.s, acc.y)};
         return;
     }
-    if (OP == TD_DLP) w *= hat * -(dx * n.x + dy * n.y + dz * n.z) / (r * r);
-    else w *= (dx * n.x + dy * n.y + dz * n.z) / (r * r);
-    const double pr = 1.0 + sr * r, pi = si * r;
-    acc = c64{fma(w, pr * e.x - pi * e.y, acc.x), fma(w, pr * e.y + pi * e.x, acc.y)};
+    const double pr = 1.0 + px;
+    acc = c64{fma(w, pr * e.c + pi * e.s, acc.x), fma(w, pi * e.c - pr * e.s, acc.y)};
 }
 TD_D float hat_at(int b, int loc, float) { return bary7f(b, loc); }
 TD_D double hat_at(int b, int loc, double) { return bary7d(b, loc); }

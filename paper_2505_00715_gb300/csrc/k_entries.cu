@@ -48,9 +48,10 @@ template <int OP, int FC>
 TD_D void point_multi(const MeshDev &m, int oa, int ob, double hat, const double *n, const double *sr, const double *si,
                       c64 *acc) {
     const double dx = m.qx[ob] - m.qx[oa], dy = m.qy[ob] - m.qy[oa], dz = m.qz[ob] - m.qz[oa];
-    const double r = sqrt(dx * dx + dy * dy + dz * dz);
-    double w = (TD_P1_TRIAL(OP) ? m.qw[ob] * hat : m.qw[ob]) / r;
-    if (OP != TD_SLP) w *= (dx * n[0] + dy * n[1] + dz * n[2]) / (r * r);
+    double ri;
+    const double r = sqrt_inv(dx * dx + dy * dy + dz * dz, ri);
+    double w = (TD_P1_TRIAL(OP) ? m.qw[ob] * hat : m.qw[ob]) * ri;
+    if (OP != TD_SLP) w *= (dx * n[0] + dy * n[1] + dz * n[2]) * ri * ri;
 #pragma unroll
     for (int j = 0; j < FC; ++j) {
         const c64 e = expm_sr(sr[j], si[j], r);
@@ -85,7 +86,7 @@ TD_D double hat7(int b, int loc, double) { return bary7d(b, loc); }
 // other by all 32 lanes, which split the up to 2 ng^4 Sauter-Schwab points (FP64 in
 // both forms), without it k_entry_sing adds them for all frequencies at once.  One
 // thread per entry left a warp waiting for the lane with the touching pair, 1250
-// points in a row at latency: 320 x 320 x 16 FP64 entries 269 -> 18.1 ms with SING, 11.9 with
+// points in a row at latency: 320 x 320 x 16 FP64 entries 269 -> 18.1 ms with SING, 10.5 with
 // k_entry_sing; 67 x 1801 x 11 double-layer entries 119 -> 6.2 and 3.3 ms.  Bound:
 // the FP64 pipe.
 template <class T, int OP, int FC, bool SING>
@@ -452,9 +453,10 @@ TD_D void pair_multi(const TestD &X, const MeshDev &m, int tj, const double *sg,
 #pragma unroll 1
         for (int a = 0; a < 7; ++a) {
             const double dx = yx - X.x[a], dy = yy - X.y[a], dz = yz - X.z[a];
-            const double r = sqrt(dx * dx + dy * dy + dz * dz);
-            double w = X.w[a] * wyb / r;
-            if (OP != TD_SLP) w *= (dx * nx + dy * ny + dz * nz) / (r * r);
+            double ri;
+            const double r = sqrt_inv(dx * dx + dy * dy + dz * dz, ri);
+            double w = X.w[a] * wyb * ri;
+            if (OP != TD_SLP) w *= (dx * nx + dy * ny + dz * nz) * ri * ri;
 #pragma unroll
             for (int j = 0; j < FC; ++j) {
                 if (j < nfc) {

@@ -116,8 +116,9 @@ TD_D double diff2(const TestD &X, int a, const Point &p, double *d) {
 // w / r (single layer) or w dn / r^3, and r
 template <int OP>
 TD_D double over_r(double w, double dn, double r2, double &r) {
-    r = sqrt(r2);
-    return OP == TD_SLP ? w / r : w * dn / (r * r * r);
+    double ri;
+    r = sqrt_inv(r2, ri);
+    return OP == TD_SLP ? w * ri : w * dn * (ri * ri * ri);
 }
 
 // Adds the moments of test triangle X and trial triangle tj to M: P terms over

@@ -156,11 +156,219 @@ TD_D void load_test(const MeshDev &m, int t, TestD &T) {
     T.nz = m.n64[2 * m.nt + t];
 }
 
+// Tables of expm_sr (FP64): 2^{j/64} rounded to nearest with its relative rounding
+// error, and cos, sin of 2 pi j / 64 with their rounding errors (from 300-bit
+// values).
+static __device__ const double2 c_exp2_64[64] = {
+    {1.0, 0.0},
+    {1.0108892860517005, -1.507066976926039e-17},
+    {1.0218971486541166, 4.9997448722726326e-17},
+    {1.0330248790212284, 7.357846871247418e-18},
+    {1.0442737824274138, 8.189317638195514e-17},
+    {1.0556451783605572, 1.6665881442326747e-18},
+    {1.0671404006768237, -7.402825309426177e-17},
+    {1.0787607977571199, -6.170654745608695e-17},
+    {1.0905077326652577, -2.7939114859515733e-17},
+    {1.102382583307841, 4.776959425256223e-17},
+    {1.1143867425958924, 9.341710609905044e-17},
+    {1.1265216186082418, 4.5856703266623505e-17},
+    {1.1387886347566916, 7.826573258636075e-17},
+    {1.1511892299529827, 2.823784425951061e-17},
+    {1.1637248587775775, 3.2904726646008416e-17},
+    {1.1763969916502812, 4.7213681211701275e-17},
+    {1.189207115002721, 3.3484623336251524e-17},
+    {1.202156731452703, 5.527550048505249e-17},
+    {1.215247359980469, -6.346552106729484e-17},
+    {1.22848053610687, -1.5456342819397733e-17},
+    {1.241857812073484, 3.7508542013031266e-17},
+    {1.255380757024691, -5.346099009198751e-18},
+    {1.2690509571917332, 2.1023049675215714e-18},
+    {1.2828700160787783, 1.3357510088834541e-17},
+    {1.2968395546510096, 1.9572585293112036e-17},
+    {1.3109612115247644, -5.4780691239267786e-17},
+    {1.3252366431597413, -2.1571477251208756e-17},
+    {1.339667524053303, 6.663804589232194e-17},
+    {1.3542555469368927, 5.68648095791174e-17},
+    {1.3690024229745905, 7.007875046906994e-17},
+    {1.383909881963832, -4.8923067513522756e-17},
+    {1.3989796725383112, -6.872303720902018e-17},
+    {1.4142135623730951, -6.835808657661923e-17},
+    {1.42961333839197, -8.416011634717156e-18},
+    {1.4451808069770467, -2.092304381843353e-17},
+    {1.460917794180647, -3.833464968654295e-17},
+    {1.4768261459394993, -2.3591094770850053e-17},
+    {1.4929077282912648, 9.50689710108796e-18},
+    {1.5091644275934228, -6.735219232374683e-17},
+    {1.5255981507445384, -7.226635472101257e-17},
+    {1.5422108254079407, 5.1548301170786783e-17},
+    {1.559004400237837, 2.4253985766689806e-17},
+    {1.5759808451078865, -6.432131775424189e-18},
+    {1.593142151342267, -6.336161863401293e-17},
+    {1.6104903319492543, 1.5341410053603723e-17},
+    {1.6280274218573478, -4.123367330661149e-17},
+    {1.645755478153965, -6.152602891550265e-17},
+    {1.6636765803267364, 3.540948262646183e-17},
+    {1.681792830507429, 4.875160526227061e-17},
+    {1.7001063537185235, -4.719539664590972e-18},
+    {1.718619298122478, -1.0772487078934056e-17},
+    {1.7373338352737062, 1.821405440362259e-17},
+    {1.7562521603732995, 1.685487290628973e-17},
+    {1.7753764925265212, 3.621615935336894e-17},
+    {1.7947090750031072, 1.01562190116415e-17},
+    {1.8142521755003989, -5.495118966122005e-17},
+    {1.8340080864093424, 1.790126907604513e-17},
+    {1.8539791250833855, 5.265370768556274e-17},
+    {1.8741676341103, -3.266924100901318e-17},
+    {1.8945759815869656, 1.7963932659833022e-17},
+    {1.9152065613971474, -5.5450656186394274e-17},
+    {1.9360617934922943, 5.336805878514151e-17},
+    {1.9571441241754002, 4.578491527706009e-17},
+    {1.978456026387951, 2.04142788975783e-17},
+};
+struct alignas(16) Cis64 { double x, y, z, w; };
+static __device__ const Cis64 c_cis_64[64] = {  // cos, sin, errors
+    {1.0, 0.0, 0.0, 0.0},
+    {0.9951847266721969, 0.0980171403295606, -4.248691367830441e-17, -1.634582362244256e-18},
+    {0.9807852804032304, 0.19509032201612828, 1.8546939997825006e-17, -7.991079068461731e-18},
+    {0.9569403357322088, 0.2902846772544624, 4.05538698618757e-17, -1.892797870777425e-17},
+    {0.9238795325112867, 0.3826834323650898, 1.7645047084336677e-17, -1.0050772696461588e-17},
+    {0.881921264348355, 0.47139673682599764, -1.9843248405890562e-17, 6.516678136069013e-18},
+    {0.8314696123025452, 0.5555702330196022, 1.4073856984728024e-18, 4.709410940561677e-17},
+    {0.773010453362737, 0.6343932841636455, -3.256590703364977e-17, 1.0420901929280035e-17},
+    {0.7071067811865476, 0.7071067811865476, -4.833646656726457e-17, -4.833646656726457e-17},
+    {0.6343932841636455, 0.773010453362737, 1.0420901929280035e-17, -3.256590703364977e-17},
+    {0.5555702330196022, 0.8314696123025452, 4.709410940561677e-17, 1.4073856984728024e-18},
+    {0.47139673682599764, 0.881921264348355, 6.516678136069013e-18, -1.9843248405890562e-17},
+    {0.3826834323650898, 0.9238795325112867, -1.0050772696461588e-17, 1.7645047084336677e-17},
+    {0.2902846772544624, 0.9569403357322088, -1.892797870777425e-17, 4.05538698618757e-17},
+    {0.19509032201612828, 0.9807852804032304, -7.991079068461731e-18, 1.8546939997825006e-17},
+    {0.0980171403295606, 0.9951847266721969, -1.634582362244256e-18, -4.248691367830441e-17},
+    {0.0, 1.0, 0.0, 0.0},
+    {-0.0980171403295606, 0.9951847266721969, 1.634582362244256e-18, -4.248691367830441e-17},
+    {-0.19509032201612828, 0.9807852804032304, 7.991079068461731e-18, 1.8546939997825006e-17},
+    {-0.2902846772544624, 0.9569403357322088, 1.892797870777425e-17, 4.05538698618757e-17},
+    {-0.3826834323650898, 0.9238795325112867, 1.0050772696461588e-17, 1.7645047084336677e-17},
+    {-0.47139673682599764, 0.881921264348355, -6.516678136069013e-18, -1.9843248405890562e-17},
+    {-0.5555702330196022, 0.8314696123025452, -4.709410940561677e-17, 1.4073856984728024e-18},
+    {-0.6343932841636455, 0.773010453362737, -1.0420901929280035e-17, -3.256590703364977e-17},
+    {-0.7071067811865476, 0.7071067811865476, 4.833646656726457e-17, -4.833646656726457e-17},
+    {-0.773010453362737, 0.6343932841636455, 3.256590703364977e-17, 1.0420901929280035e-17},
+    {-0.8314696123025452, 0.5555702330196022, -1.4073856984728024e-18, 4.709410940561677e-17},
+    {-0.881921264348355, 0.47139673682599764, 1.9843248405890562e-17, 6.516678136069013e-18},
+    {-0.9238795325112867, 0.3826834323650898, -1.7645047084336677e-17, -1.0050772696461588e-17},
+    {-0.9569403357322088, 0.2902846772544624, -4.05538698618757e-17, -1.892797870777425e-17},
+    {-0.9807852804032304, 0.19509032201612828, -1.8546939997825006e-17, -7.991079068461731e-18},
+    {-0.9951847266721969, 0.0980171403295606, 4.248691367830441e-17, -1.634582362244256e-18},
+    {-1.0, 0.0, 0.0, 0.0},
+    {-0.9951847266721969, -0.0980171403295606, 4.248691367830441e-17, 1.634582362244256e-18},
+    {-0.9807852804032304, -0.19509032201612828, -1.8546939997825006e-17, 7.991079068461731e-18},
+    {-0.9569403357322088, -0.2902846772544624, -4.05538698618757e-17, 1.892797870777425e-17},
+    {-0.9238795325112867, -0.3826834323650898, -1.7645047084336677e-17, 1.0050772696461588e-17},
+    {-0.881921264348355, -0.47139673682599764, 1.9843248405890562e-17, -6.516678136069013e-18},
+    {-0.8314696123025452, -0.5555702330196022, -1.4073856984728024e-18, -4.709410940561677e-17},
+    {-0.773010453362737, -0.6343932841636455, 3.256590703364977e-17, -1.0420901929280035e-17},
+    {-0.7071067811865476, -0.7071067811865476, 4.833646656726457e-17, 4.833646656726457e-17},
+    {-0.6343932841636455, -0.773010453362737, -1.0420901929280035e-17, 3.256590703364977e-17},
+    {-0.5555702330196022, -0.8314696123025452, -4.709410940561677e-17, -1.4073856984728024e-18},
+    {-0.47139673682599764, -0.881921264348355, -6.516678136069013e-18, 1.9843248405890562e-17},
+    {-0.3826834323650898, -0.9238795325112867, 1.0050772696461588e-17, -1.7645047084336677e-17},
+    {-0.2902846772544624, -0.9569403357322088, 1.892797870777425e-17, -4.05538698618757e-17},
+    {-0.19509032201612828, -0.9807852804032304, 7.991079068461731e-18, -1.8546939997825006e-17},
+    {-0.0980171403295606, -0.9951847266721969, 1.634582362244256e-18, 4.248691367830441e-17},
+    {0.0, -1.0, 0.0, 0.0},
+    {0.0980171403295606, -0.9951847266721969, -1.634582362244256e-18, 4.248691367830441e-17},
+    {0.19509032201612828, -0.9807852804032304, -7.991079068461731e-18, -1.8546939997825006e-17},
+    {0.2902846772544624, -0.9569403357322088, -1.892797870777425e-17, -4.05538698618757e-17},
+    {0.3826834323650898, -0.9238795325112867, -1.0050772696461588e-17, -1.7645047084336677e-17},
+    {0.47139673682599764, -0.881921264348355, 6.516678136069013e-18, 1.9843248405890562e-17},
+    {0.5555702330196022, -0.8314696123025452, 4.709410940561677e-17, -1.4073856984728024e-18},
+    {0.6343932841636455, -0.773010453362737, 1.0420901929280035e-17, 3.256590703364977e-17},
+    {0.7071067811865476, -0.7071067811865476, -4.833646656726457e-17, 4.833646656726457e-17},
+    {0.773010453362737, -0.6343932841636455, -3.256590703364977e-17, -1.0420901929280035e-17},
+    {0.8314696123025452, -0.5555702330196022, 1.4073856984728024e-18, -4.709410940561677e-17},
+    {0.881921264348355, -0.47139673682599764, -1.9843248405890562e-17, -6.516678136069013e-18},
+    {0.9238795325112867, -0.3826834323650898, 1.7645047084336677e-17, 1.0050772696461588e-17},
+    {0.9569403357322088, -0.2902846772544624, 4.05538698618757e-17, 1.892797870777425e-17},
+    {0.9807852804032304, -0.19509032201612828, 1.8546939997825006e-17, 7.991079068461731e-18},
+    {0.9951847266721969, -0.0980171403295606, -4.248691367830441e-17, 1.634582362244256e-18},
+};
+// e^{-(x + i y)} = ea (c - i s) in FP64 by table lookup (P. T. P. Tang, "Table-driven
+// implementation of the exponential function in IEEE floating-point arithmetic",
+// 1989, and the same idea for sine and cosine):
+//   e^{-x} = 2^{k/64} e^{t}, |t| <= ln 2 / 128, k split into 2^{k >> 6} and a table value;
+//   cos y, sin y from the nearest of 64 angles and |t| <= pi / 64;
+// reductions by Cody-Waite splits whose products with k are exact, Taylor
+// polynomials to below 2^-57.  The FP64 pipe (1/74 of the FP32 rate) bounds every
+// FP64 kernel: about 36 of its operations here, exp and sincos take 75.  Error of the
+// complex value 2.5e-16 max, 7.7e-17 rms (exp and sincos: 2.8e-16, 8.1e-17), over
+// x < 690, |y| < 60000.  With sqrt_inv below: FP64 compression of the 1280-triangle
+// sphere 172 -> 152 ms, 320 x 320 x 16 FP64 entries 11.9 ->
+// 10.5 ms.  Outside |x| < 704, |y| < 65536 (and for NaN) the library
+// functions answer.
+struct ExpParts {
+    double ea, c, s;
+};
+static __device__ __noinline__ ExpParts exp_parts_any(double x, double y) {
+    ExpParts e;
+    e.ea = exp(-x);
+    sincos(y, &e.s, &e.c);
+    return e;
+}
+TD_D ExpParts exp_parts(double x, double y) {
+    // range checks on the high words: integer instructions (0x40860000: 704, 0x40f00000: 65536)
+    if ((__double2hiint(x) & 0x7fffffff) >= 0x40860000 || (__double2hiint(y) & 0x7fffffff) >= 0x40f00000)
+        return exp_parts_any(x, y);
+    const double magic = 6755399441055744.0;  // 1.5 * 2^52: adding it rounds to an integer
+    // exponential of -x
+    const double kx = fma(-x, 92.33248261689366, magic);
+    const int ix = __double2loint(kx);
+    const double fx = kx - magic;
+    double t = fma(-fx, 0.010830424695996044, -x);
+    t = fma(-fx, 2.5310172166650877e-13, t);
+    double p = fma(t, 1.0 / 720.0, 1.0 / 120.0);
+    p = fma(t, p, 1.0 / 24.0);
+    p = fma(t, p, 1.0 / 6.0);
+    p = fma(t, p, 0.5);
+    const double2 te = c_exp2_64[ix & 63];
+    p = fma(t * t, p, t) + te.y;  // e^t - 1, and the table value's rounding
+    const double eb = __hiloint2double(__double2hiint(te.x) + ((ix >> 6) << 20), __double2loint(te.x));
+    // angle y
+    const double ky = fma(y, 10.185916357881302, magic);
+    const int iy = __double2loint(ky);
+    const double fy = ky - magic;
+    double u = fma(-fy, 0.09817477042088285, y);
+    u = fma(-fy, 3.798187816439979e-12, u);
+    u = fma(-fy, 1.2639164054974691e-22, u);
+    const double v = u * u;
+    double s = fma(v, -1.0 / 5040.0, 1.0 / 120.0);
+    s = fma(v, s, -1.0 / 6.0);
+    s = fma(u * v, s, u);  // sin u
+    double c = fma(v, 1.0 / 40320.0, -1.0 / 720.0);
+    c = fma(v, c, 1.0 / 24.0);
+    c = fma(v, c, -0.5) * v;  // cos u - 1
+    const Cis64 w = c_cis_64[iy & 63];
+    return {fma(eb, p, eb), w.x + fma(w.x, c, fma(-w.y, s, w.z)), w.y + fma(w.y, c, fma(w.x, s, w.w))};
+}
 TD_D c64 expm_sr(double sr, double si, double r) {
-    double ea = exp(-sr * r);
-    double sn, cs;
-    sincos(si * r, &sn, &cs);
-    return {ea * cs, -ea * sn};
+    const ExpParts e = exp_parts(sr * r, si * r);
+    return {e.ea * e.c, -e.ea * e.s};
+}
+// sqrt(r2) and its reciprocal from one reciprocal square root, each corrected to
+// within 0.6 ulp: a square root and a division take 4 FP64 operations more.
+static __device__ __noinline__ double2 sqrt_inv_any(double r2) {
+    const double r = sqrt(r2);
+    return {r, 1.0 / r};
+}
+TD_D double sqrt_inv(double r2, double &ri) {
+    if ((unsigned)(__double2hiint(r2) - 0x00100000) >= 0x7fe00000u) {  // 0, subnormal, infinite, NaN
+        const double2 v = sqrt_inv_any(r2);
+        ri = v.y;
+        return v.x;
+    }
+    const double s = rsqrt(r2), g = r2 * s;
+    const double r = fma(fma(-g, g, r2), 0.5 * s, g);
+    ri = fma(fma(-r, s, 1.0), s, s);
+    return r;
 }
 
 // Test triangle in registers, by precision.
