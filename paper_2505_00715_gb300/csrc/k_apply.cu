@@ -152,42 +152,67 @@ __global__ void __launch_bounds__(256) k_apply(ApplyArgs a, TensorOut o, int TJ,
 }
 
 // y += A(s_f) x at one point of the list: sum_d f_d[f] H_d x, one CTA per block.
-//   near: every warp takes rows, its lanes the columns (coalesced); the terms are
-//         combined first, h = sum_d f_d H_d[i][j], then multiplied with x;
-//   far:  t = f_d V_d x by warps (one factor row each, lanes along it), then rows
-//         of y from U, threads along i (coalesced), CTAs of short blocks splitting
-//         the factor rows over thread groups.
+// Both kinds of block multiply a tile A of rows with x in shared memory, the threads
+// (row, part of the columns), the parts' sums meeting in shared memory:
+//   near: A = sum_d f_d H_d, combined as it is read (contiguous loads, all lanes
+//         busy for any width), rows of y;
+//   far:  A = rows of the V_d (asynchronous copies), t = f_d (V_d x) kept in shared
+//         memory; then rows of y from U, threads along i (coalesced), CTAs of
+//         short blocks splitting the factor rows over thread groups.
 // CC right-hand sides per pass over the faces.  A conjugate point takes conj(x)
-// and conjugates its result.  Bound: HBM, every face read once per pass.  The
-// general kernel read near rows with stride |J| and one right-hand side gave it
-// 4 CTAs of work per SM at a time: 30k housing, 8 frequencies, 1 right-hand side:
-// 1043 -> 340 us (142M stored values, 3.3 TB/s); 5120-triangle sphere, 4 right-hand
-// sides: 400 -> 193 us (14,488 blocks of 1800 values: latency).
-constexpr int kOneJ = 128, kOneT = 128, kOneD = 32;  // columns, factor rows, terms in shared memory at a time
+// and conjugates its result.  Bound: HBM (every face read once per pass) for long
+// blocks, the chain of dependent loads and the instructions for short ones.
+// 5120-triangle sphere, 4 right-hand sides (14,488 blocks of 1800 values): 400 us by
+// the general kernel -> 193 us with a warp per row (a reduction per row, lanes idle in
+// rows of 20 to 40 values) -> 134 us; 30k housing, 8 frequencies, 1 right-hand side
+// (142M stored values): 1043 -> 340 -> 274 us.
+constexpr int kOneT = 128, kOneD = 32;  // factor rows, terms in shared memory at a time
+constexpr int kOneBytes = 12288;                     // the tile A
+
+TD_D void copy_async(c32 *dst, const c32 *src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+TD_D void copy_async(c64 *dst, const c64 *src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
 
 template <class T, int CC>
-__global__ void __launch_bounds__(128, sizeof(T) == 4 ? (CC == 4 ? 8 : 10) : 5) k_apply_one(ApplyArgs a, TensorOut o, int c0) {
-    __shared__ cx<T> xs[kOneJ][CC];
-    __shared__ cx<T> ts[kOneT][CC];
+__global__ void __launch_bounds__(128, sizeof(T) == 4 ? 8 : 5) k_apply_one(ApplyArgs a, TensorOut o, int c0) {
+    constexpr int kH = kOneBytes / (int)sizeof(cx<T>), kOneJ = CC == 4 ? 128 : 256;  // tile, columns of x
+    constexpr int kDQ = sizeof(T) == 8 ? 1 : CC == 1 ? 3 : 2, kUQ = CC == 1 ? 8 : 4;  // terms of a near tile, loads of U in flight
+    __shared__ alignas(16) cx<T> h[kH];
+    __shared__ alignas(16) cx<T> xs[kOneJ][CC];
+    __shared__ alignas(16) cx<T> ts[kOneT][CC];
+    __shared__ alignas(16) cx<T> red[128][CC];
     __shared__ cx<T> fs[kOneD];
-    __shared__ long long off[kOneD];
-    __shared__ int pre[kOneD + 1];
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = 4, b = blockIdx.x;
+    __shared__ long long off[kOneD], rowoff[kOneT];
+    __shared__ int pre[kOneD + 1], rowd[kOneT];
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, b = blockIdx.x;
+    const int64_t tb = (int64_t)b * a.Nu;
+    const int mp = a.qmap[a.single_f];
+    const bool cj = mp < 0;
+    const int u = (cj ? -mp : mp) - 1;
+    // the first terms' data, before the number of terms is known
+    cx<T> pf = {0, 0};
+    long long po = 0;
+    int pk = 0;
+    if (tid < min(kOneD, a.Nu)) {
+        pf = ((const cx<T> *)o.fib)[(tb + tid) * a.Nu + u];
+        po = o.foff[tb + tid];
+        pk = o.frank[tb + tid];
+    }
     const int rb = o.rank[b];
     const int *bl = a.blocks + 5 * b;
     const int nI = bl[1] - bl[0], nJ = bl[3] - bl[2], nrhs = a.nrhs;
     const bool far = bl[4] != 0;
     const int nc = min(CC, nrhs - c0);
-    const int64_t tb = (int64_t)b * a.Nu;
-    const int mp = a.qmap[a.single_f];
-    const bool cj = mp < 0;
-    const int u = (cj ? -mp : mp) - 1;
+    const int *perm = a.perm_r + bl[0];
     const cx<T> *x = (const cx<T> *)a.W, *pool = (const cx<T> *)o.face;
     cx<T> *y = (cx<T> *)a.y;
     int loaded = -1;  // first column of the x tile in shared memory
-    auto load_x = [&](int j0, int tj) {
-        __syncthreads();
+    auto load_x = [&](int j0, int tj) {  // (the caller synchronises before the tile is read)
         if (loaded == j0) return;
+        if (loaded >= 0) __syncthreads();
         loaded = j0;
         for (int e = tid; e < tj * CC; e += 128) {
             const int j = e / CC, c = e - j * CC;
@@ -195,24 +220,49 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? (CC == 4 ? 8 : 10) : 5) 
             if (c < nc) v = x[(int64_t)a.perm_c[bl[2] + j0 + j] * nrhs + c0 + c];
             xs[j][c] = cj ? cconj(v) : v;
         }
-        __syncthreads();
     };
-    auto add = [&](int i, const cx<T> *v) {
-        cx<T> *yr = y + (int64_t)a.perm_r[bl[0] + i] * nrhs + c0;
+    // the product of the tile's ti rows with the x tile, by parts of the columns, to red;
+    // one thread per (row, column) then takes the sum of the parts
+    auto product = [&](int ti, int tj, int ld, auto take) {
+        const int P = 128 / ti, part = tid / ti, row = tid - part * ti;
+        cx<T> acc[CC];
 #pragma unroll
-        for (int c = 0; c < CC; ++c)
-            if (c < nc) atomic_add_c(yr + c, cj ? cconj(v[c]) : v[c]);
+        for (int c = 0; c < CC; ++c) acc[c] = cx<T>{0, 0};
+        if (part < P) {
+            const cx<T> *hr = h + row * ld;
+#pragma unroll (CC == 4 ? 2 : 4)
+            for (int j = part; j < tj; j += P) {
+                const cx<T> v = hr[j];
+#pragma unroll
+                for (int c = 0; c < CC; ++c) cfma(acc[c], v, xs[j][c]);
+            }
+        }
+#pragma unroll
+        for (int c = 0; c < CC; ++c) red[tid][c] = acc[c];
+        __syncthreads();
+        for (int e = tid; e < ti * CC; e += 128) {
+            const int i = e / CC, c = e - i * CC;
+            cx<T> s = red[i][c];
+            for (int q = 1; q < P; ++q) s = s + red[q * ti + i][c];
+            take(i, c, s);
+        }
     };
-    if (rb > 0) load_x(0, min(kOneJ, nJ));  // its dependent loads first
     for (int d0 = 0; d0 < rb; d0 += kOneD) {
         const int r = min(kOneD, rb - d0);
-        __syncthreads();
+        if (d0 > 0) {
+            __syncthreads();
+            if (tid < r) {
+                pf = ((const cx<T> *)o.fib)[(tb + d0 + tid) * a.Nu + u];
+                po = o.foff[tb + d0 + tid];
+                pk = o.frank[tb + d0 + tid];
+            }
+        }
         if (tid < r) {
-            fs[tid] = ((const cx<T> *)o.fib)[(tb + d0 + tid) * a.Nu + u];
-            off[tid] = o.foff[tb + d0 + tid];
+            fs[tid] = pf;
+            off[tid] = po;
         }
         if (wid == 0) {  // inclusive prefix of the face ranks
-            int k = far && lane < r ? o.frank[tb + d0 + lane] : 0;
+            int k = far && lane < r ? pk : 0;
             for (int s = 1; s < 32; s <<= 1) {
                 const int v = __shfl_up_sync(0xffffffffu, k, s);
                 if (lane >= s) k += v;
@@ -220,102 +270,85 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? (CC == 4 ? 8 : 10) : 5) 
             if (lane == 0) pre[0] = 0;
             pre[lane + 1] = k;
         }
+        load_x(0, min(kOneJ, nJ));
+        __syncthreads();
         if (!far) {
             for (int j0 = 0; j0 < nJ; j0 += kOneJ) {
-                const int tj = min(kOneJ, nJ - j0);
+                const int tj = min(kOneJ, nJ - j0), ld = tj | 1, rows = min(128, kH / ld);
+                const float inv = 1.0f / (float)tj;
                 load_x(j0, tj);
-                // two rows per warp and pass
-                for (int i = 2 * wid; i < nI; i += 2 * nw) {
-                    const bool two = i + 1 < nI;
-                    cx<T> acc[2][CC];
+                for (int i0 = 0; i0 < nI; i0 += rows) {
+                    const int ti = min(rows, nI - i0), n = ti * tj;
+                    const cx<T> *hb = pool + (int64_t)i0 * nJ + j0;
+                    for (int e0 = tid; e0 < n; e0 += 4 * 128) {
+                        int src[4], dst[4];
+                        cx<T> acc[4];
 #pragma unroll
-                    for (int c = 0; c < CC; ++c) acc[0][c] = acc[1][c] = cx<T>{0, 0};
-                    const int64_t ij = (int64_t)i * nJ + j0, st = two ? nJ : 0;
-                    for (int j = lane; j < tj; j += 32) {
-                        cx<T> h[2] = {{0, 0}, {0, 0}};
-                        int d = 0;
-                        for (; d + 4 <= r; d += 4) {
-                            cx<T> v[4][2];
-#pragma unroll
-                            for (int q = 0; q < 4; ++q) {
-                                const cx<T> *p = pool + off[d + q] + ij + j;
-                                v[q][0] = p[0];
-                                v[q][1] = p[st];
-                            }
-#pragma unroll
-                            for (int q = 0; q < 4; ++q) {
-                                cfma(h[0], fs[d + q], v[q][0]);
-                                cfma(h[1], fs[d + q], v[q][1]);
-                            }
+                        for (int q = 0; q < 4; ++q) {
+                            // (row: exact, e0 < 2^11 and tj <= 256)
+                            const int e = e0 + 128 * q, i = (int)(((float)e + 0.5f) * inv), j = e - i * tj;
+                            src[q] = e < n ? i * nJ + j : -1;
+                            dst[q] = i * ld + j;
+                            acc[q] = cx<T>{0, 0};
                         }
-                        for (; d < r; ++d) {
-                            const cx<T> *p = pool + off[d] + ij + j;
-                            const cx<T> v0 = p[0], v1 = p[st];
-                            cfma(h[0], fs[d], v0);
-                            cfma(h[1], fs[d], v1);
+                        for (int d = 0; d < r; d += kDQ) {
+                            cx<T> v[kDQ][4] = {};
+#pragma unroll
+                            for (int s = 0; s < kDQ; ++s)
+                                if (d + s < r) {
+                                    const cx<T> *p = hb + off[d + s];
+#pragma unroll
+                                    for (int q = 0; q < 4; ++q)
+                                        if (src[q] >= 0) v[s][q] = p[src[q]];
+                                }
+#pragma unroll
+                            for (int s = 0; s < kDQ; ++s)
+                                if (d + s < r) {
+#pragma unroll
+                                    for (int q = 0; q < 4; ++q) cfma(acc[q], fs[d + s], v[s][q]);
+                                }
                         }
 #pragma unroll
-                        for (int c = 0; c < CC; ++c) {
-                            cfma(acc[0][c], h[0], xs[j][c]);
-                            cfma(acc[1][c], h[1], xs[j][c]);
-                        }
+                        for (int q = 0; q < 4; ++q)
+                            if (src[q] >= 0) h[dst[q]] = acc[q];
                     }
-                    T v[4 * CC];  // row, column, part
-#pragma unroll
-                    for (int c = 0; c < CC; ++c) {
-                        v[2 * c] = acc[0][c].x;
-                        v[2 * c + 1] = cj ? -acc[0][c].y : acc[0][c].y;
-                        v[2 * CC + 2 * c] = acc[1][c].x;
-                        v[2 * CC + 2 * c + 1] = cj ? -acc[1][c].y : acc[1][c].y;
-                    }
-                    const T s = warp_sum_many<4 * CC>(v, lane);
-                    const int idx = many_index<4 * CC>(lane), row = idx / (2 * CC), c = (idx >> 1) % CC;
-                    if ((lane & (32 / (4 * CC) - 1)) == 0 && row <= (two ? 1 : 0) && c < nc) {
-                        cx<T> *yc = y + (int64_t)a.perm_r[bl[0] + i + row] * nrhs + c0 + c;
-                        atomicAdd(idx & 1 ? &yc->y : &yc->x, s);
-                    }
+                    const int yr = tid < ti * CC ? perm[i0 + tid / CC] : 0;
+                    __syncthreads();
+                    product(ti, tj, ld, [&](int i, int c, cx<T> s) {
+                        const int row = i == tid / CC ? yr : perm[i0 + i];
+                        if (c < nc) atomic_add_c(y + (int64_t)row * nrhs + c0 + c, cj ? cconj(s) : s);
+                    });
                 }
             }
             continue;
         }
-        __syncthreads();  // pre
         const int R = pre[r];
         for (int r0 = 0; r0 < R; r0 += kOneT) {
             const int rc = min(kOneT, R - r0);
-            for (int j0 = 0; j0 < nJ; j0 += kOneJ) {
-                const int tj = min(kOneJ, nJ - j0);
-                load_x(j0, tj);
+            if (tid < rc) {
                 int d = 0;
-                for (int t = wid; t < rc; t += nw) {
-                    while (r0 + t >= pre[d + 1]) ++d;
-                    const int kd = pre[d + 1] - pre[d], tau = r0 + t - pre[d];
-                    const cx<T> *v = pool + off[d] + (int64_t)kd * nI + (int64_t)tau * nJ + j0;
-                    cx<T> acc[CC], w[kOneJ / 32];
-#pragma unroll
-                    for (int q = 0; q < kOneJ / 32; ++q) w[q] = lane + 32 * q < tj ? v[lane + 32 * q] : cx<T>{0, 0};
-#pragma unroll
-                    for (int c = 0; c < CC; ++c) acc[c] = cx<T>{0, 0};
-#pragma unroll
-                    for (int q = 0; q < kOneJ / 32; ++q) {
-                        if (lane + 32 * q < tj) {
-#pragma unroll
-                            for (int c = 0; c < CC; ++c) cfma(acc[c], w[q], xs[lane + 32 * q][c]);
-                        }
+                while (r0 + tid >= pre[d + 1]) ++d;
+                rowd[tid] = d;
+                rowoff[tid] = off[d] + (int64_t)(pre[d + 1] - pre[d]) * nI + (int64_t)(r0 + tid - pre[d]) * nJ;
+            }
+            __syncthreads();
+            for (int j0 = 0; j0 < nJ; j0 += kOneJ) {
+                const int tj = min(kOneJ, nJ - j0), ld = tj | 1, rows = min(128, kH / ld);
+                const float inv = 1.0f / (float)tj;
+                load_x(j0, tj);
+                for (int i0 = 0; i0 < rc; i0 += rows) {
+                    const int ti = min(rows, rc - i0), n = ti * tj;
+#pragma unroll 4
+                    for (int e = tid; e < n; e += 128) {
+                        const int i = (int)(((float)e + 0.5f) * inv), j = e - i * tj;
+                        copy_async(h + i * ld + j, pool + rowoff[i0 + i] + j0 + j);
                     }
-                    T s[2 * CC];
-#pragma unroll
-                    for (int c = 0; c < CC; ++c) {
-                        s[2 * c] = acc[c].x;
-                        s[2 * c + 1] = acc[c].y;
-                    }
-                    constexpr int LB = 32 / (2 * CC);  // lanes per value; the other part is LB lanes on
-                    const T own = warp_sum_many<2 * CC>(s, lane), oth = __shfl_xor_sync(0xffffffffu, own, LB);
-                    const int idx = many_index<2 * CC>(lane);
-                    const T val = idx & 1 ? fs[d].x * own + fs[d].y * oth : fs[d].x * own - fs[d].y * oth;
-                    if ((lane & (LB - 1)) == 0) {
-                        T *tp = reinterpret_cast<T *>(&ts[t][0]) + idx;
-                        *tp = j0 == 0 ? val : *tp + val;
-                    }
+                    asm volatile("cp.async.wait_all;" ::: "memory");
+                    __syncthreads();
+                    product(ti, tj, ld, [&](int i, int c, cx<T> s) {
+                        const cx<T> v = fs[rowd[i0 + i]] * s;
+                        ts[i0 + i][c] = j0 == 0 ? v : ts[i0 + i][c] + v;
+                    });
                 }
             }
             __syncthreads();
@@ -323,25 +356,26 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? (CC == 4 ? 8 : 10) : 5) 
             const int gi = nI >= 128 ? 128 : (nI + 31) & ~31, G = 128 / gi;
             const int g = tid / gi;
             cx<T> own[CC];
+            int yrow = 0;
             if (g < G) {
                 const int per = (rc + G - 1) / G, tA = min(rc, g * per), tB = min(rc, tA + per);
                 for (int i = tid - g * gi; i < nI && (tA < tB || G > 1); i += gi) {
+                    if (g == 0) yrow = perm[i];
                     cx<T> acc[CC];
 #pragma unroll
                     for (int c = 0; c < CC; ++c) acc[c] = cx<T>{0, 0};
-                    int d = 0;
                     for (int t = tA; t < tB;) {
-                        while (r0 + t >= pre[d + 1]) ++d;
+                        const int d = rowd[t];
                         // a run of factor rows of one term is contiguous
                         const int te = min(tB, pre[d + 1] - r0), n = te - t;
                         const cx<T> *ub = pool + off[d] + (int64_t)(r0 + t - pre[d]) * nI + i;
                         int q = 0;
-                        for (; q + 4 <= n; q += 4) {
-                            cx<T> uv[4];
+                        for (; q + kUQ <= n; q += kUQ) {
+                            cx<T> uv[kUQ];
 #pragma unroll
-                            for (int e = 0; e < 4; ++e) uv[e] = ub[(int64_t)(q + e) * nI];
+                            for (int e = 0; e < kUQ; ++e) uv[e] = ub[(int64_t)(q + e) * nI];
 #pragma unroll
-                            for (int e = 0; e < 4; ++e)
+                            for (int e = 0; e < kUQ; ++e)
 #pragma unroll
                                 for (int c = 0; c < CC; ++c) cfma(acc[c], uv[e], ts[t + q + e][c]);
                         }
@@ -352,25 +386,28 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? (CC == 4 ? 8 : 10) : 5) 
                         }
                         t = te;
                     }
-                    if (G == 1 || g == 0) {
-                        if (G == 1) add(i, acc);
+                    if (G == 1) {
 #pragma unroll
-                        for (int c = 0; c < CC; ++c) own[c] = acc[c];
-                    } else {
+                        for (int c = 0; c < CC; ++c)
+                            if (c < nc) atomic_add_c(y + (int64_t)yrow * nrhs + c0 + c, cj ? cconj(acc[c]) : acc[c]);
+                    }
 #pragma unroll
-                        for (int c = 0; c < CC; ++c) xs[tid - gi][c] = acc[c];  // (G > 1: one i per thread)
+                    for (int c = 0; c < CC; ++c) {
+                        own[c] = acc[c];
+                        if (g > 0) red[tid - gi][c] = acc[c];  // (G > 1: one i per thread)
                     }
                 }
             }
             __syncthreads();
-            if (G > 1) {  // the groups' sums meet in the place of x: one atomic add per output
+            if (G > 1) {  // the groups' sums meet: one atomic add per output
                 if (g == 0 && tid < nI) {
                     for (int q = 1; q < G; ++q)
 #pragma unroll
-                        for (int c = 0; c < CC; ++c) own[c] = own[c] + xs[(q - 1) * gi + tid][c];
-                    add(tid, own);
+                        for (int c = 0; c < CC; ++c) own[c] = own[c] + red[(q - 1) * gi + tid][c];
+#pragma unroll
+                    for (int c = 0; c < CC; ++c)
+                        if (c < nc) atomic_add_c(y + (int64_t)yrow * nrhs + c0 + c, cj ? cconj(own[c]) : own[c]);
                 }
-                loaded = -1;
                 __syncthreads();
             }
         }

@@ -115,7 +115,7 @@ __global__ void __launch_bounds__(256) k_residual(cx<T> *r, const cx<T> *b, cons
 // the modified form) so that a step is one product, six launches and one wait for
 // the host's rotations, where modified Gram-Schmidt waited for the host after
 // every inner product: 5120-triangle sphere, 4 right-hand sides, 19 steps: 212 waits,
-// 15.1 -> 10.9 ms by the single-frequency apply of k_apply_one, -> 5.8 ms by this.
+// 15.1 -> 10.9 ms by the single-frequency apply of k_apply_one, -> 5.8 ms by this (4.5 with its later form).
 template <class T>
 int gmres(tdbem_tensor *t, int fidx, const cx<T> *b, int n, cx<T> *x, double tol, int maxit, int m, int *iters,
           double *relres) {
