@@ -895,6 +895,36 @@ TensorOut tensor_out(const tdbem_tensor *t, int *flags) {
 
 }  // namespace
 
+// Blocks by stored values, largest first (to a quarter of a power of two: a counting
+// sort on the leading bits): the applies give every block a CTA, and large blocks
+// begun last left the chip idle for a quarter of the time (SM cycles active / elapsed
+// 0.76).  One frequency of the 5120-triangle sphere, 4 right-hand sides: 134 -> 103 us,
+// of the 30k housing: 274 -> 244 us; weighted apply of 1280 triangles 264 -> 246 us.
+std::vector<int32_t> td_block_order(const tdbem_tensor *t) {
+    const int64_t nb = t->nblocks;
+    std::vector<uint8_t> key(nb);
+    int count[257] = {0};
+    for (int64_t b = 0; b < nb; ++b) {
+        const int32_t *bl = &t->blocks[5 * b];
+        const int64_t nI = bl[1] - bl[0], nJ = bl[3] - bl[2];
+        const float w = 1.0f + (float)(bl[4] ? t->frank_sum[b] * (nI + nJ) : t->rank[b] * nI * nJ);
+        uint32_t bits;
+        std::memcpy(&bits, &w, 4);
+        key[b] = (uint8_t)(255 - std::min<uint32_t>(255, (bits - 0x3f800000u) >> 21));
+        ++count[key[b] + 1];
+    }
+    for (int k = 0; k < 256; ++k) count[k + 1] += count[k];
+    std::vector<int32_t> order(nb);
+    for (int64_t b = 0; b < nb; ++b) order[count[key[b]]++] = (int32_t)b;
+    return order;
+}
+
+int td_upload_order(tdbem_tensor *t) {
+    const std::vector<int32_t> order = td_block_order(t);
+    int rc = t->dorder ? TDBEM_OK : dalloc(t->ctx, &t->dorder, order.size(), &t->owned);
+    return rc ? rc : upload(t->ctx, t->dorder, order.data(), order.size());
+}
+
 extern "C" int tdbem_compress(tdbem_ctx_t ctx, tdbem_mesh_t mesh, const tdbem_op *op, tdbem_freqs_t f,
                               tdbem_tree_t tree, const tdbem_aca_cfg *cfg, tdbem_tensor_t *out) {
     cudaGetLastError();  // errors of earlier unrelated calls are not ours to report
@@ -1391,6 +1421,7 @@ extern "C" int tdbem_compress(tdbem_ctx_t ctx, tdbem_mesh_t mesh, const tdbem_op
             }
         }
     }
+    if ((rc = td_upload_order(T))) return fail(rc);
     st.dense_complex = T->nrows * T->ncols * (int64_t)Nu;
     st.entries_regular = (pf ? 0 : nent * Nu) + hev[0];
     st.entries_tube = hev[1];
@@ -1542,11 +1573,11 @@ int build_apply_plan(tdbem_tensor *t, int nrhs) {
     std::vector<int2> ftab;
     std::vector<int64_t> toff((size_t)nb * t->Nu, -1);
     int64_t tsize = 0;
-    for (int64_t b = 0; b < nb; ++b) {
+    for (const int32_t b : td_block_order(t)) {
         if (!t->blocks[5 * b + 4]) continue;
         for (int d = 0; d < t->rank[b]; ++d) {
             const int kd = frank[(size_t)b * t->Nu + d];
-            ftab.push_back(make_int2((int)b, d));
+            ftab.push_back(make_int2(b, d));
             toff[(size_t)b * t->Nu + d] = tsize;
             tsize += (int64_t)rpt * std::max(kd, 0) * nrhs;
         }
@@ -1639,6 +1670,7 @@ int apply_tc(tdbem_tensor *t, const void *W, int nrhs, void *y) {
     ApplyZArgs a{};
     a.nb = (int)t->nblocks;
     a.blocks = t->dblocks;
+    a.order = t->dorder;
     a.perm_r = t->dperm_r;
     a.Nu = t->Nu;
     a.nrhs = nrhs;
@@ -1666,6 +1698,7 @@ int apply_impl(tdbem_tensor *t, const void *W, int nrhs, void *y, int single_f) 
     ApplyArgs a{};
     a.nb = (int)t->nblocks;
     a.blocks = t->dblocks;
+    a.order = t->dorder;
     a.perm_r = t->dperm_r;
     a.perm_c = t->dperm_c;
     a.Nu = t->Nu;

@@ -104,6 +104,7 @@ struct tdbem_tensor {
     int Nu = 0, NQ = 0;
     int64_t nblocks = 0;
     int32_t *dblocks = nullptr;     // [nb][5] permuted ranges
+    int32_t *dorder = nullptr;      // [nb] blocks by stored values, largest first (applies)
     int32_t *dperm_r = nullptr, *dperm_c = nullptr;   // position -> DOF
     int32_t *dinv_r = nullptr, *dinv_c = nullptr;     // DOF -> position
     // per block: number of terms, per term (fixed slots [nb][Nu]): selected
@@ -152,6 +153,9 @@ int td_fail(tdbem_ctx *ctx, int code, const char *fmt, ...);
 // a mesh's tables (Gauss-Legendre rule gx/gw and touching-pair slots as given)
 struct MeshDev;
 int td_check_op(tdbem_ctx *ctx, const tdbem_op *op);
+// blocks of a tensor by stored values, largest first; uploaded to t->dorder
+std::vector<int32_t> td_block_order(const tdbem_tensor *t);
+int td_upload_order(tdbem_tensor *t);
 MeshDev td_mesh_dev(const tdbem_mesh *m, int ng, const double *gx, const double *gw, const int *tp_slot);
 // noalloc.cu: device address of the allocation-free entry point's scratch on
 // the current device `device` (once per device, cached)

@@ -164,8 +164,8 @@ __global__ void __launch_bounds__(256) k_apply(ApplyArgs a, TensorOut o, int TJ,
 // blocks, the chain of dependent loads and the instructions for short ones.
 // 5120-triangle sphere, 4 right-hand sides (14,488 blocks of 1800 values): 400 us by
 // the general kernel -> 193 us with a warp per row (a reduction per row, lanes idle in
-// rows of 20 to 40 values) -> 134 us; 30k housing, 8 frequencies, 1 right-hand side
-// (142M stored values): 1043 -> 340 -> 274 us.
+// rows of 20 to 40 values) -> 134 us, 103 with the largest blocks first; 30k housing,
+// 8 frequencies, 1 right-hand side (142M stored values): 1043 -> 340 -> 274, 244 us.
 constexpr int kOneT = 128, kOneD = 32;  // factor rows, terms in shared memory at a time
 constexpr int kOneBytes = 12288;                     // the tile A
 
@@ -187,7 +187,7 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 8 : 5) k_apply_one(Apply
     __shared__ cx<T> fs[kOneD];
     __shared__ long long off[kOneD], rowoff[kOneT];
     __shared__ int pre[kOneD + 1], rowd[kOneT];
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, b = blockIdx.x;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, b = a.order[blockIdx.x];
     const int64_t tb = (int64_t)b * a.Nu;
     const int mp = a.qmap[a.single_f];
     const bool cj = mp < 0;
@@ -479,7 +479,7 @@ __global__ void __launch_bounds__(128) k_apply_faces(ApplyZArgs a, TensorOut o, 
         d0 = bd.y;
         d1 = bd.y + 1;
     } else {
-        b = blockIdx.x;
+        b = a.order[blockIdx.x];
         d0 = 0;
         d1 = o.rank[b];
         if (d1 == 0 || a.zbase[b] < 0) return;

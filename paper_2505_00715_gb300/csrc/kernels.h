@@ -142,6 +142,7 @@ struct ApplyArgs {
     int kcap;              // largest far face rank
     int max_near_rows;     // largest row count of a near block
     int64_t acc_max;       // accumulator size (complex units), set by the launcher
+    const int *order;      // blocks by stored values, largest first
 };
 int td_launch_apply(cudaStream_t st, int prec, const ApplyArgs &a, const TensorOut &o, int num_sms);
 
@@ -184,6 +185,7 @@ int td_zgemm_tile_cols();
 struct ApplyZArgs {
     int nb;
     const int *blocks;
+    const int *order;       // blocks by stored values, largest first
     const int *perm_r;
     int Nu, nrhs, rpt;      // rpt: Z rows per term (2 with a conjugate half, else 1)
     const int64_t *zbase;   // [nb] Z offset of the block's row (term 0, half 0) (-1: rank 0);

@@ -115,7 +115,8 @@ __global__ void __launch_bounds__(256) k_residual(cx<T> *r, const cx<T> *b, cons
 // the modified form) so that a step is one product, six launches and one wait for
 // the host's rotations, where modified Gram-Schmidt waited for the host after
 // every inner product: 5120-triangle sphere, 4 right-hand sides, 19 steps: 212 waits,
-// 15.1 -> 10.9 ms by the single-frequency apply of k_apply_one, -> 5.8 ms by this (4.5 with its later form).
+// 15.1 -> 10.9 ms by the single-frequency apply of k_apply_one, -> 5.8 ms by this,
+// -> 4.0 ms by later forms of that apply.
 template <class T>
 int gmres(tdbem_tensor *t, int fidx, const cx<T> *b, int n, cx<T> *x, double tol, int maxit, int m, int *iters,
           double *relres) {
@@ -407,6 +408,11 @@ extern "C" int tdbem_tensor_load(tdbem_ctx_t ctx, const char *path, tdbem_tensor
         return td_fail(ctx, TDBEM_ERR_ARG, "reading %s failed", path);
     }
     t->face_cap = used;
+    if (const int rc = td_upload_order(t)) {
+        for (void *p : t->owned) cudaFree(p);
+        delete t;
+        return rc;
+    }
     *out = t;
     return TDBEM_OK;
 }
