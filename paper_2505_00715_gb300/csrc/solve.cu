@@ -19,6 +19,20 @@
 
 namespace {
 
+// red[c] = sum over the threads c, c + n, c + 2 n, ... < act of red, by halves (a thread
+// per column adding 64 values in a row was a fifth of k_dots)
+template <class R>
+TD_D void column_sums(R *red, int act, int n) {
+    const int g = threadIdx.x / n;
+    for (int G = act / n; G > 1;) {
+        const int half = (G + 1) / 2;
+        __syncthreads();
+        if (g < G - half) red[threadIdx.x] = red[threadIdx.x] + red[threadIdx.x + half * n];
+        G = half;
+    }
+    __syncthreads();
+}
+
 // out[i n + c] += sum_r conj(V_i[r][c]) w[r][c] for the vectors V_i, i = blockIdx.y
 // (FP64 accumulation; n <= 64 columns).  A thread keeps to one column: the
 // block's active threads are a multiple of n.
@@ -36,10 +50,9 @@ __global__ void __launch_bounds__(256) k_dots(const cx<T> *V, const cx<T> *w, in
             im += (double)x.x * y.y - (double)x.y * y.x;
         }
     red[tid] = c64{re, im};
-    __syncthreads();
+    column_sums(red, act, n);
     if (tid < n) {
-        c64 s = {0.0, 0.0};
-        for (int t = tid; t < act; t += n) s = s + red[t];
+        const c64 s = red[tid];
         c64 *o = out + (int64_t)blockIdx.y * n + tid;
         atomicAdd(&o->x, s.x);
         atomicAdd(&o->y, s.y);
@@ -68,12 +81,8 @@ __global__ void __launch_bounds__(256) k_combine(cx<T> *y, const cx<T> *V, const
         }
     if (!norm2) return;
     red[tid] = s2;
-    __syncthreads();
-    if (tid < n) {
-        double s = 0.0;
-        for (int t = tid; t < act; t += n) s += red[t];
-        atomicAdd(&norm2[tid], s);
-    }
+    column_sums(red, act, n);
+    if (tid < n) atomicAdd(&norm2[tid], red[tid]);
 }
 
 // y[r][c] = x[r][c] / sqrt(norm2[c]) (0 where the norm is 0)
@@ -102,12 +111,8 @@ __global__ void __launch_bounds__(256) k_residual(cx<T> *r, const cx<T> *b, cons
             s2 += (double)v.x * v.x + (double)v.y * v.y;
         }
     red[tid] = s2;
-    __syncthreads();
-    if (tid < n) {
-        double s = 0.0;
-        for (int t = tid; t < act; t += n) s += red[t];
-        atomicAdd(&norm2[tid], s);
-    }
+    column_sums(red, act, n);
+    if (tid < n) atomicAdd(&norm2[tid], red[tid]);
 }
 
 // Restarted GMRES.  Arnoldi by classical Gram-Schmidt applied twice (two passes of
@@ -116,7 +121,8 @@ __global__ void __launch_bounds__(256) k_residual(cx<T> *r, const cx<T> *b, cons
 // the host's rotations, where modified Gram-Schmidt waited for the host after
 // every inner product: 5120-triangle sphere, 4 right-hand sides, 19 steps: 212 waits,
 // 15.1 -> 10.9 ms by the single-frequency apply of k_apply_one, -> 5.8 ms by this,
-// -> 4.0 ms by later forms of that apply.
+// -> 4.0 ms by later forms of that apply, -> 3.6 ms by one copy of a step's sums and
+// their reduction by halves.
 template <class T>
 int gmres(tdbem_tensor *t, int fidx, const cx<T> *b, int n, cx<T> *x, double tol, int maxit, int m, int *iters,
           double *relres) {
@@ -124,7 +130,7 @@ int gmres(tdbem_tensor *t, int fidx, const cx<T> *b, int n, cx<T> *x, double tol
     cudaStream_t st = ctx->stream;
     const int64_t M = t->nrows, Mn = M * n;
     using C = std::complex<double>;
-    // one allocation: V [m + 1] | w | r, then FP64 h1 [m + 1][n] | h2 [m + 1][n] | norm2 [n]
+    // one allocation: V [m + 1] | w | r, then FP64 sums [2 (m + 1)][n] complex | norm2 [n]
     const size_t vb = (sizeof(cx<T>) * Mn * (m + 3) + 255) & ~(size_t)255;
     const size_t nh = (size_t)(m + 1) * n, hb = sizeof(c64) * 2 * nh + sizeof(double) * n;
     char *mem = nullptr;
@@ -133,9 +139,9 @@ int gmres(tdbem_tensor *t, int fidx, const cx<T> *b, int n, cx<T> *x, double tol
         return TDBEM_ERR_OOM;
     }
     cx<T> *V = (cx<T> *)mem, *w = V + (int64_t)(m + 1) * Mn, *r = w + Mn;
-    c64 *h1 = (c64 *)(mem + vb), *h2 = h1 + nh;
-    double *norm2 = (double *)(h2 + nh);
-    std::vector<C> hh(2 * nh);
+    c64 *h1 = (c64 *)(mem + vb);
+    double *norm2 = (double *)(h1 + 2 * nh);
+    std::vector<C> hh(2 * nh + (n + 1) / 2);
     std::vector<double> hn(n);
     const int act = 256 / n * n;
     const unsigned g = (unsigned)std::max<int64_t>(1, std::min<int64_t>((Mn + act - 1) / act, (int64_t)ctx->num_sms * 2));
@@ -174,21 +180,24 @@ int gmres(tdbem_tensor *t, int fidx, const cx<T> *b, int n, cx<T> *x, double tol
         for (; j < m && it < maxit; ++j, ++it) {
             cx<T> *Vj = V + (int64_t)j * Mn, *Vn = V + (int64_t)(j + 1) * Mn;
             if ((rc = tdbem_apply_freq(t, fidx, Vj, n, w))) break;
-            cudaMemsetAsync(h1, 0, hb, st);
+            // the step's sums h1 [j + 1][n] | h2 [j + 1][n] | squared norms [n], read back by one copy
+            const size_t nj = (size_t)(j + 1) * n, sb = sizeof(c64) * 2 * nj + sizeof(double) * n;
+            c64 *h2 = h1 + nj;
+            double *nw = (double *)(h2 + nj);
+            cudaMemsetAsync(h1, 0, sb, st);
             const dim3 gd(std::max(1u, std::min(g, 2u * (unsigned)ctx->num_sms / (unsigned)(j + 1) + 1u)), j + 1);
             k_dots<T><<<gd, 256, 0, st>>>(V, w, M, n, h1);
             k_combine<T><<<g, 256, 0, st>>>(w, V, h1, j + 1, -1.0, M, n, nullptr);
             k_dots<T><<<gd, 256, 0, st>>>(V, w, M, n, h2);
-            k_combine<T><<<g, 256, 0, st>>>(w, V, h2, j + 1, -1.0, M, n, norm2);
-            k_normalise<T><<<g, 256, 0, st>>>(Vn, w, norm2, M, n);
-            cudaMemcpyAsync(hh.data(), h1, sizeof(c64) * (j + 1) * n, cudaMemcpyDeviceToHost, st);
-            cudaMemcpyAsync(hh.data() + nh, h2, sizeof(c64) * (j + 1) * n, cudaMemcpyDeviceToHost, st);
-            cudaMemcpyAsync(hn.data(), norm2, sizeof(double) * n, cudaMemcpyDeviceToHost, st);
+            k_combine<T><<<g, 256, 0, st>>>(w, V, h2, j + 1, -1.0, M, n, nw);
+            k_normalise<T><<<g, 256, 0, st>>>(Vn, w, nw, M, n);
+            cudaMemcpyAsync(hh.data(), h1, sb, cudaMemcpyDeviceToHost, st);
             if ((rc = ok(cudaStreamSynchronize(st)))) break;
+            const double *hw = reinterpret_cast<const double *>(hh.data() + 2 * nj);
             bool all = true;
             for (int c = 0; c < n; ++c) {
-                for (int i = 0; i <= j; ++i) H[c][i * m + j] = hh[i * n + c] + hh[nh + i * n + c];
-                const double h = std::sqrt(std::max(hn[c], 0.0));
+                for (int i = 0; i <= j; ++i) H[c][i * m + j] = hh[i * n + c] + hh[nj + i * n + c];
+                const double h = std::sqrt(std::max(hw[c], 0.0));
                 H[c][(j + 1) * m + j] = h;
                 // Givens rotations on column j
                 for (int i = 0; i < j; ++i) {
