@@ -101,10 +101,10 @@ typedef struct {
     int64_t sum_face_rank;          /* ACA ranks of the far faces, summed */
     int64_t stored_complex;         /* complex numbers stored (faces + fibres) */
     int64_t dense_complex;          /* rows * cols * unique frequencies */
-    int64_t entries_regular;        /* regular entries evaluated (near and far; a near block of the
-                                       mixed form evaluates the frequencies it selects) */
-    int64_t entries_tube;           /* fibre (all-frequency) entries evaluated (far blocks, and near
-                                       blocks of the mixed form) */
+    int64_t entries_regular;        /* regular entries: the near blocks' at every unique frequency (of
+                                       which the mixed form evaluates the slices that the
+                                       approximation selects) and those evaluated by far fibres */
+    int64_t entries_tube;           /* fibre (all-frequency) entries evaluated (far blocks) */
     int64_t pairs_singular;         /* touching pairs integrated (per frequency) */
     double ms_plan, ms_singular, ms_near, ms_far, ms_total;
     int64_t pool_growths;           /* face pool grown during compression: far blocks redone

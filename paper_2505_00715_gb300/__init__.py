@@ -79,7 +79,7 @@ class Context:
         self.check(self.L.tdbem_ctx_set_wait_limit(self.h, int(polls)), "tdbem_ctx_set_wait_limit")
 
     def set_near_batch(self, nbytes):
-        """Buffer size (bytes) of the batched near-field tensor in compress."""
+        """Buffer size (bytes) of the FP64 form's batched near-field tensor in compress."""
         self.check(self.L.tdbem_ctx_set_near_batch(self.h, int(nbytes)), "tdbem_ctx_set_near_batch")
 
     def __del__(self):
@@ -201,8 +201,8 @@ PATH_GENERIC, PATH_NEAR, PATH_FIBRE = 0, 1, 2
 def entries(mesh, op, freqs, rows, cols, fidx, prec=MIXED, c=1.0, ng=5, path=PATH_GENERIC):
     """A[rows, cols](s_fidx) as a device tensor [nf, nr, nc] (complex64 MIXED, complex128 FP64).
     path selects the kernel: PATH_GENERIC (tdbem_entries), PATH_NEAR (the
-    compression's touching-pair table and near-field tensor kernels on the
-    block rows x cols) or PATH_FIBRE (the far-field engine's point-pair groups;
+    compression's touching-pair table and near-field sums on the block
+    rows x cols) or PATH_FIBRE (the far-field engine's point-pair groups;
     regular rule on every pair)."""
     torch = _torch()
     ctx = mesh.ctx
@@ -348,7 +348,7 @@ def compress(mesh, op, freqs, tree, eps=1e-4, eps_aca=1e-6, prec=MIXED, c=1.0, n
 def autotune(mesh, op, freqs, tree, eps=1e-4, eps_aca=1e-6, prec=MIXED, c=1.0, ng=5, max_face_rank=64, model=None):
     """Time the compression with candidate launch parameters and keep the fastest
     per phase in the context; returns (far threads per CTA, far CTAs per SM,
-    touching-pair frequencies per pass, near-field frequencies per pass)."""
+    touching-pair frequencies per pass, frequencies per pass of PATH_NEAR (not tuned))."""
     ctx = mesh.ctx
     o = _op(op, prec, c, ng)
     cfg = _lib.AcaCfg(eps, eps_aca, max_face_rank, 0, model.h if model is not None else None)

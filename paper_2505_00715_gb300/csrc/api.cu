@@ -1143,7 +1143,6 @@ extern "C" int tdbem_compress(tdbem_ctx_t ctx, tdbem_mesh_t mesh, const tdbem_op
     na.nentries = nent;
     na.near = nearbuf;
     na.table = table;
-    na.evals = evals;
     AcaParams ap{cfg->eps, cfg->eps_aca, kcap};
     FarArgs fa{};
     fa.nfar = (int)far_ids.size();
@@ -1423,7 +1422,7 @@ extern "C" int tdbem_compress(tdbem_ctx_t ctx, tdbem_mesh_t mesh, const tdbem_op
     }
     if ((rc = td_upload_order(T))) return fail(rc);
     st.dense_complex = T->nrows * T->ncols * (int64_t)Nu;
-    st.entries_regular = (pf ? 0 : nent * Nu) + hev[0];
+    st.entries_regular = nent * Nu + hev[0];
     st.entries_tube = hev[1];
     st.aca_tests = hev[2];
     st.pairs_singular = (int64_t)npairs * Nu;

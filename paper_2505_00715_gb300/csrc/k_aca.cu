@@ -130,7 +130,6 @@ __global__ void __launch_bounds__(128) k_near_aca(MeshDev m, NearArgs a, TensorO
     cx<T> *H = scratch + (int64_t)blockIdx.x * sper;
     cx<T> *fib = (cx<T> *)o.fib;
     cx<T> *pool = (cx<T> *)o.face;
-    long long ev_face = 0, ev_tube = 0;  // entries evaluated on demand
     for (int nb = blockIdx.x; nb < a.nnear; nb += gridDim.x) {
         const int b = a.near_ids[nb];
         const int *bl = a.blocks + 5 * b;
@@ -164,14 +163,12 @@ __global__ void __launch_bounds__(128) k_near_aca(MeshDev m, NearArgs a, TensorO
                 const auto key = pivot_key(h);
                 if (am_better(key, (int)e, am.v, am.i)) am = {key, (int)e};
             }
-            ev_face += nIJ;
             am = block_argmax(am, red);
             if (!(am.v > 0)) {
                 r = l;
                 break;
             }
             const int ep = am.i;
-            ev_tube += Nu;
             const cx<T> piv = H[ep];
             for (int d = tid; d < l; d += blockDim.x) s_hd[d] = pool[o.foff[tb + d] + ep];
             __syncthreads();
@@ -254,10 +251,6 @@ __global__ void __launch_bounds__(128) k_near_aca(MeshDev m, NearArgs a, TensorO
         if (r < 0) r = l;
         if (tid == 0) o.rank[b] = r;
         __syncthreads();
-    }
-    if (OP >= 0 && tid == 0 && a.evals) {
-        atomicAdd((unsigned long long *)&a.evals[0], (unsigned long long)ev_face);
-        atomicAdd((unsigned long long *)&a.evals[1], (unsigned long long)ev_tube);
     }
 }
 

@@ -19,7 +19,6 @@ struct NearArgs {
     int64_t nentries;
     void *near;              // near tensor (FP64 form)
     const c64 *table;        // touching-pair table (mixed form: entries on demand)
-    int64_t *evals;          // [2] regular, tube entries evaluated on demand
 };
 
 // Output arrays of the compressed tensor (fixed slots per block and term).
