@@ -9,10 +9,10 @@
 //   ||C^(l)||_F^2 = sum_{d,d'} <H_d, H_d'> <f_d, f_d'>   (eq. norm, FP64),
 //   k_{l+1} = argmax |f_l[k]| over frequencies not selected yet.
 // Near-field blocks (k_near_aca): dense faces, from the precomputed near tensor
-// (FP64 form) or evaluated on demand (mixed form), one CTA per block.  Far-field blocks (k_far_aca): every residual face is
-// compressed by ACA with partial pivoting (row fibre at i*, column fibre at
-// j*, FP64 norm recursion of the matrix analogue of eq. norm) from entries
-// evaluated on the fly; the face is rebuilt to find the pivot and discarded
+// (FP64 form) or evaluated on demand (mixed form), one CTA per block.
+// Far-field blocks (k_far_aca): every residual face is compressed by ACA with
+// partial pivoting (row fibre at i*, column fibre at j*, FP64 norm recursion of
+// the matrix analogue of eq. norm) from entries evaluated on the fly; the face is rebuilt to find the pivot and discarded
 // (Sec. 4); the frequency tube at the pivot is evaluated with one warp per
 // frequency.  Persistent CTAs take far blocks from an atomic work queue
 // ordered by decreasing size.
@@ -396,7 +396,8 @@ TD_D cx<T> group_entry(const MeshDev &m, int row, int col, T sr, T si, bool vali
 // the lanes read their test point of the next row.  Every lane of a group used to
 // read all seven trial points itself, 14 16-byte loads an entry through an L1
 // that shared memory leaves a quarter of: 30k housing 617 -> 547 ms (whole far
-// phase), 5120-triangle sphere 61 -> 57, double layer 133 -> 97 ms.
+// phase; 484 with more loads in flight in the corrections, norm tests and Grams),
+// 5120-triangle sphere 61 -> 57 (52), double layer 133 -> 97 (86) ms.
 // P1 columns: every support triangle in turn (row), group_entry (column).
 template <class T, int OP, class F>
 TD_D void row_fibre(const MeshDev &m, QPoint<T> *ex, int row, const int *cols, int nJ, T sr, T si, F out) {

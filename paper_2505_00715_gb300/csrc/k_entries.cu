@@ -87,7 +87,7 @@ TD_D double hat7(int b, int loc, double) { return bary7d(b, loc); }
 // both forms), without it k_entry_sing adds them for all frequencies at once.  One
 // thread per entry left a warp waiting for the lane with the touching pair, 1250
 // points in a row at latency: 320 x 320 x 16 FP64 entries 269 -> 18.1 ms with SING, 10.5 with
-// k_entry_sing; 67 x 1801 x 11 double-layer entries 119 -> 6.2 and 3.3 ms.  Bound:
+// k_entry_sing; 67 x 1801 x 11 double-layer entries 119 -> 6.2 and 2.9 ms.  Bound:
 // the FP64 pipe.
 template <class T, int OP, int FC, bool SING>
 __global__ void __launch_bounds__(128) k_entries_generic(MeshDev m, const double *s, double c, int nq, const int *rows,
